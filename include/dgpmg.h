@@ -484,9 +484,8 @@ int dg_plan_destroy(dg_plan* plan);
 #define DG_TUNE_FP64 0  /* the FP64 Jacobian action (outer FGMRES products, FP64 cycle) */
 #define DG_TUNE_FP32 1  /* the FP32 Jacobian action and block-Jacobi apply of the FP32 cycle */
 typedef struct dg_tuning {
-  int face_warps;        /* faces per CTA of the face pass (one warp each): 2, 4 or 8 (default 4) */
-  int vol_threads;       /* threads per CTA of the volume pass (one element per CTA): 64, 128, 160, 192
-                            or 256 (128) */
+  int face_warps;        /* warps per CTA of the face pass: 2, 4 or 8 (default 4) */
+  int vol_threads;       /* threads per CTA of the volume pass: 64, 128, 160, 192 or 256 (128) */
   int face_ctas_per_sm;  /* cap on resident CTAs per SM of the face pass, 0..32 (0: shared memory decides) */
   int vol_ctas_per_sm;   /* the same for the volume pass */
   int jacobi_stage_kb;   /* FP32 cycle: KB of element inverses per bulk-copy stage of the fine-level

@@ -246,7 +246,7 @@ static void free_all(Handle* h) {
   F(T.D2_idx); F(T.D2_val);
   TablesF& TF = h->tabf;
   F(TF.Bvol); F(TF.L1); F(TF.wvol); F(TF.B2); F(TF.W2); F(TF.pv); F(TF.pd); F(TF.Drow_val); F(TF.Dcol_val); F(TF.D2_val);
-  F(h->face_out_f); F(h->face_lift_f); F(h->ubar_f); F(h->dFlux_f);
+  F(h->face_buf_f); F(h->ubar_f); F(h->dFlux_f);
   F(h->tc_tab[0]); F(h->tc_tab[1]); F(h->ubar_scale);
   for (int d = 0; d < 3; ++d) F(h->dnode[d]);
   F(h->geo);
@@ -260,7 +260,7 @@ static void free_all(Handle* h) {
     F(h->lev[l].LUf); F(h->lev[l].Bsrf); F(h->lev[l].t0f); F(h->lev[l].t1f); F(h->lev[l].t2f);
     F(h->lev[l].LU16); F(h->lev[l].Bsr16);
   }
-  F(h->face_out); F(h->face_lift); F(h->wlin); F(h->flin); F(h->ubar); F(h->dFlux); F(h->wnorm2);
+  F(h->face_buf); F(h->wlin); F(h->flin); F(h->ubar); F(h->dFlux); F(h->wnorm2);
   F(h->fd_w); F(h->fd_f); F(h->red); F(h->red_out); F(h->status); F(h->V); F(h->Z); F(h->hcol);
   if (h->hcol_host) cudaFreeHost(h->hcol_host);
   for (int l = 0; l < DG_MAX_LEVELS; ++l) F(h->smV[l]);
@@ -407,16 +407,15 @@ static int create(const dg_params* p, const std::vector<Box>& boxes, Handle* h) 
   }
   const long long n0 = h->lev[0].n;
   const int n2f = h->tab.n2;
-  if ((rc = dalloc(h, &h->face_out, (size_t)ne * 6 * 4 * n2f)) || (rc = dalloc(h, &h->face_lift, (size_t)ne * 6 * 3 * n2f)) ||
+  if ((rc = dalloc(h, &h->face_buf, (size_t)(3 * ne + h->nbf) * 7 * n2f)) ||
       (rc = dalloc(h, &h->wlin, n0)) || (rc = dalloc(h, &h->flin, n0)) || (rc = dalloc(h, &h->fd_w, n0)) ||
       (rc = dalloc(h, &h->fd_f, n0)) || (rc = dalloc(h, &h->ubar, (size_t)ne * 3 * h->tab.nq)) ||
-      (rc = dalloc(h, &h->dFlux, (size_t)(3 * ne + h->nbf) * h->tab.nqf * 32)) || (rc = dalloc(h, &h->wnorm2, 1)) ||
+      (rc = dalloc(h, &h->dFlux, (size_t)(3 * ne + h->nbf) * h->tab.nqf * 16)) || (rc = dalloc(h, &h->wnorm2, 1)) ||
       (rc = dalloc(h, &h->red, 4096)) || (rc = dalloc(h, &h->red_out, 8)) || (rc = dalloc(h, &h->status, 3)))
     return rc;
-  if ((rc = dalloc(h, &h->face_out_f, (size_t)ne * 6 * 4 * n2f)) ||
-      (rc = dalloc(h, &h->face_lift_f, (size_t)ne * 6 * 3 * n2f)) ||
+  if ((rc = dalloc(h, &h->face_buf_f, (size_t)(3 * ne + h->nbf) * 7 * n2f)) ||
       (rc = dalloc(h, &h->ubar_f, (size_t)ne * 3 * h->tab.nq)) ||
-      (rc = dalloc(h, &h->dFlux_f, (size_t)(3 * ne + h->nbf) * h->tab.nqf * 32)))
+      (rc = dalloc(h, &h->dFlux_f, (size_t)(3 * ne + h->nbf) * h->tab.nqf * 16)))
     return rc;
   DG_CUDA(h, cudaDeviceSynchronize());
   return DG_OK;

@@ -77,6 +77,22 @@ struct AsmArgs {
   double inv_gdt;
 };
 
+// Entry (i, j) of the Riemann flux's Jacobian at a face point with normal d, columns of the - side
+// (s = 0) or the + side (s = 1), from its 16 stored values (ac_riemann in dg_riemann.h; quad k of the
+// point at p + k * stride).
+template <class R>
+__device__ __forceinline__ R flux_jacobian(const R* p, int stride, int d, int i, int j, int s) {
+  if (i == 3 || i == d) {  // du* or dF_n: normal velocity and pressure only
+    if (j != 3 && j != d) return R(0);
+    return p[(i == d ? stride : 0) + 2 * s + (j == 3)];
+  }
+  if (j == i) return p[2 * stride + 2 + s];
+  if (j != 3 && j != d) return R(0);
+  const int t = i == (d == 2 ? 0 : d + 1) ? 0 : 1;
+  const R v = p[2 * stride + t] * p[2 * s + (j == 3)];
+  return j == 3 ? v : v + p[3 * stride + 2 * t + s];
+}
+
 template <int K, class R>
 __global__ void __launch_bounds__(256) assemble_state_kernel(AsmArgs<R> a) {
   using L = AsmSmem<K, R>;
@@ -133,14 +149,14 @@ __global__ void __launch_bounds__(256) assemble_state_kernel(AsmArgs<R> a) {
         R v = R(0);
         if (!oth) {
           const int f = side == 0 ? 3 * e + d : (nb_ >= 0 ? 3 * nb_ + d : 3 * a.M.ne + a.M.bslot[e]);
-          const R* Jq = a.dFlux + ((size_t)f * NQF + q) * 32 + i * 8;
-          v = Jq[(side == 0 ? 0 : 4) + j];
+          const R* Jq = a.dFlux + ((size_t)f * 4 * NQF + q) * 4;
+          v = flux_jacobian(Jq, 4 * NQF, d, i, j, side);
           // at a wall the ghost state (-u_K, p_K) is the element's own: its columns add with
           // sign -1 (velocity) and +1 (pressure)
-          if (nb_ < 0) v += (j == 3 ? R(1) : -R(1)) * Jq[(side == 0 ? 4 : 0) + j];
+          if (nb_ < 0) v += (j == 3 ? R(1) : -R(1)) * flux_jacobian(Jq, 4 * NQF, d, i, j, 1 - side);
         } else if (nb_ >= 0 && nb1 > 0) {
           const int f = side == 0 ? 3 * e + d : 3 * nb_ + d;
-          v = a.dFlux[((size_t)f * NQF + q) * 32 + i * 8 + (side == 0 ? 4 : 0) + j];
+          v = flux_jacobian(a.dFlux + ((size_t)f * 4 * NQF + q) * 4, 4 * NQF, d, i, j, 1 - side);
         }
         dst[t] = v * sW2[q];
       }

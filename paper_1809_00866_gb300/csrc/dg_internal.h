@@ -88,7 +88,7 @@ struct Level {
 // Launch shapes of the tangent operator passes and of the staged block-Jacobi apply
 // (dg_set_tuning / dg_autotune); every shape gives the same results.
 struct OpTune {
-  int face_warps = 4;         // faces per CTA of the face pass: 2, 4 or 8
+  int face_warps = 4;         // warps per CTA of the face pass: 2, 4 or 8
   int vol_threads = 128;      // threads per CTA of the volume pass: 64, 128 or 256
   int face_per_sm = 0;        // cap on CTAs per SM (0: shared memory decides)
   int vol_per_sm = 0;
@@ -143,10 +143,8 @@ struct Handle {
   int device = 0;               // the CUDA device that was current at dg_create (holds every buffer)
 
   // scratch of the matrix-free operator
-  double* face_out = nullptr;  // [ne][6][4][n2] face-term contributions per element face slot (2D modes)
-  double* face_lift = nullptr; // [ne][6][3][n2] BR2 local lifting (scaled 2D jump) per element face slot
-  float* face_out_f = nullptr;   // FP32 scratch of the FP32 operator
-  float* face_lift_f = nullptr;
+  double* face_buf = nullptr;  // [3*ne+nbf][7][n2] normal flux (4) and velocity jump (3) per face, 2D modes
+  float* face_buf_f = nullptr; // FP32 scratch of the FP32 operator
   void* tc_tab[2] = {nullptr, nullptr};  // 16-bit basis tables of the tensor-core volume pass (FP16, BF16)
   float* ubar_scale = nullptr;            // [ne] power-of-two scale of the FP32 linearisation velocity
   float* ubar_f = nullptr;       // FP32 copies of the linearisation cache
@@ -169,7 +167,8 @@ struct Handle {
   double* wlin = nullptr;   // [n0]
   double* flin = nullptr;   // [n0] f_h(wlin)
   double* ubar = nullptr;   // [ne][3][nq] velocity at the volume points
-  double* dFlux = nullptr;  // [3*ne][nqf][4][8] Jacobian of the Riemann flux at the face points
+  double* dFlux = nullptr;  // [3*ne+nbf][4][nqf][4] Jacobian of the Riemann flux at the face points: 16
+                            // values in the face's frame (ac_riemann in dg_riemann.h), as four quads
   double* wnorm2 = nullptr; // device scalar ||wlin||^2
   // finite-difference scratch
   double* fd_w = nullptr;

@@ -570,7 +570,7 @@ static int mg_full(Handle* h, int l, const double* g, double* x, const dg_solve_
 int prepare_lin_fp32(Handle* h, cudaStream_t st) {
   if (h->lin_f_ready) return DG_OK;
   const int ne = h->ne;
-  const long long nu = (long long)ne * 3 * h->tab.nq, nf = (long long)(3 * ne + h->nbf) * h->tab.nqf * 32;
+  const long long nu = (long long)ne * 3 * h->tab.nq, nf = (long long)(3 * ne + h->nbf) * h->tab.nqf * 16;
   convert_kernel<double, float><<<grid_for(h, nu / 256 + 1), 256, 0, st>>>(nu, h->ubar, h->ubar_f);
   DG_LAUNCH_CHECK(h);
   convert_kernel<double, float><<<grid_for(h, nf / 256 + 1), 256, 0, st>>>(nf, h->dFlux, h->dFlux_f);

@@ -40,6 +40,7 @@
 
 #include "dg_async.h"
 #include "dg_internal.h"
+#include "dg_pencil.h"
 
 namespace dg {
 namespace {
@@ -154,12 +155,10 @@ struct TcVolArgs {
   const int* fa;
   const float* Drow_val;
   const float* Dcol_val;
-  const float* pv;
   const float* wvol;
   const float* in;
   float* out;
-  const float* face_out;
-  const float* face_lift;
+  const float* face_buf;
   const float* ubar;
   const float* ubar_scale;
   const uint4* tab;  // TA1 then TB2, 16-bit, in the operand layout (kTabBytes)
@@ -237,7 +236,9 @@ __global__ void __launch_bounds__(kTcThreads) tc_vol_kernel(TcVolArgs a) {
   __shared__ uint64_t bar;
   __shared__ unsigned tslot;
   __shared__ float sSig[kTcE], sTau[kTcE], sJ[kTcE][3], sShift[kTcE];
-  __shared__ float PV[2 * K1];
+  __shared__ float sAl[kTcE][3];  // A4 / (2 s) of the faces normal to each axis
+  __shared__ int sFid[kTcE][6];   // face numbers of the slots -x, +x, -y, ...
+  __shared__ float QT[3 * NB];    // s_a / (s_b s_c): the face buffer's plain Legendre modes to orthonormal ones
   __shared__ int FMAP[3 * NB], FA[3 * NB];
   float* sC = reinterpret_cast<float*>(sm + Z::SC);    // [E][4][NB]
   float* sFv = reinterpret_cast<float*>(sm + Z::FV);   // [E][6][NB]
@@ -259,8 +260,11 @@ __global__ void __launch_bounds__(kTcThreads) tc_vol_kernel(TcVolArgs a) {
     for (int i = tid; i < (int)(kTabBytes / 16); i += nt) s4[i] = a.tab[i];
     for (int i = tid; i < (int)((kA2 - kB1) / 16); i += nt) s4[kB1 / 16 + i] = make_uint4(0, 0, 0, 0);
   }
-  for (int t = tid; t < 2 * K1; t += nt) PV[t] = a.pv[t];
-  for (int t = tid; t < 3 * NB; t += nt) { FMAP[t] = a.fmap[t]; FA[t] = a.fa[t]; }
+  for (int t = tid; t < 3 * NB; t += nt) {
+    FMAP[t] = a.fmap[t];
+    FA[t] = a.fa[t];
+    QT[t] = (float)((FA[t] + 0.5) * mode_scale<K>.inv[t % NB]);
+  }
   fence_proxy_async_smem();
   tc_fence_before();
   __syncthreads();
@@ -280,9 +284,8 @@ __global__ void __launch_bounds__(kTcThreads) tc_vol_kernel(TcVolArgs a) {
       // the next tile's contiguous inputs into L2 while this tile is computed
       const int n0 = (tile + gridDim.x) * kTcE, n1 = min(ne, n0 + kTcE);
       prefetch_l2(a.in + (size_t)n0 * 4 * NB, a.in + (size_t)n1 * 4 * NB);
-      prefetch_l2(a.face_lift + (size_t)n0 * 6 * 3 * N2, a.face_lift + (size_t)n1 * 6 * 3 * N2);
+      prefetch_l2(a.face_buf + (size_t)n0 * 21 * N2, a.face_buf + (size_t)n1 * 21 * N2);
       prefetch_l2(a.ubar + (size_t)n0 * 3 * NQ, a.ubar + (size_t)n1 * 3 * NQ);
-      prefetch_l2(a.face_out + (size_t)n0 * 6 * 4 * N2, a.face_out + (size_t)n1 * 6 * 4 * N2);
     }
     // 1. input coefficients (FP32, contiguous), element geometry
     for (int t = tid; t < kTcE * 4 * NB; t += nt)
@@ -294,7 +297,17 @@ __global__ void __launch_bounds__(kTcThreads) tc_vol_kernel(TcVolArgs a) {
       sJ[t][1] = (float)G[6];
       sJ[t][2] = (float)G[7];
       sShift[t] = (float)(a.inv_gdt * G[11]);
+      for (int d = 0; d < 3; ++d) sAl[t][d] = (float)(0.125 * G[(d + 1) % 3] * G[(d + 2) % 3] * G[4]);
       sTau[t] = ok ? a.ubar_scale[e0 + t] : 1.0f;
+    }
+    for (int t = tid; t < kTcE * 6; t += nt) {
+      const int el = t / 6, sl = t - 6 * el, d = sl >> 1, e = e0 + (el < cnt ? el : 0);
+      int f = 3 * e + d;
+      if (!(sl & 1)) {
+        const int p = a.M.nbr[(size_t)e * 6 + sl];
+        f = p >= 0 ? 3 * p + d : 3 * ne + a.M.bslot[e];
+      }
+      sFid[el][sl] = f;
     }
     __syncthreads();
     // 2. per-element scale of the velocity coefficients (warp per element)
@@ -337,15 +350,16 @@ __global__ void __launch_bounds__(kTcThreads) tc_vol_kernel(TcVolArgs a) {
         dv[j] = a.Drow_val[o];
       }
       const int j2 = FMAP[b * NB + m], ex = FA[b * NB + m];
-      const float p1 = PV[K1 + ex], p0 = PV[ex], jb = sJ[el][b];
-      const float* Lf = a.face_lift + (size_t)(e0 + el) * 6 * 3 * N2;
+      const float jb = sJ[el][b], p0 = QT[b * NB + m] * sAl[el][b], p1 = (ex & 1) ? -p0 : p0;
+      const float* L0 = a.face_buf + ((size_t)sFid[el][2 * b + 1] * 7 + 4) * N2 + j2;
+      const float* L1 = a.face_buf + ((size_t)sFid[el][2 * b] * 7 + 4) * N2 + j2;
       const float* cv0 = sC + el * 4 * NB;
 #pragma unroll
       for (int av = 0; av < 3; ++av) {
         float acc = 0.0f;
 #pragma unroll
         for (int j = 0; j < DW; ++j) acc += dv[j] * cv0[av * NB + di[j]];
-        const float rl = p1 * Lf[(2 * b) * 3 * N2 + av * N2 + j2] + p0 * Lf[(2 * b + 1) * 3 * N2 + av * N2 + j2];
+        const float rl = p1 * L1[av * N2] + p0 * L0[av * N2];
         sG[(el * 9 + av * 3 + b) * NB + m] = acc * jb - rl;
       }
     }
@@ -450,14 +464,14 @@ __global__ void __launch_bounds__(kTcThreads) tc_vol_kernel(TcVolArgs a) {
 #pragma unroll
         for (int i = 0; i < 4; ++i) acc[i] += sJ[el][pp] * s2[i];
       }
-      const float* FO = a.face_out + (size_t)e * 6 * 4 * N2;
 #pragma unroll
-      for (int sl = 0; sl < 6; ++sl) {
-        const int dd = sl >> 1, side = (sl & 1) ? 0 : 1;
-        const float pw = PV[side * K1 + FA[dd * NB + m]];
-        const int fm = FMAP[dd * NB + m];
+      for (int sl = 0; sl < 6; ++sl) {  // + side: F, - side: -F times (-1)^a
+        const int dd = sl >> 1;
+        const float w2 = 2.0f * QT[dd * NB + m] * sAl[el][dd];
+        const float pw = (sl & 1) || (FA[dd * NB + m] & 1) ? w2 : -w2;
+        const float* FO = a.face_buf + (size_t)sFid[el][sl] * 7 * N2 + FMAP[dd * NB + m];
 #pragma unroll
-        for (int i = 0; i < 4; ++i) acc[i] += pw * FO[sl * 4 * N2 + i * N2 + fm];
+        for (int i = 0; i < 4; ++i) acc[i] += pw * FO[i * N2];
       }
 #pragma unroll
       for (int i = 0; i < 4; ++i) {
@@ -560,12 +574,10 @@ int tc_volume_tangent(Handle* h, const float* in, float* out, int tc, cudaStream
   a.fa = T.fa;
   a.Drow_val = F.Drow_val;
   a.Dcol_val = F.Dcol_val;
-  a.pv = F.pv;
   a.wvol = F.wvol;
   a.in = in;
   a.out = out;
-  a.face_out = h->face_out_f;
-  a.face_lift = h->face_lift_f;
+  a.face_buf = h->face_buf_f;
   a.ubar = h->ubar_f;
   a.ubar_scale = h->ubar_scale;
   a.tab = static_cast<const uint4*>(h->tc_tab[bf]);

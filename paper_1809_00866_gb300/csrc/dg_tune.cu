@@ -1,4 +1,4 @@
-// Launch-shape tuning of the hot kernels per (degree k, quadrature size N_q): the faces per CTA
+// Launch-shape tuning of the hot kernels per (degree k, quadrature size N_q): the warps per CTA
 // of the face pass, the threads per CTA of the volume pass, the CTAs per SM of both, and the
 // element blocks staged per bulk copy of the FP32 block-Jacobi apply. The paper's CPU code has no
 // counterpart; on a GPU the best shapes depend on k (the shared-memory footprint of a face or an
@@ -126,7 +126,6 @@ static int autotune(Handle* h, int which, bool use_cache, double* report, cudaSt
     auto op = [&]() -> int { return f32 ? op_tangent_f32(h, xf, yf, 0, st) : op_tangent(h, L0.t0, L0.t1, st); };
     const int cf = f32 ? DG_PROF_FACE_TAN32 : DG_PROF_FACE_TAN, cv = f32 ? DG_PROF_VOL_TAN32 : DG_PROF_VOL_TAN;
     const int face_w[3] = {2, 4, 8};
-    // 160 threads: one pass over the 4 N_b outputs of the last volume phase at P4 (140)
     const int vol_t[5] = {64, 128, 160, 192, 256};
     const int vol_cap[2] = {0, 4};
     double ms[DG_PROF_N];
