@@ -540,8 +540,9 @@ __global__ void inherit_kernel(int nblocks, int nbs, const R* src, long long src
 
 // In-place LU factorisation with partial (row) pivoting of one b x b block per CTA in
 // shared memory (row-major, padded leading dimension). Output, column-major per block:
-// the unit-lower L below the diagonal, U above it, and 1/U_kk on the diagonal; and the
-// row permutation pi (row i of P A is row pi[i] of A).
+// the unit-lower L below the diagonal, U with its rows scaled by 1/U_kk above it, and 1/U_kk on the
+// diagonal (backward substitution then needs no division or product per step); and the row
+// permutation pi (row i of P A is row pi[i] of A).
 template <class R>
 __global__ void __launch_bounds__(256) lu_factor_kernel(int nblk, int b, const R* in, R* out, int* perm,
                                                        unsigned* status) {
@@ -603,7 +604,7 @@ __global__ void __launch_bounds__(256) lu_factor_kernel(int nblk, int b, const R
     R* dst = out + (size_t)blk * b * b;
     for (int t = tid; t < b * b; t += nt) {
       const int c = t / b, r = t - c * b;
-      dst[t] = A[r * LD + c];
+      dst[t] = r < c ? A[r * LD + c] * A[r * LD + r] : A[r * LD + c];
     }
     if (tid == 0) {
       // compose the swaps into pi: apply them in order to the identity

@@ -66,7 +66,7 @@ struct Level {
   int k = 0, nb = 0, b = 0;  // degree, modes per variable, block size 4*nb
   long long n = 0;           // vector length ne*4*nb
   double* Dblk = nullptr;    // [ne][b][b] diagonal blocks, column-major per block
-  double* Dinv = nullptr;    // [ne][b][b] LU factors (unit L, U, 1/U_kk on the diagonal), column-major per block
+  double* Dinv = nullptr;    // [ne][b][b] LU factors (unit L, U with rows over U_kk, 1/U_kk on the diagonal), column-major per block
   int* perm = nullptr;       // [ne][b] row permutation of the LU factors
   double* Bsr = nullptr;     // [ne][7][b][b] level >= 1: slot 0 diagonal, slots 1..6 faces -x,+x,-y,+y,-z,+z
   double* Dlin = nullptr;    // level 0: [ne][b][b] diagonal blocks of the state-independent linear part

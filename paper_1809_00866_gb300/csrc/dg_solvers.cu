@@ -187,46 +187,107 @@ __global__ void __launch_bounds__(128) bsr_t_kernel(int ne, int b, const int* nb
 }
 
 // x[e] = x[e] + omega * D[e]^-1 (g[e] - Gx[e]) with the LU factors of D[e]
-// (Gx == nullptr: Gx = 0; x_zero: the old x is 0). One warp per element: the
-// residual is gathered in row order pi into shared memory, then forward substitution
-// with the unit-lower L and backward substitution with U (1/U_kk stored on the
-// diagonal), both along contiguous columns.
+// (Gx == nullptr: Gx = 0; x_zero: the old x is 0). One warp per element, the vector in its
+// registers: forward substitution with the unit-lower L, then backward substitution with U whose rows
+// are scaled by 1/U_kk (lu_factor_kernel), both along contiguous columns: a step broadcasts one
+// entry by shuffle and takes it times the column off the others.
+//
+// Bound: the FP64 pipe, B^2 FMA per element (0.25 FLOP per byte of factors). The forward pass deals
+// the rows to the lanes from the last one back and the backward pass from the first one on, so the
+// rows still to be updated fill the fewest slots of 32 (385 warp FMAs per pass at B = 140, of
+// 304 in full lanes). Columns are loaded kLuAhead at a time, one group ahead of their use: the
+// first version (vector in shared memory, no load ahead) waited on memory at every one of its 2B
+// dependent steps and took 0.495 ms at 16^3 P4 (642 MB of factors).
 constexpr int kApplyWarps = 4;
-template <class R>
-__global__ void __launch_bounds__(32 * kApplyWarps) bj_update_kernel(int ne, int b, const R* LU, const int* perm,
-                                                                    const R* g, const R* Gx, R omega, int x_zero,
-                                                                    R* x) {
-  extern __shared__ __align__(16) unsigned char sraw_[];
-  R* sz = reinterpret_cast<R*>(sraw_);  // [warps][b]
+constexpr int kLuAhead = 4;
+
+// kLuAhead columns j0, j0 + step, ... of slots 0..M of this lane's rows (row(s) in [0, B), or not loaded)
+template <int M, class Row>
+__device__ __forceinline__ void lu_load(double (&A)[kLuAhead][M + 1], const double* L, int B, int j0, int step, int j1,
+                                        Row row) {
+#pragma unroll
+  for (int u = 0; u < kLuAhead; ++u) {
+    const int j = j0 + u * step;
+    const bool on = step > 0 ? j < j1 : j > j1;
+#pragma unroll
+    for (int s = 0; s <= M; ++s) {
+      const int r = row(s, j);
+      A[u][s] = on && r >= 0 ? __ldg(L + (size_t)j * B + r) : 0.0;
+    }
+  }
+}
+
+// Substitution over the columns whose own row sits in slot M (then M - 1, ...): FWD from column
+// B - 1 - (32 M + 31) on with rows dealt from the end, else from column 32 M + 31 down.
+template <int B, int M, bool FWD, int SL>
+__device__ __forceinline__ void lu_substitute(double (&z)[SL], const double* L, int lane) {
+  // columns in the order of elimination: index q = 32 M + 31 .. 32 M, where q is the row's place
+  // in the lane order (row = B - 1 - q forward, q backward)
+  constexpr int q1 = 32 * M + 31 < B - 1 ? 32 * M + 31 : B - 1, q0 = 32 * M;
+  const int jf = FWD ? B - 1 - q1 : q1, step = FWD ? 1 : -1, je = FWD ? B - q0 : q0 - 1;
+  // the lane's row in slot s if column j updates it (place below the column's), else -1
+  auto row = [&](int s, int j) {
+    const int q = lane + 32 * s, qj = FWD ? B - 1 - j : j;
+    return q < qj ? (FWD ? B - 1 - q : q) : -1;
+  };
+  double A[kLuAhead][M + 1], N[kLuAhead][M + 1];
+  lu_load<M>(A, L, B, jf, step, je, row);
+  for (int j = jf; FWD ? j < je : j > je; j += kLuAhead * step) {
+    lu_load<M>(N, L, B, j + kLuAhead * step, step, je, row);
+#pragma unroll
+    for (int u = 0; u < kLuAhead; ++u) {
+      const int ju = j + u * step, q = (FWD ? B - 1 - ju : ju) - 32 * M;
+      if (q < 0) break;  // past this slot's last column
+      const double zj = __shfl_sync(0xffffffffu, z[M], q);
+#pragma unroll
+      for (int s = 0; s < M; ++s) z[s] = fma(-A[u][s], zj, z[s]);
+      if (lane < q) z[M] = fma(-A[u][M], zj, z[M]);
+    }
+#pragma unroll
+    for (int u = 0; u < kLuAhead; ++u)
+#pragma unroll
+      for (int s = 0; s <= M; ++s) A[u][s] = N[u][s];
+  }
+  if constexpr (M > 0) lu_substitute<B, M - 1, FWD>(z, L, lane);
+}
+
+template <int B>
+__global__ void __launch_bounds__(32 * kApplyWarps) bj_update_kernel(int ne, const double* __restrict__ LU,
+                                                                    const int* __restrict__ perm, const double* g,
+                                                                    const double* Gx, double omega, int x_zero,
+                                                                    double* x) {
+  constexpr int SL = (B + 31) / 32;
+  __shared__ double sz[kApplyWarps][B];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  R* z = sz + warp * b;
-  for (int e = blockIdx.x * kApplyWarps + warp; e < ne; e += gridDim.x * kApplyWarps) {
-    const int* pi = perm + (size_t)e * b;
-    const R* ge = g + (size_t)e * b;
-    const R* gx = Gx ? Gx + (size_t)e * b : nullptr;
-    for (int i = lane; i < b; i += 32) {
+  const int e = blockIdx.x * kApplyWarps + warp;
+  if (e >= ne) return;
+  const int* pi = perm + (size_t)e * B;
+  const double* ge = g + (size_t)e * B;
+  const double* L = LU + (size_t)e * B * B;
+  double z[SL], dg[SL];
+#pragma unroll
+  for (int s = 0; s < SL; ++s) {
+    const int i = B - 1 - (lane + 32 * s), k = lane + 32 * s;
+    z[s] = 0.0;
+    if (i >= 0) {
       const int r = pi[i];
-      z[i] = ge[r] - (gx ? gx[r] : R(0));
+      z[s] = ge[r] - (Gx ? Gx[(size_t)e * B + r] : 0.0);
     }
-    __syncwarp();
-    const R* M = LU + (size_t)e * b * b;
-    for (int j = 0; j < b; ++j) {  // z <- L^-1 z
-      const R zj = z[j];
-      const R* col = M + (size_t)j * b;
-      for (int i = j + 1 + lane; i < b; i += 32) z[i] = fma(-col[i], zj, z[i]);
-      __syncwarp();
-    }
-    for (int j = b - 1; j >= 0; --j) {  // z <- U^-1 z
-      const R* col = M + (size_t)j * b;
-      const R zj = z[j] * col[j];
-      __syncwarp();
-      if (lane == 0) z[j] = zj;
-      for (int i = lane; i < j; i += 32) z[i] = fma(-col[i], zj, z[i]);
-      __syncwarp();
-    }
-    R* xe = x + (size_t)e * b;
-    for (int i = lane; i < b; i += 32) xe[i] = (x_zero ? R(0) : xe[i]) + omega * z[i];
-    __syncwarp();
+    dg[s] = k < B ? __ldg(L + (size_t)k * (B + 1)) : 0.0;
+  }
+  lu_substitute<B, SL - 1, true>(z, L, lane);
+#pragma unroll
+  for (int s = 0; s < SL; ++s)
+    if (lane + 32 * s < B) sz[warp][B - 1 - (lane + 32 * s)] = z[s];
+  __syncwarp();
+#pragma unroll
+  for (int s = 0; s < SL; ++s) z[s] = lane + 32 * s < B ? sz[warp][lane + 32 * s] * dg[s] : 0.0;
+  lu_substitute<B, SL - 1, false>(z, L, lane);
+  double* xe = x + (size_t)e * B;
+#pragma unroll
+  for (int s = 0; s < SL; ++s) {
+    const int i = lane + 32 * s;
+    if (i < B) xe[i] = (x_zero ? 0.0 : xe[i]) + omega * z[s];
   }
 }
 
@@ -236,11 +297,19 @@ static int grid_for(const Handle* h, long long work) {
   return g < 1 ? 1 : (int)g;
 }
 
-static int apply_grid(const Handle* h) {
-  long long g = (h->ne + kApplyWarps - 1) / kApplyWarps;
-  const long long cap = (long long)h->nsm * 16;
-  if (g > cap) g = cap;
-  return (int)(g < 1 ? 1 : g);
+// x <- (x_zero ? 0 : x) + omega D^-1 (g - Gx) on level L (block sizes 4 N_b(k), k = 1..4)
+static int apply_block_inverse(Handle* h, const Level& L, const double* g, const double* Gx, double omega, int x_zero,
+                               double* x, cudaStream_t st) {
+  const int grid = (h->ne + kApplyWarps - 1) / kApplyWarps, nt = 32 * kApplyWarps;
+  switch (L.b) {
+    case 16: bj_update_kernel<16><<<grid, nt, 0, st>>>(h->ne, L.Dinv, L.perm, g, Gx, omega, x_zero, x); break;
+    case 40: bj_update_kernel<40><<<grid, nt, 0, st>>>(h->ne, L.Dinv, L.perm, g, Gx, omega, x_zero, x); break;
+    case 80: bj_update_kernel<80><<<grid, nt, 0, st>>>(h->ne, L.Dinv, L.perm, g, Gx, omega, x_zero, x); break;
+    case 140: bj_update_kernel<140><<<grid, nt, 0, st>>>(h->ne, L.Dinv, L.perm, g, Gx, omega, x_zero, x); break;
+    default: return fail(h, DG_ERR_ARG, "unsupported block size");
+  }
+  DG_LAUNCH_CHECK(h);
+  return DG_OK;
 }
 
 static int run_bsr(Handle* h, int lvl, double alpha, const double* x, double beta, double* y, cudaStream_t st) {
@@ -261,7 +330,6 @@ int level_matvec(Handle* h, int lvl, const double* x, double* y, cudaStream_t st
 static int jacobi_sweeps(Handle* h, int lvl, const double* g, double* x, int sweeps, double omega, bool x_zero,
                          cudaStream_t st) {
   Level& L = h->lev[lvl];
-  const size_t smem = sizeof(double) * L.b * kApplyWarps;
   for (int s = 0; s < sweeps; ++s) {
     const bool zero = x_zero && s == 0;
     if (!zero) {
@@ -271,9 +339,7 @@ static int jacobi_sweeps(Handle* h, int lvl, const double* g, double* x, int swe
     cudaEvent_t e0 = nullptr;
     int rc;
     if (lvl == 0 && (rc = prof_begin(h, st, &e0))) return rc;
-    bj_update_kernel<double><<<apply_grid(h), 32 * kApplyWarps, smem, st>>>(h->ne, L.b, L.Dinv, L.perm, g,
-                                                                    zero ? nullptr : L.t2, omega, zero ? 1 : 0, x);
-    DG_LAUNCH_CHECK(h);
+    if ((rc = apply_block_inverse(h, L, g, zero ? nullptr : L.t2, omega, zero ? 1 : 0, x, st))) return rc;
     if (lvl == 0) {  // algorithmic bytes: LU factors and permutation, g, Gx, old x read; x written
       const double vec = (double)h->ne * L.b * sizeof(double);
       const double bytes = (double)h->ne * L.b * ((double)L.b * sizeof(double) + sizeof(int)) +
@@ -376,14 +442,11 @@ static int gmres_smooth(Handle* h, int lvl, const double* g, double* x, int its,
   double* hn2 = h->smSmall + kSmHn2;
   double* beta2 = h->smSmall + kSmBeta2;
   double* ny = h->smSmall + kSmNy;
-  const size_t smem = sizeof(double) * L.b * kApplyWarps;
   const int ld = its + 1;
   int rc;
   // v0 = D^-1 (g - G x)
   if (!x_zero && (rc = level_matvec(h, lvl, x, L.t2, st))) return rc;
-  bj_update_kernel<double><<<apply_grid(h), 32 * kApplyWarps, smem, st>>>(h->ne, L.b, L.Dinv, L.perm, g,
-                                                                  x_zero ? nullptr : L.t2, 1.0, 1, V);
-  DG_LAUNCH_CHECK(h);
+  if ((rc = apply_block_inverse(h, L, g, x_zero ? nullptr : L.t2, 1.0, 1, V, st))) return rc;
   if ((rc = vec_norm2(h, V, n, beta2, st))) return rc;
   normalize_kernel<<<grid_for(h, n / 256 + 1), 256, 0, st>>>(n, V, beta2);
   DG_LAUNCH_CHECK(h);
@@ -391,9 +454,7 @@ static int gmres_smooth(Handle* h, int lvl, const double* g, double* x, int its,
     double* vj = V + (size_t)j * n;
     double* w = V + (size_t)(j + 1) * n;
     if ((rc = level_matvec(h, lvl, vj, L.t2, st))) return rc;
-    bj_update_kernel<double><<<apply_grid(h), 32 * kApplyWarps, smem, st>>>(h->ne, L.b, L.Dinv, L.perm, L.t2, nullptr, 1.0,
-                                                                    1, w);
-    DG_LAUNCH_CHECK(h);
+    if ((rc = apply_block_inverse(h, L, L.t2, nullptr, 1.0, 1, w, st))) return rc;
     for (int pass = 0; pass < 2; ++pass) {
       if ((rc = multidot(h, n, j + 1, V, w, tmp, st))) return rc;
       multi_axpy_kernel<<<grid_for(h, n / 256 + 1), 256, 0, st>>>(n, j + 1, V, n, tmp, w);
