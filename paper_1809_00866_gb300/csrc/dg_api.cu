@@ -289,8 +289,10 @@ struct Box {
   const double* node[3];
 };
 
-// Reduction chunks of about kChunkDoubles level-0 entries, never across two problems.
-constexpr int kChunkDoubles = 2048;
+// Reduction chunks: about kChunks per problem (four CTAs per SM on one large problem, few enough
+// that one CTA adds their partials in a few microseconds), of kChunkDoubles level-0 entries at
+// least, never across two problems. A problem's chunks depend on its own size alone.
+constexpr int kChunkDoubles = 1024, kChunks = 608;
 
 static int create(const dg_params* p, const std::vector<Box>& boxes, Handle* h) {
   if (!p) return fail(h, DG_ERR_ARG, "null params");
@@ -376,11 +378,11 @@ static int create(const dg_params* p, const std::vector<Box>& boxes, Handle* h) 
   if ((rc = upload(h, &h->dshift, std::vector<double>(h->nprob, 1.0)))) return rc;
   {
     const int b0 = 4 * nb_of(p->k[0]);
-    const int ce = std::max(1, kChunkDoubles / b0);
     std::vector<int2> ch;
     std::vector<int> cp, pc0(h->nprob + 1, 0);
     for (int q = 0; q < h->nprob; ++q) {
       pc0[q] = (int)ch.size();
+      const int ce = std::max(std::max(1, kChunkDoubles / b0), (h->pe0[q + 1] - h->pe0[q] + kChunks - 1) / kChunks);
       for (int e = h->pe0[q]; e < h->pe0[q + 1]; e += ce) {
         ch.push_back(make_int2(e, std::min(e + ce, h->pe0[q + 1])));
         cp.push_back(q);

@@ -20,6 +20,7 @@
 #include <vector>
 
 #include "dg_internal.h"
+#include "dg_reduce.h"
 
 namespace dg {
 
@@ -59,33 +60,12 @@ __global__ void __launch_bounds__(kSegThreads) seg_dot_kernel(int nchunk, const 
                                                               const double* w, double* part, int ld) {
   __shared__ double red[kSegThreads / 32][8];
   const int nv = nv_fixed > 0 ? nv_fixed : jdev[0] + 1;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   for (int c = blockIdx.x; c < nchunk; c += gridDim.x) {
     const long long i0 = (long long)chunk[c].x * per_e, i1 = (long long)chunk[c].y * per_e;
     for (int v0 = 0; v0 < nv; v0 += 8) {
       const int cnt = min(8, nv - v0);
-      double acc[8];
-#pragma unroll
-      for (int v = 0; v < 8; ++v) acc[v] = 0.0;
-      for (long long i = i0 + threadIdx.x; i < i1; i += kSegThreads) {
-        const double wi = w[i];
-#pragma unroll
-        for (int v = 0; v < 8; ++v)
-          if (v < cnt) acc[v] += V[(size_t)(v0 + v) * ldv + i] * wi;
-      }
-#pragma unroll
-      for (int v = 0; v < 8; ++v) {
-        double a = acc[v];
-        for (int o = 16; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
-        if (lane == 0) red[warp][v] = a;
-      }
-      __syncthreads();
-      if (threadIdx.x < cnt) {
-        double t = 0.0;
-        for (int q = 0; q < kSegThreads / 32; ++q) t += red[q][threadIdx.x];
-        part[(size_t)c * ld + v0 + threadIdx.x] = t;
-      }
-      __syncthreads();
+      const double s = block_dots<kSegThreads>(V + (size_t)v0 * ldv, ldv, cnt, w, i0, i1, kSegThreads, red);
+      if (threadIdx.x < cnt) part[(size_t)c * ld + v0 + threadIdx.x] = s;
     }
   }
 }
@@ -102,7 +82,7 @@ __global__ void __launch_bounds__(kSegThreads) seg_reduce_kernel(const int* pchu
   for (int v = warp; v < nv; v += kSegThreads / 32) {
     double a = 0.0;
     for (int c = c0 + lane; c < c1; c += 32) a += part[(size_t)c * ld + v];
-    for (int o = 16; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
+    a = warp_sum(a);
     if (lane == 0) {
       pass[(size_t)p * pld + v] = a;
       if (sum) sum[(size_t)p * pld + v] = accumulate ? sum[(size_t)p * pld + v] + a : a;

@@ -7,73 +7,42 @@
 #include <vector>
 
 #include "dg_internal.h"
+#include "dg_reduce.h"
 
 namespace dg {
 
-constexpr int kRedBlocks = 512;  // fixed partial count: reductions are bitwise reproducible
+constexpr int kRedBlocks = 512;  // partials per vector at most; their number depends on n alone, so the
+                                 // reductions are bitwise reproducible
+static int red_blocks(long long n) { return (int)std::min<long long>(kRedBlocks, (n + 2047) / 2048); }
 
 // ------------------------------------------------------------ reductions
-__global__ void __launch_bounds__(256) norm2_partial_kernel(long long n, const double* x, double* part) {
-  __shared__ double s[256];
-  double acc = 0.0;
-  for (long long i = blockIdx.x * 256LL + threadIdx.x; i < n; i += (long long)gridDim.x * 256) acc += x[i] * x[i];
-  s[threadIdx.x] = acc;
-  __syncthreads();
-  for (int o = 128; o > 0; o >>= 1) {
-    if (threadIdx.x < o) s[threadIdx.x] += s[threadIdx.x + o];
-    __syncthreads();
-  }
-  if (threadIdx.x == 0) part[blockIdx.x] = s[0];
+// part[b][j] = sum over this block's entries of V[j][i] * w[i], j < nv (nv <= 8 per launch)
+__global__ void __launch_bounds__(256) multidot_partial_kernel(long long n, int nv, const double* V, long long ldv,
+                                                               const double* w, double* part, int stride) {
+  __shared__ double red[8][8];
+  const double s = block_dots<256>(V, ldv, nv, w, blockIdx.x * 256LL, n, gridDim.x * 256LL, red);
+  if (threadIdx.x < nv) part[(size_t)blockIdx.x * stride + threadIdx.x] = s;
 }
 
-// out[j] = sum_b part[b * stride + j] for j < nvec, in a fixed order.
+// out[j] = sum_b part[b * stride + j] for j < nvec, in a fixed order: a warp per vector.
 __global__ void __launch_bounds__(256) reduce_partials_kernel(int nblk, int nvec, int stride, const double* part,
                                                               double* out) {
-  __shared__ double s[256];
-  for (int j = 0; j < nvec; ++j) {
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  for (int j = warp; j < nvec; j += 8) {
     double acc = 0.0;
-    for (int b = threadIdx.x; b < nblk; b += 256) acc += part[(size_t)b * stride + j];
-    s[threadIdx.x] = acc;
-    __syncthreads();
-    for (int o = 128; o > 0; o >>= 1) {
-      if (threadIdx.x < o) s[threadIdx.x] += s[threadIdx.x + o];
-      __syncthreads();
-    }
-    if (threadIdx.x == 0) out[j] = s[0];
-    __syncthreads();
+    for (int b = lane; b < nblk; b += 32) acc += part[(size_t)b * stride + j];
+    acc = warp_sum(acc);
+    if (lane == 0) out[j] = acc;
   }
 }
 
 int vec_norm2(Handle* h, const double* x, long long n, double* dev_out, cudaStream_t st) {
-  norm2_partial_kernel<<<kRedBlocks, 256, 0, st>>>(n, x, h->red);
+  const int nb = red_blocks(n);
+  multidot_partial_kernel<<<nb, 256, 0, st>>>(n, 1, x, n, x, h->red, 1);
   DG_LAUNCH_CHECK(h);
-  reduce_partials_kernel<<<1, 256, 0, st>>>(kRedBlocks, 1, 1, h->red, dev_out);
+  reduce_partials_kernel<<<1, 256, 0, st>>>(nb, 1, 1, h->red, dev_out);
   DG_LAUNCH_CHECK(h);
   return DG_OK;
-}
-
-// part[b][j] = sum over this block's slice of V[j][i] * w[i], j < nv (nv <= 8 per launch)
-__global__ void __launch_bounds__(256) multidot_partial_kernel(long long n, int nv, const double* V, long long ldv,
-                                                               const double* w, double* part, int stride) {
-  __shared__ double s[8][256];
-  double acc[8];
-#pragma unroll
-  for (int j = 0; j < 8; ++j) acc[j] = 0.0;
-  for (long long i = blockIdx.x * 256LL + threadIdx.x; i < n; i += (long long)gridDim.x * 256) {
-    const double wi = w[i];
-#pragma unroll
-    for (int j = 0; j < 8; ++j)
-      if (j < nv) acc[j] += V[j * ldv + i] * wi;
-  }
-#pragma unroll
-  for (int j = 0; j < 8; ++j) s[j][threadIdx.x] = acc[j];
-  __syncthreads();
-  for (int o = 128; o > 0; o >>= 1) {
-    if (threadIdx.x < o)
-      for (int j = 0; j < nv; ++j) s[j][threadIdx.x] += s[j][threadIdx.x + o];
-    __syncthreads();
-  }
-  if (threadIdx.x < nv) part[(size_t)blockIdx.x * stride + threadIdx.x] = s[threadIdx.x][0];
 }
 
 // w -= sum_j hcoef[j] * V[j], j < nv; also w is scaled by nothing
@@ -838,9 +807,9 @@ static int outer_matvec(Handle* h, const dg_solve_opts& o, const double* x, doub
 static int multidot(Handle* h, long long n, int nv, const double* V, const double* w, double* hout, cudaStream_t st) {
   for (int j0 = 0; j0 < nv; j0 += 8) {
     const int c = nv - j0 < 8 ? nv - j0 : 8;
-    multidot_partial_kernel<<<kRedBlocks, 256, 0, st>>>(n, c, V + (size_t)j0 * n, n, w, h->red, 8);
+    multidot_partial_kernel<<<red_blocks(n), 256, 0, st>>>(n, c, V + (size_t)j0 * n, n, w, h->red, 8);
     DG_LAUNCH_CHECK(h);
-    reduce_partials_kernel<<<1, 256, 0, st>>>(kRedBlocks, c, 8, h->red, hout + j0);
+    reduce_partials_kernel<<<1, 256, 0, st>>>(red_blocks(n), c, 8, h->red, hout + j0);
     DG_LAUNCH_CHECK(h);
   }
   return DG_OK;
