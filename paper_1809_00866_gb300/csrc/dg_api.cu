@@ -409,13 +409,13 @@ static int create(const dg_params* p, const std::vector<Box>& boxes, Handle* h) 
   }
   const long long n0 = h->lev[0].n;
   const int n2f = h->tab.n2;
-  if ((rc = dalloc(h, &h->face_buf, (size_t)(3 * ne + h->nbf) * 7 * n2f)) ||
+  if ((rc = dalloc(h, &h->face_buf, face_buf_size((int)ne, h->nbf, n2f))) ||
       (rc = dalloc(h, &h->wlin, n0)) || (rc = dalloc(h, &h->flin, n0)) || (rc = dalloc(h, &h->fd_w, n0)) ||
       (rc = dalloc(h, &h->fd_f, n0)) || (rc = dalloc(h, &h->ubar, (size_t)ne * 3 * h->tab.nq)) ||
       (rc = dalloc(h, &h->dFlux, (size_t)(3 * ne + h->nbf) * h->tab.nqf * 16)) || (rc = dalloc(h, &h->wnorm2, 1)) ||
       (rc = dalloc(h, &h->red, 4096)) || (rc = dalloc(h, &h->red_out, 8)) || (rc = dalloc(h, &h->status, 3)))
     return rc;
-  if ((rc = dalloc(h, &h->face_buf_f, (size_t)(3 * ne + h->nbf) * 7 * n2f)) ||
+  if ((rc = dalloc(h, &h->face_buf_f, face_buf_size((int)ne, h->nbf, n2f))) ||
       (rc = dalloc(h, &h->ubar_f, (size_t)ne * 3 * h->tab.nq)) ||
       (rc = dalloc(h, &h->dFlux_f, (size_t)(3 * ne + h->nbf) * h->tab.nqf * 16)))
     return rc;

@@ -33,6 +33,23 @@ __device__ __forceinline__ void prefetch_l2(const void* lo, const void* hi) {
   const unsigned long long b = reinterpret_cast<unsigned long long>(hi) & ~15ull;
   if (b > a) asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(a), "r"((unsigned)(b - a)) : "memory");
 }
+// One 4- or 8-byte value global -> shared memory without a register; on = false writes zero. The
+// copies of a thread are complete after its async_wait_all().
+__device__ __forceinline__ void async_value(float* dst, const float* src, bool on) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(smem_u32(dst)), "l"(src), "r"(on ? 4 : 0)
+               : "memory");
+}
+__device__ __forceinline__ void async_value(double* dst, const double* src, bool on) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;" ::"r"(smem_u32(dst)), "l"(src), "r"(on ? 8 : 0)
+               : "memory");
+}
+// the same for 8 bytes of either type (both addresses 8-byte aligned)
+template <class R>
+__device__ __forceinline__ void async_value8(R* dst, const R* src, bool on) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;" ::"r"(smem_u32(dst)), "l"(src), "r"(on ? 8 : 0)
+               : "memory");
+}
+__device__ __forceinline__ void async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 // Order this thread's earlier generic-proxy accesses of shared memory (ordinary loads and
 // stores) before later async-proxy accesses of it (a bulk copy that overwrites the same bytes).
 // Every thread that wrote a buffer executes it before the barrier after which one thread

@@ -143,7 +143,7 @@ struct Handle {
   int device = 0;               // the CUDA device that was current at dg_create (holds every buffer)
 
   // scratch of the matrix-free operator
-  double* face_buf = nullptr;  // [3*ne+nbf][7][n2] normal flux (4) and velocity jump (3) per face, 2D modes
+  double* face_buf = nullptr;  // normal flux (4) and velocity jump (3) per face, 2D modes (face_record)
   float* face_buf_f = nullptr; // FP32 scratch of the FP32 operator
   void* tc_tab[2] = {nullptr, nullptr};  // 16-bit basis tables of the tensor-core volume pass (FP16, BF16)
   float* ubar_scale = nullptr;            // [ne] power-of-two scale of the FP32 linearisation velocity
@@ -253,6 +253,24 @@ struct MeshDev {
 };
 inline MeshDev mesh_dev(const Handle* h) {
   return MeshDev{h->n[0], h->n[1], h->n[2], h->ne, h->geo, h->geof, h->nbr, h->nbf, h->bface, h->bslot};
+}
+
+// What the face pass hands to the volume pass, 7 n2 values per face: the + faces of eight consecutive
+// elements along one axis form a group (then the walls below the lowest row), [group][7][n2][8 faces],
+// so that the eight elements of a volume group read, and the eight faces of a face group write, whole
+// sectors (a record per face had 32 lanes read 32 cache lines in the volume pass).
+constexpr int kFaceGroup = 8;
+__host__ __device__ inline int face_slot(int e, int d) { return (3 * (e / kFaceGroup) + d) * kFaceGroup + e % kFaceGroup; }
+__host__ __device__ inline int wall_slot(int ne, int b) {
+  return 3 * ((ne + kFaceGroup - 1) / kFaceGroup) * kFaceGroup + b;
+}
+// index of component c's first 2D mode of the face in a slot; the modes follow kFaceGroup apart
+template <int N2>
+__host__ __device__ inline size_t face_record(int slot, int c) {
+  return ((size_t)(slot / kFaceGroup) * 7 + c) * N2 * kFaceGroup + slot % kFaceGroup;
+}
+inline size_t face_buf_size(int ne, int nbf, int n2) {
+  return (size_t)(3 * ((ne + kFaceGroup - 1) / kFaceGroup) + (nbf + kFaceGroup - 1) / kFaceGroup) * kFaceGroup * 7 * n2;
 }
 
 struct ElemGeom {

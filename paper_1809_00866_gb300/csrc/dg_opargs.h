@@ -15,10 +15,11 @@ struct OpArgsT {
   MeshDev M;
   const R* in;
   R* out;
-  R* face_buf;  // [faces][7][n2] what the face pass hands to the volume pass (see dg_face.cu)
+  R* face_buf;  // what the face pass hands to the volume pass (face_record)
   R* ubar;      // [ne][3][nq] velocity of the linearisation at the volume points
   R* dFlux;     // [faces][4][nqf][4] Jacobian of the Riemann flux at the face points (see dg_face.cu)
-  double nu, c, eta, inv_gdt;
+  R nu, eta8;  // viscosity; penalty / 8
+  double c, inv_gdt;
   unsigned* status;
   int riemann_its;  // iteration cap of the star-state solve
 };

@@ -117,9 +117,9 @@ static OpArgsT<R> make_args(Handle* h, const R* in, R* out) {
     a.ubar = h->ubar_f;
     a.dFlux = h->dFlux_f;
   }
-  a.nu = h->p.nu;
+  a.nu = R(h->p.nu);
+  a.eta8 = R(0.125 * h->p.eta);
   a.c = h->p.ac_c;
-  a.eta = h->p.eta;
   a.inv_gdt = h->inv_gdt;
   a.status = h->status;
   a.riemann_its = h->dbg.riemann_its;
@@ -301,6 +301,6 @@ extern "C" int dg_residual_noalloc(dg_handle* hh, const double* w, double* f, vo
   int rc = noalloc_scratch(h, &scratch);
   if (rc) return rc;
   OpArgs a = make_args(h, w, f);
-  a.face_buf = scratch;  // (3 N_e + wall faces) * 7 * N_2 doubles, well below N_e * 42 * N_2
+  a.face_buf = scratch;  // face_buf_size: about half of N_e * 42 * N_2
   return run_operator(h, a, MODE_RES, as_stream(stream));
 }

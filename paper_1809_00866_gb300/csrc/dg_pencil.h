@@ -74,25 +74,56 @@ constexpr PencilTab<R, K> make_pencil_tab() {
 template <class R, int K>
 __constant__ PencilTab<R, K> pencil_tab = make_pencil_tab<R, K>();
 
-// scale s_m of every 3D mode of degree K and its inverse, in mode order
-template <int K>
-struct ModeScale {
-  double s[nb_of(K)], inv[nb_of(K)];
-};
-template <int K>
-constexpr ModeScale<K> make_mode_scale() {
-  ModeScale<K> t{};
-  int m = 0;
-  for (int g = 0; g <= K; ++g)
+// compile-time loop: f(integral_constant 0), ..., f(integral_constant N - 1)
+template <class F, int... I>
+__device__ __forceinline__ void static_for_(F& f, std::integer_sequence<int, I...>) {
+  (f(std::integral_constant<int, I>{}), ...);
+}
+template <int N, class F>
+__device__ __forceinline__ void static_for(F f) {
+  static_for_(f, std::make_integer_sequence<int, N>{});
+}
+
+// Modes are ordered by degree, then by the x exponent descending, then by the y exponent descending;
+// the 2D modes (b, c) of a face by degree, then by b descending.
+__host__ __device__ constexpr int mode_exp(int m, int axis) {
+  for (int g = 0;; ++g)
     for (int a = g; a >= 0; --a)
-      for (int b = g - a; b >= 0; --b, ++m) {
-        t.s[m] = leg_scale(a) * leg_scale(b) * leg_scale(g - a - b);
-        t.inv[m] = 1.0 / t.s[m];
-      }
+      for (int b = g - a; b >= 0; --b, --m)
+        if (m == 0) return axis == 0 ? a : (axis == 1 ? b : g - a - b);
+}
+__host__ __device__ constexpr int mode_at(int a, int b, int c) {  // exponents along x, y, z
+  return tet(a + b + c) + tri(b + c) + c;
+}
+// mode with exponent a along axis d, b along (d+1)%3 and c along (d+2)%3
+__host__ __device__ constexpr int mode_along(int d, int a, int b, int c) {
+  return d == 0 ? mode_at(a, b, c) : (d == 1 ? mode_at(c, a, b) : mode_at(b, c, a));
+}
+// degree of 2D mode j
+__host__ __device__ constexpr int face_degree(int j) {
+  int g = 0;
+  while (tri(g + 1) <= j) ++g;
+  return g;
+}
+
+// scale s_m of every 3D mode of degree K and its inverse, in mode order, in the kernel's precision
+// (a conversion from FP64 at run time would go through GB300's FP64 pipe)
+template <class R, int K>
+struct ModeScale {
+  R s[nb_of(K)], inv[nb_of(K)];
+};
+template <class R, int K>
+constexpr ModeScale<R, K> make_mode_scale() {
+  ModeScale<R, K> t{};
+  for (int m = 0; m < nb_of(K); ++m) {
+    const double s = leg_scale(mode_exp(m, 0)) * leg_scale(mode_exp(m, 1)) * leg_scale(mode_exp(m, 2));
+    t.s[m] = R(s);
+    t.inv[m] = R(1.0 / s);
+  }
   return t;
 }
-template <int K>
-__constant__ ModeScale<K> mode_scale = make_mode_scale<K>();
+template <class R, int K>
+__constant__ ModeScale<R, K> mode_scale = make_mode_scale<R, K>();
 
 // c[0..N) -> values at the K + 1 Gauss nodes (ascending)
 template <int K, int N, class R>
@@ -149,23 +180,50 @@ __device__ __forceinline__ void project_pencil(const R (&v)[K + 1], R (&o)[N]) {
   }
 }
 
-// Index of the 3D mode with exponent A along axis d, b along (d+1)%3 and c along (d+2)%3,
-// g = b + c. Modes are ordered by degree t, then by the x exponent descending, then by the y
-// exponent descending: tet(t) + tri(t - ex) + ez.
-template <int A>
-__device__ __forceinline__ int pencil_mode(int d, int g, int b, int c) {
-  const int r = d == 0 ? g : A + (d == 1 ? b : c);
-  const int ez = d == 0 ? c : (d == 1 ? b : A);
-  return tet(A + g) + tri(r) + ez;
+// 2D transforms in registers: the triangle c[(b, x)], b + x <= n - 1, of 2D coefficients (ordered as the
+// face modes) at the (K+1)^2 points, handed to put(q1, q2, value); and point values v[q1][q2] to the
+// triangle o.
+template <int K, int N, class R, class Put>
+__device__ __forceinline__ void interp_triangle(const R (&c)[N * (N + 1) / 2], Put put) {
+  R u[N][K + 1];  // [b][q2]
+  static_for<N>([&](auto bc) {
+    constexpr int B = decltype(bc)::value;
+    R p[N - B];
+#pragma unroll
+    for (int x = 0; x < N - B; ++x) p[x] = c[tri(B + x) + x];
+    interp_pencil<K, N - B>(p, u[B]);
+  });
+#pragma unroll
+  for (int q2 = 0; q2 <= K; ++q2) {
+    R p[N], v[K + 1];
+#pragma unroll
+    for (int b = 0; b < N; ++b) p[b] = u[b][q2];
+    interp_pencil<K, N>(p, v);
+#pragma unroll
+    for (int q1 = 0; q1 <= K; ++q1) put(q1, q2, v[q1]);
+  }
 }
-template <int N, int... A>
-__device__ __forceinline__ void pencil_modes_(int (&idx)[N], int d, int g, int b, int c,
-                                              std::integer_sequence<int, A...>) {
-  ((idx[A] = pencil_mode<A>(d, g, b, c)), ...);
-}
-template <int N>
-__device__ __forceinline__ void pencil_modes(int (&idx)[N], int d, int g, int b, int c) {
-  pencil_modes_(idx, d, g, b, c, std::make_integer_sequence<int, N>{});
+template <int K, int N, int ACC = 0, class R, class Get>
+__device__ __forceinline__ void project_triangle(Get get, R (&o)[N * (N + 1) / 2]) {
+  R u[N][K + 1];  // [b][q2]
+#pragma unroll
+  for (int q2 = 0; q2 <= K; ++q2) {
+    R v[K + 1], p[N];
+#pragma unroll
+    for (int q1 = 0; q1 <= K; ++q1) v[q1] = get(q1, q2);
+    project_pencil<K, N>(v, p);
+#pragma unroll
+    for (int b = 0; b < N; ++b) u[b][q2] = p[b];
+  }
+  static_for<N>([&](auto bc) {
+    constexpr int B = decltype(bc)::value;
+    R p[N - B];
+#pragma unroll
+    for (int x = 0; x < N - B; ++x) p[x] = ACC ? o[tri(B + x) + x] : R(0);
+    project_pencil<K, N - B, ACC>(u[B], p);
+#pragma unroll
+    for (int x = 0; x < N - B; ++x) o[tri(B + x) + x] = p[x];
+  });
 }
 
 // The warps of a CTA over the items of a phase. The items come in classes G = 0 .. NC-1 of
@@ -184,9 +242,8 @@ __device__ __forceinline__ void for_classes_(int t, int nw, int lane, Count coun
   }
 }
 template <int NC, class Count, class F>
-__device__ __forceinline__ int for_classes(int vw, int nw, int lane, Count count, F f) {
+__device__ __forceinline__ void for_classes(int vw, int nw, int lane, Count count, F f) {
   for_classes_<0, NC>(vw, nw, lane, count, f);
-  return vw;
 }
 
 __device__ __forceinline__ bool finite_bits(double x) { return (__double2hiint(x) & 0x7ff00000) != 0x7ff00000; }

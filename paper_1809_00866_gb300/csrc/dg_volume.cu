@@ -17,46 +17,51 @@
 //    so a warp runs one length and its 32 lanes are busy also where one element has few pencils.
 #include <algorithm>
 
+#include "dg_async.h"
 #include "dg_opargs.h"
-#include "dg_pencil.h"
+#include "dg_volume_phases.h"
 
 namespace dg {
 namespace {
 
 template <int K, class R, int E>
-struct VolSmem {
-  static constexpr int NB = nb_of(K), NBM = nb_of(K - 1), N1 = K + 1, NN = N1 * N1, NQ = NN * N1;
-  static constexpr int N2 = N1 * (K + 2) / 2;
-  static constexpr int LD = E + 1;  // elements of a row, odd: rows and elements both spread over the banks
-  static constexpr int GROW = 3 * N1 * NN;  // rows of X that hold the gradient while T1 / T2 fill the first ones
+struct VolSmem : VolPhases<K, R, E> {
+  using Ph = VolPhases<K, R, E>;
+  using Ph::GEO, Ph::LD, Ph::N1, Ph::NB, Ph::NN, Ph::NT;
+  // X: planes of (K+1)^2 rows (PL apart, odd), the fields at the (q1, q2) points per x exponent a in
+  // plane 3 a + f, then, in place, the products' projections in plane 6 a + sp: a thread of phase (3)
+  // reads and writes one row of every plane
+  static constexpr int PL = NN | 1;
+  static constexpr int GROW = 3 * N1 * PL;  // rows of X that hold the gradient meanwhile
   static constexpr int mx(int a, int b) { return a > b ? a : b; }
-  static constexpr int XROWS = mx(mx(6 * K * NN, GROW + 9 * NBM), 4 * NB);
+  static constexpr int XROWS = mx(mx(6 * K * PL, GROW + 9 * NT), 4 * NB);
   static constexpr int C = 0;                  // [4][NB] scaled coefficients
   static constexpr int T = C + 4 * NB * LD;    // [6][NBM] symmetric flux pairs
-  static constexpr int X = T + 6 * NBM * LD;   // the sum factorisation's partial results, in place; then the output
+  static constexpr int X = T + 6 * NT * LD;    // the sum factorisation's partial results, in place; then the output
   static constexpr int SC = X + XROWS * LD;    // [2][NB] mode scales and their inverses
-  static constexpr int GEO = SC + 2 * NB;      // [2 parities][E][8] 1/s, 2/h[3], A4/(2 s)[3], mass shift
-  static constexpr int REALS = GEO + 16 * E;
-  static constexpr size_t bytes() { return sizeof(R) * REALS + sizeof(int) * 12 * E; }  // + [2][E][6] face ids
+  static constexpr int GE = SC + 2 * NB;       // [2 parities][E][GEO]
+  static constexpr int REALS = GE + 2 * GEO * E;
+  static constexpr int INTS = 12 * E;          // [2 parities][E][6] face numbers
+  static constexpr size_t bytes() { return sizeof(R) * REALS + sizeof(int) * INTS; }
 };
 
 template <int K, int MODE, class R, int E>
-__global__ void __launch_bounds__(256, 2) vol_kernel(OpArgsT<R> a) {
+__global__ void __launch_bounds__(256, sizeof(R) == 4 ? 3 : 2) vol_kernel(OpArgsT<R> a) {
   using L = VolSmem<K, R, E>;
-  constexpr int NB = L::NB, NBM = L::NBM, N1 = L::N1, NN = L::NN, NQ = L::NQ, N2 = L::N2, LD = L::LD;
+  constexpr int N1 = L::N1, NN = L::NN, NQ = L::NQ, N2 = L::N2, NB = L::NB, NT = L::NT, PL = L::PL, LD = L::LD;
   constexpr bool kPoints = MODE != MODE_LINPART;
   extern __shared__ __align__(16) unsigned char smraw_[];
   R* sm = reinterpret_cast<R*>(smraw_);
   R* sC = sm + L::C;
   R* sT = sm + L::T;
   R* X = sm + L::X;
-  R* sS = sm + L::SC;
-  R* sI = sS + NB;
   int* sFid0 = reinterpret_cast<int*>(sm + L::REALS);
   const int tid = threadIdx.x, nt = blockDim.x, nw = nt >> 5, warp = tid >> 5, lane = tid & 31;
+  R* sS = sm + L::SC;
+  R* sI = sS + NB;
   for (int t = tid; t < NB; t += nt) {
-    sS[t] = R(mode_scale<K>.s[t]);
-    sI[t] = R(mode_scale<K>.inv[t]);
+    sS[t] = mode_scale<R, K>.s[t];
+    sI[t] = mode_scale<R, K>.inv[t];
   }
   __syncthreads();
   bool nonfinite = false;
@@ -65,113 +70,54 @@ __global__ void __launch_bounds__(256, 2) vol_kernel(OpArgsT<R> a) {
   // the warp that starts the task list moves on with every group, so that the remainders of the
   // task lists fall on all four schedulers of the SM alike
   int vw = (warp + blockIdx.x) % nw;
+  // the group's rows, copied while the previous group is stored, and its other inputs on their way to L2
+  auto fetch = [&](int grp) {
+    const int e0 = grp * E, cnt = min(E, a.M.ne - e0);
+    L::fetch(a.in, e0, cnt, sC, tid, nt);
+    if (tid == 0) {
+      if constexpr (MODE == MODE_TAN)
+        prefetch_l2(a.ubar + (size_t)e0 * 3 * NQ, a.ubar + (size_t)(e0 + cnt) * 3 * NQ);
+      if constexpr (E == kFaceGroup) {
+        const R* f = a.face_buf + face_record<N2>(face_slot(e0, 0), 0);
+        prefetch_l2(f, f + 21 * N2 * kFaceGroup);
+      }
+    }
+  };
+  if ((int)blockIdx.x < ngrp) fetch(blockIdx.x);
   for (int grp = blockIdx.x; grp < ngrp; grp += gridDim.x, par ^= 1) {
     const int e0 = grp * E, cnt = min(E, a.M.ne - e0);
-    R* sGeo = sm + L::GEO + par * 8 * E;
+    R* sGeo = sm + L::GE + par * L::GEO * E;
     int* sFid = sFid0 + par * 6 * E;
     vw = vw + 1 == nw ? 0 : vw + 1;
-    // scaled coefficients (rows of a partly filled group are zero), geometry, face numbers
-    for (int t = tid; t < E * 4 * NB; t += nt) {
-      const int e = t / (4 * NB), r = t - e * 4 * NB;
-      sC[r * LD + e] = e < cnt ? a.in[(size_t)e0 * 4 * NB + t] * sS[r % NB] : R(0);
-    }
-    for (int t = tid; t < 6 * E; t += nt) {
-      const int e = t / 6, sl = t - 6 * e, d = sl >> 1, el = e0 + (e < cnt ? e : 0);
-      int f = 3 * el + d;  // slot 2d+1: the element's own + face; 2d: its - neighbour's, or the wall below
-      if (!(sl & 1)) {
-        const int p = a.M.nbr[(size_t)el * 6 + sl];
-        f = p >= 0 ? 3 * p + d : 3 * a.M.ne + a.M.bslot[el];
-      }
-      sFid[t] = f;
-    }
-    for (int e = tid; e < E; e += nt) {
-      const R* g = geo_row<R>(a.M, e0 + (e < cnt ? e : 0));
-      R* o = sGeo + 8 * e;
-      o[0] = g[4];
-#pragma unroll
-      for (int d = 0; d < 3; ++d) {
-        o[1 + d] = g[5 + d];
-        o[4 + d] = R(0.125) * g[(d + 1) % 3] * g[(d + 2) % 3] * g[4];
-      }
-      o[7] = R(a.inv_gdt * a.M.geo[(size_t)(e0 + (e < cnt ? e : 0)) * kGeo + 11]);
-    }
+    L::meta(a.M, a.inv_gdt, e0, cnt, sGeo, sFid, tid, nt);
+    L::scale(sS, sC, tid, nt);
     __syncthreads();
-    // (1) nu times the corrected gradient, modes of degree <= K - 1: along axis d, with the
-    // scaled jumps f of the two faces and alpha = A4 / (2 s),
-    //   G_a = (2a+1) alpha/2 [4/s sum_{n = a+1, a+3, ..} c_n - (f_+ + (-1)^a f_-)]
-    for_classes<K>(vw, nw, lane, [](auto g) { return 3 * (decltype(g)::value + 1) * E; }, [&](auto gc, int it) {
-      constexpr int G = decltype(gc)::value, N = K + 1 - G;
-      const int e = it % E, p = it / E, d = p / (G + 1), c = p - d * (G + 1), b = G - c, j = tri(G) + c;
-      int idx[N];
-      pencil_modes(idx, d, G, b, c);
-      const R* ge = sGeo + 8 * e;
-      const R is4 = R(4) * ge[0], beta = R(0.5) * R(a.nu) * ge[4 + d];
-      const R* fp = a.face_buf + ((size_t)sFid[6 * e + 2 * d + 1] * 7 + 4) * N2 + j;
-      const R* fm = a.face_buf + ((size_t)sFid[6 * e + 2 * d] * 7 + 4) * N2 + j;
-      R bf[N - 1];
-#pragma unroll
-      for (int x = 0; x < N - 1; ++x) bf[x] = R(2 * x + 1) * beta;
-#pragma unroll
-      for (int av = 0; av < 3; ++av) {
-        const R f1 = fp[av * N2], f0 = fm[av * N2];
-        const R S = f1 + f0, D = f1 - f0;
-        R sg[N + 1];
-        sg[N - 1] = sg[N] = R(0);
-#pragma unroll
-        for (int x = N - 2; x >= 0; --x) {
-          const R cn = sC[(av * NB + idx[x + 1]) * LD + e];
-          sg[x] = x + 2 < N - 1 ? cn + sg[x + 2] : cn;
-          X[(L::GROW + (av * 3 + d) * NBM + idx[x]) * LD + e] = bf[x] * (is4 * sg[x] - (x % 2 ? D : S));
-        }
-      }
-    });
-    // interpolation step 1, along z: rows [(field, a)][b][q2]
+    // (1) corrected gradient
+    L::gradient(sC, a.face_buf, sGeo, sFid, a.nu, X + L::GROW * LD, vw, nw, lane);
+    // interpolation along z and y: for every x exponent a the triangle of the (y, z) exponents at the
+    // points, rows [(field, a)][q1 q2]
     if constexpr (kPoints)
-      for_classes<K + 1>(vw, nw, lane, [](auto g) { return 3 * (decltype(g)::value + 1) * E; }, [&](auto gc, int it) {
-        constexpr int G = decltype(gc)::value, N = K + 1 - G;
-        const int e = it % E, p = it / E, f = p / (G + 1), b = p - f * (G + 1), ax = G - b;
-        int idx[N];
-        pencil_modes(idx, 2, G, ax, b);
-        R c[N], v[N1];
-#pragma unroll
-        for (int x = 0; x < N; ++x) c[x] = sC[(f * NB + idx[x]) * LD + e];
-        interp_pencil<K, N>(c, v);
-#pragma unroll
-        for (int q = 0; q < N1; ++q) X[((f * N1 + ax) * NN + b * N1 + q) * LD + e] = v[q];
+      for_classes<K + 1>(vw, nw, lane, [](auto) { return 3 * E; }, [&](auto ac, int it) {
+        constexpr int A = decltype(ac)::value, N = K + 1 - A;
+        const int f = it / E, e = it - f * E;
+        const R* ce = sC + f * NB * LD + e;
+        R* x = X + (3 * A + f) * PL * LD + e;
+        R c[tri(N)];
+        static_for<tri(N)>([&](auto jc) {
+          constexpr int J = decltype(jc)::value, GD = face_degree(J), z = J - tri(GD);
+          c[J] = ce[mode_at(A, GD - z, z) * LD];
+        });
+        interp_triangle<K, N>(c, [&](int q1, int q2, R v) { x[(q1 * N1 + q2) * LD] = v; });
       });
     __syncthreads();
-    // (2) viscous flux minus pressure, nu (G_ip + G_pi - 2/3 delta tr G) - delta p, and
-    // interpolation step 2, along y
-    for_classes<1>(vw, nw, lane, [](auto) { return NBM * E; }, [&](auto, int it) {
-      const int e = it % E, m = it / E;
-      auto g = [&](int av, int b) { return X[(L::GROW + (av * 3 + b) * NBM + m) * LD + e]; };
-      const R g00 = g(0, 0), g11 = g(1, 1), g22 = g(2, 2);
-      const R tr = R(2.0 / 3.0) * (g00 + g11 + g22) + sC[(3 * NB + m) * LD + e];
-      R* t = sT + m * LD + e;
-      t[0 * NBM * LD] = R(2) * g00 - tr;
-      t[1 * NBM * LD] = R(2) * g11 - tr;
-      t[2 * NBM * LD] = R(2) * g22 - tr;
-      t[3 * NBM * LD] = g(0, 1) + g(1, 0);
-      t[4 * NBM * LD] = g(0, 2) + g(2, 0);
-      t[5 * NBM * LD] = g(1, 2) + g(2, 1);
-    });
+    // (2) viscous flux minus pressure
+    L::viscous(sC, X + L::GROW * LD, sT, vw, nw, lane);
     if constexpr (kPoints) {
-      for_classes<K + 1>(vw, nw, lane, [](auto) { return 3 * N1 * E; }, [&](auto gc, int it) {
-        constexpr int G = decltype(gc)::value, N = K + 1 - G;
-        const int e = it % E, p = it / E, f = p / N1, q2 = p - f * N1;
-        R* x = X + ((f * N1 + G) * NN + q2) * LD + e;
-        R c[N], v[N1];
-#pragma unroll
-        for (int b = 0; b < N; ++b) c[b] = x[b * N1 * LD];
-        interp_pencil<K, N>(c, v);
-#pragma unroll
-        for (int q = 0; q < N1; ++q) x[q * N1 * LD] = v[q];
-      });
       __syncthreads();
       // (3) one pencil of points along x per thread: interpolation step 3, the products with the
       // linearisation velocity (or with itself), projection step 1; rows [(product, a)][q1 q2]
       for_classes<1>(vw, nw, lane, [](auto) { return NN * E; }, [&](auto, int it) {
-        const int e = it / NN, r = it - e * NN;
+        const int r = it / E, e = it - r * E;
         const bool on = e < cnt;
         R* x = X + r * LD + e;
         R u[3][N1], ub[3][N1];
@@ -179,7 +125,7 @@ __global__ void __launch_bounds__(256, 2) vol_kernel(OpArgsT<R> a) {
         for (int f = 0; f < 3; ++f) {
           R c[N1];
 #pragma unroll
-          for (int n = 0; n < N1; ++n) c[n] = x[(f * N1 + n) * NN * LD];
+          for (int n = 0; n < N1; ++n) c[n] = x[(3 * n + f) * PL * LD];
           interp_pencil<K, N1>(c, u[f]);
         }
         R* ug = a.ubar + (size_t)(e0 + (on ? e : 0)) * 3 * NQ + r;
@@ -208,82 +154,66 @@ __global__ void __launch_bounds__(256, 2) vol_kernel(OpArgsT<R> a) {
           if (MODE == MODE_TAN && sp < 3) project_pencil<K, K, 0, true>(v, o);
           else project_pencil<K, K>(v, o);
 #pragma unroll
-          for (int n = 0; n < K; ++n) x[(sp * K + n) * NN * LD] = o[n];
+          for (int n = 0; n < K; ++n) x[(6 * n + sp) * PL * LD] = o[n];
         }
       });
       __syncthreads();
-      // (4) projection step 2, along y, in place
-      for_classes<K>(vw, nw, lane, [](auto) { return 6 * N1 * E; }, [&](auto gc, int it) {
-        constexpr int G = decltype(gc)::value, N = K - G;
-        const int e = it % E, p = it / E, sp = p / N1, q2 = p - sp * N1;
-        R* x = X + ((sp * K + G) * NN + q2) * LD + e;
-        R v[N1], o[N];
+      // (4) projection along y and z, taken off the viscous flux: in FP32 for every x exponent a the
+      // points (q1 q2) onto the triangle of the (y, z) exponents in one thread's registers; in FP64,
+      // where idle lanes cost pipe time (6 x 8 items are one and a half warps), in two steps
+      if constexpr (sizeof(R) == 4) {
+        for_classes<K>(vw, nw, lane, [](auto) { return 6 * E; }, [&](auto ac, int it) {
+          constexpr int A = decltype(ac)::value, N = K - A;
+          const int sp = it / E, e = it - sp * E;
+          const R* x = X + (6 * A + sp) * PL * LD + e;
+          R* t = sT + sp * NT * LD + e;
+          R o[tri(N)];
+          static_for<tri(N)>([&](auto jc) {
+            constexpr int J = decltype(jc)::value, GD = face_degree(J), z = J - tri(GD);
+            o[J] = t[mode_at(A, GD - z, z) * LD];
+          });
+          project_triangle<K, N, -1>([&](int q1, int q2) { return x[(q1 * N1 + q2) * LD]; }, o);
+          static_for<tri(N)>([&](auto jc) {
+            constexpr int J = decltype(jc)::value, GD = face_degree(J), z = J - tri(GD);
+            t[mode_at(A, GD - z, z) * LD] = o[J];
+          });
+        });
+      } else {
+        for_classes<K>(vw, nw, lane, [](auto) { return 6 * N1 * E; }, [&](auto gc, int it) {
+          constexpr int G = decltype(gc)::value, N = K - G;
+          const int e = it % E, p = it / E, sp = p / N1, q2 = p - sp * N1;
+          R* x = X + ((6 * G + sp) * PL + q2) * LD + e;
+          R v[N1], o[N];
 #pragma unroll
-        for (int q = 0; q < N1; ++q) v[q] = x[q * N1 * LD];
-        project_pencil<K, N>(v, o);
+          for (int q = 0; q < N1; ++q) v[q] = x[q * N1 * LD];
+          project_pencil<K, N>(v, o);
 #pragma unroll
-        for (int n = 0; n < N; ++n) x[n * N1 * LD] = o[n];
-      });
-      __syncthreads();
-      // (5) projection step 3, along z, taken off the viscous flux
-      for_classes<K>(vw, nw, lane, [](auto g) { return 6 * (decltype(g)::value + 1) * E; }, [&](auto gc, int it) {
-        constexpr int G = decltype(gc)::value, N = K - G;
-        const int e = it % E, p = it / E, sp = p / (G + 1), b = p - sp * (G + 1), ax = G - b;
-        int idx[N];
-        pencil_modes(idx, 2, G, ax, b);
-        const R* x = X + ((sp * K + ax) * NN + b * N1) * LD + e;
-        R* t = sT + sp * NBM * LD + e;
-        R v[N1], o[N];
+          for (int n = 0; n < N; ++n) x[n * N1 * LD] = o[n];
+        });
+        __syncthreads();
+        for_classes<K>(vw, nw, lane, [](auto g) { return 6 * (decltype(g)::value + 1) * E; }, [&](auto gc, int it) {
+          constexpr int G = decltype(gc)::value, N = K - G;
+          const int e = it % E, p = it / E, sp = p / (G + 1), b = p - sp * (G + 1), ax = G - b;
+          const R* x = X + ((6 * ax + sp) * PL + b * N1) * LD + e;
+          R* t = sT + sp * NT * LD + e;
+          R v[N1], o[N];
 #pragma unroll
-        for (int q = 0; q < N1; ++q) v[q] = x[q * LD];
+          for (int q = 0; q < N1; ++q) v[q] = x[q * LD];
 #pragma unroll
-        for (int n = 0; n < N; ++n) o[n] = t[idx[n] * LD];
-        project_pencil<K, N, -1>(v, o);
+          for (int n = 0; n < N; ++n) o[n] = t[mode_at(ax, b, n) * LD];
+          project_pencil<K, N, -1>(v, o);
 #pragma unroll
-        for (int n = 0; n < N; ++n) t[idx[n] * LD] = o[n];
-      });
+          for (int n = 0; n < N; ++n) t[mode_at(ax, b, n) * LD] = o[n];
+        });
+      }
     }
     __syncthreads();
-    // (6) modal derivatives of the fluxes (continuity: of -u) and the face terms, axis by axis:
-    //   out_a += (2a+1) [2/h sum_{n = a-1, a-3, ..} T_n + alpha (F_+ - (-1)^a F_-)]
-#pragma unroll
-    for (int d = 0; d < 3; ++d) {
-      for_classes<K + 1>(vw, nw, lane, [](auto g) { return 4 * (decltype(g)::value + 1) * E; }, [&](auto gc, int it) {
-        constexpr int G = decltype(gc)::value, N = K + 1 - G;
-        const int e = it % E, p = it / E, i = p / (G + 1), c = p - i * (G + 1), b = G - c, j = tri(G) + c;
-        int idx[N];
-        pencil_modes(idx, d, G, b, c);
-        const R* ge = sGeo + 8 * e;
-        const R al = ge[4 + d], J = i == 3 ? -ge[1 + d] : ge[1 + d];
-        const R fp = a.face_buf[((size_t)sFid[6 * e + 2 * d + 1] * 7 + i) * N2 + j];
-        const R fm = a.face_buf[((size_t)sFid[6 * e + 2 * d] * 7 + i) * N2 + j];
-        const R se = al * (fp - fm), so = al * (fp + fm);
-        const R* t = (i == 3 ? sC + d * NB * LD : sT + (i == d ? d : i + d + 2) * NBM * LD) + e;
-        R* o = X + i * NB * LD + e;
-        R pi[N + 1];
-        pi[0] = R(0);
-#pragma unroll
-        for (int x = 0; x < N; ++x) {
-          if (x >= 1) {
-            const R tn = t[idx[x - 1] * LD];
-            pi[x] = x >= 3 ? tn + pi[x - 2] : tn;
-          }
-          const R s = x % 2 ? so : se;
-          const R v = x ? J * pi[x] + s : s;
-          o[idx[x] * LD] = d ? o[idx[x] * LD] + R(2 * x + 1) * v : R(2 * x + 1) * v;
-        }
-      });
-      __syncthreads();
-    }
-    // (7) back to the orthonormal basis, mass shift, output
-    for (int t = tid; t < cnt * 4 * NB; t += nt) {
-      const int e = t / (4 * NB), r = t - e * 4 * NB;
-      R v = X[r * LD + e] * sI[r % NB];
-      if (MODE == MODE_TAN && r < 3 * NB) v += sGeo[8 * e + 7] * a.in[(size_t)e0 * 4 * NB + t];
-      nonfinite |= !finite_bits(v);
-      a.out[(size_t)e0 * 4 * NB + t] = v;
-    }
-    // the next group's first writes go to sC and the other parity's geometry, which (7) does not read
+    // (5) modal derivatives of the fluxes and the face terms; (6) output
+    L::divergence(sC, sT, a.face_buf, sGeo, sFid, X, vw, nw, lane);
+    __syncthreads();
+    if (grp + (int)gridDim.x < ngrp) fetch(grp + gridDim.x);
+    nonfinite |= L::template store<MODE == MODE_TAN>(a.in, a.out, e0, cnt, sI, X, sGeo, tid, nt);
+    // the next group's first writes go to sC and the other parity's geometry, which (6) does not read
   }
   // scan of the outputs: a non-finite entry (from a non-finite input or an overflow) sets the
   // status bit, once per thread that wrote one
