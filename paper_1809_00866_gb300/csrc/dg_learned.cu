@@ -293,23 +293,36 @@ __global__ void __launch_bounds__(32 * kWarps) mlp_forward_kernel(const unsigned
 }
 
 // -------------------------------------------------------------- training
-// One CTA: forward and backward of 64 samples, then its share of the weight gradient
+// One CTA: forward and backward of 128 samples, then its share of the weight gradient
 // dW = dZ^T H (a contraction over its samples) on the tensor cores, written as one
 // partial row; grad_reduce_kernel sums the rows in a fixed order.
-constexpr int kLdT = 72;  // feature-major tiles [feature][64 samples + 8] (bank-conflict-free fragments)
-constexpr int sXT = kPBytes;
-constexpr int sH1T = sXT + kIn * kLdT * 2;
-constexpr int sH2T = sH1T + kHid * kLdT * 2;
-constexpr int sDZ1T = sH2T + kHid * kLdT * 2;
-constexpr int sDZ2T = sDZ1T + kHid * kLdT * 2;
-constexpr int sDYT = sDZ2T + kHid * kLdT * 2;
-constexpr int sG = sDYT + kOut * kLdT * 2;           // gelu' of layers 1, 2: [warp][2][64 regs][32 lanes] bf16
-constexpr int sBsum = sG + kWarps * 2 * 64 * 32 * 2;  // [warp][128 + 128 + 16] column sums of dZ1, dZ2, dY
-constexpr int sLoss = sBsum + kWarps * (2 * kHid + kOut) * 4;
-constexpr int kTrainSmem = sLoss + 16 * 4;
-constexpr int kPartLd = kNP + 16;  // partial row: gradient, then the loss sum
+//
+// Latency and issue bound it (the arithmetic of 16384 samples is 2.8 GFMA, the data 8.4 MB):
+// GELU and its derivative cost about as many issue slots as everything else, and one warp's
+// chain of layers is serial. So a CTA has 16 warps, each with a 32 x 32 tile of every
+// 128-wide layer: the four warps of a 32-sample stripe exchange activations through shared
+// memory under a barrier of their own, so that stripes drift apart and one's matrix products
+// run beside another's GELU. Every tile is kept sample-major and read by ldmatrix, transposed
+// where the samples are the contraction, and the 16384 samples are one wave of 128 CTAs.
+// gelu' stays in registers. With four warps per CTA, each with 16 samples and all columns,
+// feature-major copies by 2-byte stores and 64 samples per CTA (1.7 waves):
+// 63 us at 16384 samples; now 19 us.
+constexpr int kTRows = 128, kTWarps = 16, kStripes = 4, kLdY = 24;
+constexpr int sX = kPBytes;
+constexpr int sH1 = sX + kTRows * kLd1 * 2;
+constexpr int sH2 = sH1 + kTRows * kLd2 * 2;
+constexpr int sDZ2 = sH2 + kTRows * kLd2 * 2;
+constexpr int sDY = sDZ2 + kTRows * kLd2 * 2;
+constexpr int sDZ1 = kPW2;                       // takes the place of W2 once dH1 has been formed
+constexpr int sBsum = sDY + kTRows * kLdY * 2;   // [stripe][128 + 128 + 16] column sums of dZ1, dZ2, dY
+constexpr int sLoss = sBsum + kStripes * (2 * kHid + kOut) * 4;
+constexpr int sRow = sLoss + kTWarps * 4;        // the pair each sample slot holds, -1 past the batch
+constexpr int kTrainSmem = sRow + kTRows * 8;
+constexpr int kPartLd = kNP + 16;                // partial row: gradient, then the loss sum
 static_assert(kTrainSmem <= 227 * 1024, "training tile exceeds shared memory");
-static_assert(sXT % 16 == 0 && sG % 16 == 0 && sBsum % 16 == 0, "alignment");
+static_assert(sX % 16 == 0 && sH1 % 16 == 0 && sDY % 16 == 0 && sBsum % 16 == 0 && sRow % 8 == 0, "alignment");
+static_assert(kHid * kLd2 >= kTRows * kLd2, "dZ1 fits in the place of W2");
+static_assert(kPartLd % 4 == 0 && kPBytes % 16 == 0, "partial rows are read by 16 bytes");
 
 __device__ __forceinline__ long long sample_row(long long seed, long long step, long long s, long long npairs) {
   if (seed < 0) return s;
@@ -323,96 +336,184 @@ __device__ __forceinline__ long long sample_row(long long seed, long long step, 
   return (long long)(z % (unsigned long long)npairs);
 }
 
-// store a feature-major BF16 value T[col][s]
-__device__ __forceinline__ void stT(unsigned char* sm, int off, int col, int s, uint16_t v) {
-  reinterpret_cast<uint16_t*>(sm + off)[col * kLdT + s] = v;
+// four 8 x 8 BF16 matrices, one row address per lane; trans: each is transposed on the way
+template <bool TRANS>
+__device__ __forceinline__ void ldmatrix4(uint32_t (&r)[4], const unsigned char* p) {
+  const uint32_t a = static_cast<uint32_t>(__cvta_generic_to_shared(p));
+  if constexpr (TRANS)
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(a) : "memory");
+  else
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(a) : "memory");
 }
 
-// column sums over the 16 rows of a warp of C-fragment values v[j][4] (cols 8j+2t, +1)
-template <int NB>
-__device__ __forceinline__ void warp_colsum(const float (&v)[NB][4], float* dst, int lane) {
+// acc[mt][nt] += A B over KS steps of 16 for a (16 MT) x (8 NT) tile at (m0, n0).
+// A: [m][k] in shared memory, or [k][m] with TA; B: [n][k], or [k][n] with TB; LDA, LDB the
+// row lengths. With TA or TB the matrix loads transpose.
+template <int MT, int NT, int KS, bool TA, bool TB, int LDA, int LDB>
+__device__ __forceinline__ void tile_mma(const unsigned char* A, const unsigned char* B, int m0, int n0, int lane,
+                                         float (&acc)[MT][NT][4]) {
+  static_assert(NT % 2 == 0, "B is loaded two column groups at a time");
+  const int lo = lane & 7, q = (lane >> 3) & 1, hi = lane >> 4;
+  const unsigned char* pa = A + 2 * (TA ? (lo + 8 * hi) * LDA + m0 + 8 * q : (m0 + lo + 8 * q) * LDA + 8 * hi);
+  const unsigned char* pb = B + 2 * (TB ? (lo + 8 * q) * LDB + n0 + 8 * hi : (n0 + lo + 8 * hi) * LDB + 8 * q);
 #pragma unroll
-  for (int j = 0; j < NB; ++j) {
-    float c0 = v[j][0] + v[j][2], c1 = v[j][1] + v[j][3];
+  for (int k = 0; k < KS; ++k) {
+    uint32_t a[MT][4], b[NT / 2][4];
+#pragma unroll
+    for (int m = 0; m < MT; ++m) ldmatrix4<TA>(a[m], pa + 2 * (TA ? 16 * k * LDA + 16 * m : 16 * m * LDA + 16 * k));
+#pragma unroll
+    for (int n = 0; n < NT / 2; ++n) ldmatrix4<TB>(b[n], pb + 2 * (TB ? 16 * k * LDB + 16 * n : 16 * n * LDB + 16 * k));
+#pragma unroll
+    for (int m = 0; m < MT; ++m)
+#pragma unroll
+      for (int n = 0; n < NT; ++n) mma16816(acc[m][n], a[m], b[n >> 1][2 * (n & 1)], b[n >> 1][2 * (n & 1) + 1]);
+  }
+}
+
+template <int MT, int NT>
+__device__ __forceinline__ void zero_tile(float (&acc)[MT][NT][4]) {
+#pragma unroll
+  for (int m = 0; m < MT; ++m)
+#pragma unroll
+    for (int n = 0; n < NT; ++n) acc[m][n][0] = acc[m][n][1] = acc[m][n][2] = acc[m][n][3] = 0.f;
+}
+
+// a tile as BF16 into a sample-major array [sample][LD] at (m0, n0)
+template <int MT, int NT, int LD>
+__device__ __forceinline__ void put_tile(unsigned char* dst, int m0, int n0, int g, int t,
+                                         const float (&v)[MT][NT][4]) {
+#pragma unroll
+  for (int m = 0; m < MT; ++m)
+#pragma unroll
+    for (int n = 0; n < NT; ++n) {
+      unsigned char* p = dst + 2 * ((m0 + 16 * m + g) * LD + n0 + 8 * n + 2 * t);
+      *reinterpret_cast<uint32_t*>(p) = pack2(v[m][n][0], v[m][n][1]);
+      *reinterpret_cast<uint32_t*>(p + 16 * LD) = pack2(v[m][n][2], v[m][n][3]);
+    }
+}
+
+// a tile in FP32 into the row-major matrix dst [.][ld] at (m0, n0)
+template <int MT, int NT>
+__device__ __forceinline__ void put_grad(float* dst, int ld, int m0, int n0, int g, int t,
+                                         const float (&v)[MT][NT][4]) {
+#pragma unroll
+  for (int m = 0; m < MT; ++m)
+#pragma unroll
+    for (int n = 0; n < NT; ++n) {
+      float* p = dst + (m0 + 16 * m + g) * ld + n0 + 8 * n + 2 * t;
+      *reinterpret_cast<float2*>(p) = make_float2(v[m][n][0], v[m][n][1]);
+      *reinterpret_cast<float2*>(p + 8 * ld) = make_float2(v[m][n][2], v[m][n][3]);
+    }
+}
+
+// column sums over the rows of a tile -> dst[8 n + .]
+template <int MT, int NT>
+__device__ __forceinline__ void tile_colsum(const float (&v)[MT][NT][4], float* dst, int lane) {
+#pragma unroll
+  for (int n = 0; n < NT; ++n) {
+    float c0 = 0.f, c1 = 0.f;
+#pragma unroll
+    for (int m = 0; m < MT; ++m) {
+      c0 += v[m][n][0] + v[m][n][2];
+      c1 += v[m][n][1] + v[m][n][3];
+    }
 #pragma unroll
     for (int o = 4; o < 32; o <<= 1) {
       c0 += __shfl_xor_sync(0xffffffffu, c0, o);
       c1 += __shfl_xor_sync(0xffffffffu, c1, o);
     }
     if (lane < 4) {
-      dst[8 * j + 2 * lane] = c0;
-      dst[8 * j + 2 * lane + 1] = c1;
+      dst[8 * n + 2 * lane] = c0;
+      dst[8 * n + 2 * lane + 1] = c1;
     }
   }
 }
 
-// one 16-row block of dW = A B^T over the CTA's 64 samples: A rows from the feature-major
-// tile at offA (rows m0..m0+15), B rows nb = 0..NB-1 of the tile at offB; writes NB tiles.
-template <int NB>
-__device__ __forceinline__ void wgrad_block(const unsigned char* sm, int offA, int m0, int offB, int nb0, int g, int t,
-                                            float* dst, int ldd) {
-  const uint16_t* A = reinterpret_cast<const uint16_t*>(sm + offA);
-  const uint16_t* B = reinterpret_cast<const uint16_t*>(sm + offB);
-  float acc[NB][4];
+// acc = bias, per column
+template <int MT, int NT>
+__device__ __forceinline__ void bias_tile(const float* b, int n0, int t, float (&acc)[MT][NT][4]) {
 #pragma unroll
-  for (int j = 0; j < NB; ++j) acc[j][0] = acc[j][1] = acc[j][2] = acc[j][3] = 0.f;
+  for (int n = 0; n < NT; ++n) {
+    const float2 bb = *reinterpret_cast<const float2*>(b + n0 + 8 * n + 2 * t);
 #pragma unroll
-  for (int kk = 0; kk < 4; ++kk) {
-    uint32_t a[4];
-    a[0] = *reinterpret_cast<const uint32_t*>(A + (m0 + g) * kLdT + 16 * kk + 2 * t);
-    a[1] = *reinterpret_cast<const uint32_t*>(A + (m0 + g + 8) * kLdT + 16 * kk + 2 * t);
-    a[2] = *reinterpret_cast<const uint32_t*>(A + (m0 + g) * kLdT + 16 * kk + 8 + 2 * t);
-    a[3] = *reinterpret_cast<const uint32_t*>(A + (m0 + g + 8) * kLdT + 16 * kk + 8 + 2 * t);
-#pragma unroll
-    for (int j = 0; j < NB; ++j) {
-      const uint16_t* b = B + (8 * (nb0 + j) + g) * kLdT + 16 * kk + 2 * t;
-      mma16816(acc[j], a, *reinterpret_cast<const uint32_t*>(b), *reinterpret_cast<const uint32_t*>(b + 8));
+    for (int m = 0; m < MT; ++m) {
+      acc[m][n][0] = acc[m][n][2] = bb.x;
+      acc[m][n][1] = acc[m][n][3] = bb.y;
     }
-  }
-#pragma unroll
-  for (int j = 0; j < NB; ++j) {
-    const int c = 8 * (nb0 + j) + 2 * t;
-    *reinterpret_cast<float2*>(dst + (m0 + g) * ldd + c) = make_float2(acc[j][0], acc[j][1]);
-    *reinterpret_cast<float2*>(dst + (m0 + g + 8) * ldd + c) = make_float2(acc[j][2], acc[j][3]);
   }
 }
 
-__global__ void __launch_bounds__(32 * kWarps) mlp_grad_kernel(const unsigned char* __restrict__ net,
-                                                               const float* __restrict__ X, const float* __restrict__ T,
-                                                               long long npairs, int batch, long long seed,
-                                                               long long step, float* __restrict__ part,
-                                                               unsigned* status) {
+// z -> gelu(z) in place; gelu'(z) as packed BF16
+__device__ __forceinline__ void gelu_tile(float (&z)[2][4][4], uint32_t (&d)[2][4][2]) {
+#pragma unroll
+  for (int m = 0; m < 2; ++m)
+#pragma unroll
+    for (int n = 0; n < 4; ++n)
+#pragma unroll
+      for (int q = 0; q < 2; ++q) {
+        const float z0 = z[m][n][2 * q], z1 = z[m][n][2 * q + 1];
+        d[m][n][q] = pack2(gelu_d(z0), gelu_d(z1));
+        z[m][n][2 * q] = gelu(z0);
+        z[m][n][2 * q + 1] = gelu(z1);
+      }
+}
+
+__device__ __forceinline__ void scale_tile(float (&v)[2][4][4], const uint32_t (&d)[2][4][2]) {
+#pragma unroll
+  for (int m = 0; m < 2; ++m)
+#pragma unroll
+    for (int n = 0; n < 4; ++n)
+#pragma unroll
+      for (int q = 0; q < 2; ++q) {
+        v[m][n][2 * q] *= bf16_to_f(d[m][n][q] & 0xffff);
+        v[m][n][2 * q + 1] *= bf16_to_f(d[m][n][q] >> 16);
+      }
+}
+
+// the 128 threads of one 32-sample stripe
+__device__ __forceinline__ void stripe_sync(int stripe) {
+  asm volatile("bar.sync %0, %1;" ::"r"(stripe + 1), "r"(32 * kTWarps / kStripes) : "memory");
+}
+
+__global__ void __launch_bounds__(32 * kTWarps, 1) mlp_grad_kernel(const unsigned char* __restrict__ net,
+                                                                  const float* __restrict__ X,
+                                                                  const float* __restrict__ T, long long npairs,
+                                                                  int batch, long long seed, long long step,
+                                                                  float* __restrict__ part, unsigned* status) {
   extern __shared__ __align__(128) unsigned char sm[];
   __shared__ uint64_t bar;
   __shared__ int ok_all;
-  start_weights(sm, net, &bar);
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
-  const int la = warp * 16 + g, lb = la + 8;  // local sample slots
-  const long long sa = (long long)blockIdx.x * kRows + la, sb = sa + 8;
-  const bool va = sa < batch, vb = sb < batch;
-  const long long ra = va ? sample_row(seed, step, sa, npairs) : 0, rb = vb ? sample_row(seed, step, sb, npairs) : 0;
-  // inputs: A fragments and the feature-major copy XT
-  uint32_t a1[7][4];
-#pragma unroll
-  for (int kk = 0; kk < 7; ++kk) {
-    float2 p0 = make_float2(0.f, 0.f), p1 = p0, p2 = p0, p3 = p0;
-    if (va) {
-      p0 = *reinterpret_cast<const float2*>(X + ra * kIn + 16 * kk + 2 * t);
-      p2 = *reinterpret_cast<const float2*>(X + ra * kIn + 16 * kk + 8 + 2 * t);
-    }
-    if (vb) {
-      p1 = *reinterpret_cast<const float2*>(X + rb * kIn + 16 * kk + 2 * t);
-      p3 = *reinterpret_cast<const float2*>(X + rb * kIn + 16 * kk + 8 + 2 * t);
-    }
-    a1[kk][0] = pack2(p0.x, p0.y);
-    a1[kk][1] = pack2(p1.x, p1.y);
-    a1[kk][2] = pack2(p2.x, p2.y);
-    a1[kk][3] = pack2(p3.x, p3.y);
+  long long* row = reinterpret_cast<long long*>(sm + sRow);
+  if (threadIdx.x < kTRows) {
+    const long long s = (long long)blockIdx.x * kTRows + threadIdx.x;
+    row[threadIdx.x] = s < batch ? sample_row(seed, step, s, npairs) : -1;
   }
   if (threadIdx.x == 0) ok_all = 1;
-  const bool ok = mbar_wait(&bar, 0);
-  __syncthreads();
-  if (!ok) ok_all = 0;
+  start_weights(sm, net, &bar);  // its barrier also orders row[] and ok_all
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
+  const int stripe = warp / (kTWarps / kStripes), wc = warp % (kTWarps / kStripes);
+  const int m0 = 32 * stripe, n0 = 32 * wc;
+  {
+    // the samples' features, BF16: 28 groups of four per row
+    constexpr int kC4 = kIn / 4, kN = kTRows * kC4 / (32 * kTWarps);
+    static_assert(kTRows * kC4 % (32 * kTWarps) == 0, "whole groups per thread");
+    float4 v[kN];
+#pragma unroll
+    for (int i = 0; i < kN; ++i) {
+      const int c = threadIdx.x + i * 32 * kTWarps;
+      const long long r = row[c / kC4];
+      v[i] = r >= 0 ? *reinterpret_cast<const float4*>(X + r * kIn + 4 * (c % kC4)) : make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+#pragma unroll
+    for (int i = 0; i < kN; ++i) {
+      const int c = threadIdx.x + i * 32 * kTWarps;
+      *reinterpret_cast<uint2*>(sm + sX + 2 * ((c / kC4) * kLd1 + 4 * (c % kC4))) =
+          make_uint2(pack2(v[i].x, v[i].y), pack2(v[i].z, v[i].w));
+    }
+  }
+  if (!mbar_wait(&bar, 0)) ok_all = 0;
   __syncthreads();
   if (!ok_all) {
     if (threadIdx.x == 0) {  // report; the copy in flight lands before the CTA leaves
@@ -422,190 +523,131 @@ __global__ void __launch_bounds__(32 * kWarps) mlp_grad_kernel(const unsigned ch
     __syncthreads();
     return;
   }
-  // XT (after the weights landed: the bulk copy only writes the network region)
-#pragma unroll
-  for (int kk = 0; kk < 7; ++kk) {
-    const int c = 16 * kk + 2 * t;
-    stT(sm, sXT, c, la, a1[kk][0] & 0xffff); stT(sm, sXT, c + 1, la, a1[kk][0] >> 16);
-    stT(sm, sXT, c, lb, a1[kk][1] & 0xffff); stT(sm, sXT, c + 1, lb, a1[kk][1] >> 16);
-    stT(sm, sXT, c + 8, la, a1[kk][2] & 0xffff); stT(sm, sXT, c + 9, la, a1[kk][2] >> 16);
-    stT(sm, sXT, c + 8, lb, a1[kk][3] & 0xffff); stT(sm, sXT, c + 9, lb, a1[kk][3] >> 16);
-  }
-  uint16_t* Gs = reinterpret_cast<uint16_t*>(sm + sG) + warp * 2 * 64 * 32;
-  const uint16_t* W2s = reinterpret_cast<const uint16_t*>(sm + kPW2);
-  const uint16_t* W3s = reinterpret_cast<const uint16_t*>(sm + kPW3);
-  const uint16_t* W1s = reinterpret_cast<const uint16_t*>(sm + kPW1);
   const float* Bs = reinterpret_cast<const float*>(sm + kPB);
-  float* bsum = reinterpret_cast<float*>(sm + sBsum) + warp * (2 * kHid + kOut);
-  float acc[16][4];
-  uint32_t a[8][4];
-  // ---- forward: layer 1
-#pragma unroll
-  for (int j = 0; j < 16; ++j) {
-    const float2 bb = *reinterpret_cast<const float2*>(Bs + 8 * j + 2 * t);
-    acc[j][0] = bb.x; acc[j][1] = bb.y; acc[j][2] = bb.x; acc[j][3] = bb.y;
-  }
-#pragma unroll
-  for (int kk = 0; kk < 7; ++kk)
-#pragma unroll
-    for (int j = 0; j < 16; ++j) {
-      const uint32_t* w = reinterpret_cast<const uint32_t*>(W1s + (8 * j + g) * kLd1 + 16 * kk + 2 * t);
-      mma16816(acc[j], a1[kk], w[0], w[4]);
-    }
-  // H1 = gelu(Z1) (A fragments and H1T), G1 = gelu'(Z1)
-#pragma unroll
-  for (int j = 0; j < 16; ++j) {
-    const int c = 8 * j + 2 * t;
-#pragma unroll
-    for (int q = 0; q < 4; ++q) Gs[(0 * 64 + 4 * j + q) * 32 + lane] = bf16_bits(gelu_d(acc[j][q]));
-    const uint32_t lo = pack2(gelu(acc[j][0]), gelu(acc[j][1])), hi = pack2(gelu(acc[j][2]), gelu(acc[j][3]));
-    a[j >> 1][(j & 1) * 2 + 0] = lo;
-    a[j >> 1][(j & 1) * 2 + 1] = hi;
-    stT(sm, sH1T, c, la, lo & 0xffff); stT(sm, sH1T, c + 1, la, lo >> 16);
-    stT(sm, sH1T, c, lb, hi & 0xffff); stT(sm, sH1T, c + 1, lb, hi >> 16);
-  }
-  // ---- layer 2
-#pragma unroll
-  for (int j = 0; j < 16; ++j) {
-    const float2 bb = *reinterpret_cast<const float2*>(Bs + kHid + 8 * j + 2 * t);
-    acc[j][0] = bb.x; acc[j][1] = bb.y; acc[j][2] = bb.x; acc[j][3] = bb.y;
-  }
-#pragma unroll
-  for (int kk = 0; kk < 8; ++kk)
-#pragma unroll
-    for (int j = 0; j < 16; ++j) {
-      const uint32_t* w = reinterpret_cast<const uint32_t*>(W2s + (8 * j + g) * kLd2 + 16 * kk + 2 * t);
-      mma16816(acc[j], a[kk], w[0], w[4]);
-    }
-#pragma unroll
-  for (int j = 0; j < 16; ++j) {
-    const int c = 8 * j + 2 * t;
-#pragma unroll
-    for (int q = 0; q < 4; ++q) Gs[(1 * 64 + 4 * j + q) * 32 + lane] = bf16_bits(gelu_d(acc[j][q]));
-    const uint32_t lo = pack2(gelu(acc[j][0]), gelu(acc[j][1])), hi = pack2(gelu(acc[j][2]), gelu(acc[j][3]));
-    a[j >> 1][(j & 1) * 2 + 0] = lo;
-    a[j >> 1][(j & 1) * 2 + 1] = hi;
-    stT(sm, sH2T, c, la, lo & 0xffff); stT(sm, sH2T, c + 1, la, lo >> 16);
-    stT(sm, sH2T, c, lb, hi & 0xffff); stT(sm, sH2T, c + 1, lb, hi >> 16);
-  }
-  // ---- layer 3 and the loss
-  float out[2][4];
-#pragma unroll
-  for (int j = 0; j < 2; ++j) {
-    const float2 bb = *reinterpret_cast<const float2*>(Bs + 2 * kHid + 8 * j + 2 * t);
-    out[j][0] = bb.x; out[j][1] = bb.y; out[j][2] = bb.x; out[j][3] = bb.y;
-  }
-#pragma unroll
-  for (int kk = 0; kk < 8; ++kk)
-#pragma unroll
-    for (int j = 0; j < 2; ++j) {
-      const uint32_t* w = reinterpret_cast<const uint32_t*>(W3s + (8 * j + g) * kLd2 + 16 * kk + 2 * t);
-      mma16816(out[j], a[kk], w[0], w[4]);
-    }
-  const float sc = 2.0f / (float)batch;
+  float* bsum = reinterpret_cast<float*>(sm + sBsum) + stripe * (2 * kHid + kOut);
+  float acc[2][4][4];
+  uint32_t G1[2][4][2], G2[2][4][2];
+  // ---- forward
+  bias_tile<2, 4>(Bs, n0, t, acc);
+  tile_mma<2, 4, kIn / 16, false, false, kLd1, kLd1>(sm + sX, sm + kPW1, m0, n0, lane, acc);
+  gelu_tile(acc, G1);
+  put_tile<2, 4, kLd2>(sm + sH1, m0, n0, g, t, acc);
+  stripe_sync(stripe);
+  bias_tile<2, 4>(Bs + kHid, n0, t, acc);
+  tile_mma<2, 4, kHid / 16, false, false, kLd2, kLd2>(sm + sH1, sm + kPW2, m0, n0, lane, acc);
+  gelu_tile(acc, G2);
+  put_tile<2, 4, kLd2>(sm + sH2, m0, n0, g, t, acc);
+  stripe_sync(stripe);
+  // ---- layer 3 and the loss: warps 0 and 1 of the stripe take 16 samples and all 16 outputs each
   float lsum = 0.f;
+  if (wc < 2) {
+    float out[1][2][4];
+    const int mb = m0 + 16 * wc;
+    bias_tile<1, 2>(Bs + 2 * kHid, 0, t, out);
+    tile_mma<1, 2, kHid / 16, false, false, kLd2, kLd2>(sm + sH2, sm + kPW3, mb, 0, lane, out);
+    const float sc = 2.0f / (float)batch;
 #pragma unroll
-  for (int j = 0; j < 2; ++j) {
-    const int c = 8 * j + 2 * t;
-    float2 ta = make_float2(0.f, 0.f), tb = ta;
-    if (va) ta = *reinterpret_cast<const float2*>(T + ra * kOut + c);
-    if (vb) tb = *reinterpret_cast<const float2*>(T + rb * kOut + c);
-    const float r0 = va ? out[j][0] - ta.x : 0.f, r1 = va ? out[j][1] - ta.y : 0.f;
-    const float r2 = vb ? out[j][2] - tb.x : 0.f, r3 = vb ? out[j][3] - tb.y : 0.f;
-    lsum += r0 * r0 + r1 * r1 + r2 * r2 + r3 * r3;
-    out[j][0] = sc * r0; out[j][1] = sc * r1; out[j][2] = sc * r2; out[j][3] = sc * r3;  // dY
-    stT(sm, sDYT, c, la, bf16_bits(out[j][0])); stT(sm, sDYT, c + 1, la, bf16_bits(out[j][1]));
-    stT(sm, sDYT, c, lb, bf16_bits(out[j][2])); stT(sm, sDYT, c + 1, lb, bf16_bits(out[j][3]));
+    for (int q = 0; q < 2; ++q) {
+      const long long r = row[mb + g + 8 * q];
+#pragma unroll
+      for (int n = 0; n < 2; ++n) {
+        const float2 y = r >= 0 ? *reinterpret_cast<const float2*>(T + r * kOut + 8 * n + 2 * t) : make_float2(0.f, 0.f);
+        const float r0 = r >= 0 ? out[0][n][2 * q] - y.x : 0.f, r1 = r >= 0 ? out[0][n][2 * q + 1] - y.y : 0.f;
+        lsum += r0 * r0 + r1 * r1;
+        out[0][n][2 * q] = sc * r0;  // dY
+        out[0][n][2 * q + 1] = sc * r1;
+      }
+    }
+    put_tile<1, 2, kLdY>(sm + sDY, mb, 0, g, t, out);
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) lsum += __shfl_xor_sync(0xffffffffu, lsum, o);
+    // the stripe's column sums of dY: both halves' below, each from its own 16-column slot
+    tile_colsum<1, 2>(out, bsum + (wc ? kHid : 0), lane);
   }
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) lsum += __shfl_xor_sync(0xffffffffu, lsum, o);
   if (lane == 0) reinterpret_cast<float*>(sm + sLoss)[warp] = lsum;
-  warp_colsum<2>(out, bsum + 2 * kHid, lane);
-  // ---- dH2 = dY W3 (one k-step over the 16 outputs), dZ2 = dH2 . G2
-  {
-    uint32_t ay[4] = {pack2(out[0][0], out[0][1]), pack2(out[0][2], out[0][3]), pack2(out[1][0], out[1][1]),
-                      pack2(out[1][2], out[1][3])};
-#pragma unroll
-    for (int j = 0; j < 16; ++j) {
-      acc[j][0] = acc[j][1] = acc[j][2] = acc[j][3] = 0.f;
-      const int col = 8 * j + g;
-      const uint32_t b0 = (uint32_t)W3s[(2 * t) * kLd2 + col] | ((uint32_t)W3s[(2 * t + 1) * kLd2 + col] << 16);
-      const uint32_t b1 =
-          (uint32_t)W3s[(2 * t + 8) * kLd2 + col] | ((uint32_t)W3s[(2 * t + 9) * kLd2 + col] << 16);
-      mma16816(acc[j], ay, b0, b1);
-    }
-  }
-#pragma unroll
-  for (int j = 0; j < 16; ++j)
-#pragma unroll
-    for (int q = 0; q < 4; ++q) acc[j][q] *= bf16_to_f(Gs[(1 * 64 + 4 * j + q) * 32 + lane]);
-  warp_colsum<16>(acc, bsum + kHid, lane);
-#pragma unroll
-  for (int j = 0; j < 16; ++j) {
-    const int c = 8 * j + 2 * t;
-    const uint32_t lo = pack2(acc[j][0], acc[j][1]), hi = pack2(acc[j][2], acc[j][3]);
-    a[j >> 1][(j & 1) * 2 + 0] = lo;
-    a[j >> 1][(j & 1) * 2 + 1] = hi;
-    stT(sm, sDZ2T, c, la, lo & 0xffff); stT(sm, sDZ2T, c + 1, la, lo >> 16);
-    stT(sm, sDZ2T, c, lb, hi & 0xffff); stT(sm, sDZ2T, c + 1, lb, hi >> 16);
-  }
-  // ---- dH1 = dZ2 W2 (B fragments read down the columns of W2), dZ1 = dH1 . G1
-#pragma unroll
-  for (int j = 0; j < 16; ++j) acc[j][0] = acc[j][1] = acc[j][2] = acc[j][3] = 0.f;
-#pragma unroll
-  for (int kk = 0; kk < 8; ++kk)
-#pragma unroll
-    for (int j = 0; j < 16; ++j) {
-      const int col = 8 * j + g, k0 = 16 * kk + 2 * t;
-      const uint32_t b0 = (uint32_t)W2s[k0 * kLd2 + col] | ((uint32_t)W2s[(k0 + 1) * kLd2 + col] << 16);
-      const uint32_t b1 = (uint32_t)W2s[(k0 + 8) * kLd2 + col] | ((uint32_t)W2s[(k0 + 9) * kLd2 + col] << 16);
-      mma16816(acc[j], a[kk], b0, b1);
-    }
-#pragma unroll
-  for (int j = 0; j < 16; ++j)
-#pragma unroll
-    for (int q = 0; q < 4; ++q) acc[j][q] *= bf16_to_f(Gs[(0 * 64 + 4 * j + q) * 32 + lane]);
-  warp_colsum<16>(acc, bsum, lane);
-#pragma unroll
-  for (int j = 0; j < 16; ++j) {
-    const int c = 8 * j + 2 * t;
-    stT(sm, sDZ1T, c, la, bf16_bits(acc[j][0])); stT(sm, sDZ1T, c + 1, la, bf16_bits(acc[j][1]));
-    stT(sm, sDZ1T, c, lb, bf16_bits(acc[j][2])); stT(sm, sDZ1T, c + 1, lb, bf16_bits(acc[j][3]));
-  }
+  stripe_sync(stripe);
+  if (wc == 0 && lane < kOut) bsum[2 * kHid + lane] = bsum[lane] + bsum[kHid + lane];
+  stripe_sync(stripe);
+  // ---- dH2 = dY W3, dZ2 = dH2 . gelu'(Z2)
+  zero_tile<2, 4>(acc);
+  tile_mma<2, 4, 1, false, true, kLdY, kLd2>(sm + sDY, sm + kPW3, m0, n0, lane, acc);
+  scale_tile(acc, G2);
+  tile_colsum<2, 4>(acc, bsum + kHid + n0, lane);
+  put_tile<2, 4, kLd2>(sm + sDZ2, m0, n0, g, t, acc);
+  stripe_sync(stripe);
+  // ---- dH1 = dZ2 W2, dZ1 = dH1 . gelu'(Z1)
+  zero_tile<2, 4>(acc);
+  tile_mma<2, 4, kHid / 16, false, true, kLd2, kLd2>(sm + sDZ2, sm + kPW2, m0, n0, lane, acc);
+  scale_tile(acc, G1);
+  tile_colsum<2, 4>(acc, bsum + n0, lane);
+  __syncthreads();  // every stripe is through with W2
+  put_tile<2, 4, kLd2>(sm + sDZ1, m0, n0, g, t, acc);
   __syncthreads();
   // ---- weight gradients of this CTA: dW1 = dZ1^T X, dW2 = dZ2^T H1, dW3 = dY^T H2
   float* P = part + (size_t)blockIdx.x * kPartLd;
-#pragma unroll 1
-  for (int mb = 2 * warp; mb < 2 * warp + 2; ++mb) {
-    wgrad_block<14>(sm, sDZ1T, 16 * mb, sXT, 0, g, t, P + oW1, kIn);
-    wgrad_block<16>(sm, sDZ2T, 16 * mb, sH1T, 0, g, t, P + oW2, kHid);
+  zero_tile<2, 4>(acc);
+  tile_mma<2, 4, kTRows / 16, true, true, kLd2, kLd2>(sm + sDZ2, sm + sH1, m0, n0, lane, acc);
+  put_grad<2, 4>(P + oW2, kHid, m0, n0, g, t, acc);
+  zero_tile<2, 4>(acc);
+  static_assert(kIn == 3 * 32 + 16, "three warps with 32 columns of dW1 and one with 16");
+  if (wc < 3) {
+    tile_mma<2, 4, kTRows / 16, true, true, kLd2, kLd1>(sm + sDZ1, sm + sX, m0, n0, lane, acc);
+    put_grad<2, 4>(P + oW1, kIn, m0, n0, g, t, acc);
+  } else {
+    float last[2][2][4], w3[1][4][4];
+    zero_tile<2, 2>(last);
+    tile_mma<2, 2, kTRows / 16, true, true, kLd2, kLd1>(sm + sDZ1, sm + sX, m0, n0, lane, last);
+    put_grad<2, 2>(P + oW1, kIn, m0, n0, g, t, last);
+    zero_tile<1, 4>(w3);
+    tile_mma<1, 4, kTRows / 16, true, true, kLdY, kLd2>(sm + sDY, sm + sH2, 0, m0, lane, w3);
+    put_grad<1, 4>(P + oW3, kHid, 0, m0, g, t, w3);
   }
-  wgrad_block<4>(sm, sDYT, 0, sH2T, 4 * warp, g, t, P + oW3, kHid);
-  // bias gradients and the loss: sums over the warps in a fixed order
+  // bias gradients and the loss: sums over the stripes or warps in a fixed order
   const float* bs = reinterpret_cast<const float*>(sm + sBsum);
   for (int i = threadIdx.x; i < 2 * kHid + kOut; i += blockDim.x) {
     float s = 0.f;
-    for (int w = 0; w < kWarps; ++w) s += bs[w * (2 * kHid + kOut) + i];
+    for (int w = 0; w < kStripes; ++w) s += bs[w * (2 * kHid + kOut) + i];
     const int dst = i < kHid ? ob1 + i : i < 2 * kHid ? ob2 + (i - kHid) : ob3 + (i - 2 * kHid);
     P[dst] = s;
   }
   if (threadIdx.x == 0) {
     const float* ls = reinterpret_cast<const float*>(sm + sLoss);
     float s = 0.f;
-    for (int w = 0; w < kWarps; ++w) s += ls[w];
+    for (int w = 0; w < kTWarps; ++w) s += ls[w];
     P[kNP] = s;
   }
 }
 
-// grad[p] = sum_c part[c][p]; loss = sum_c part[c][kNP] / batch (fixed order)
-__global__ void grad_reduce_kernel(const float* __restrict__ part, int nparts, int batch, float* __restrict__ grad,
-                                   float* __restrict__ loss) {
-  const int p = blockIdx.x * blockDim.x + threadIdx.x;
+// grad[p] = sum_c part[c][p]; loss = sum_c part[c][kNP] / batch (fixed order). Bound by the
+// latency of its loads: 16 bytes of four consecutive entries per thread, eight threads per
+// group with every eighth partial row each, their sums joined in shared memory. One thread
+// per entry over all rows: 8.2 us for 16384 samples (256 rows), now 3.5 us (128 rows).
+constexpr int kRedCols = 32, kRedRows = 8;
+__global__ void __launch_bounds__(kRedCols* kRedRows) grad_reduce_kernel(const float* __restrict__ part, int nparts,
+                                                                         int batch, float* __restrict__ grad,
+                                                                         float* __restrict__ loss) {
+  __shared__ float4 sum[kRedRows][kRedCols];
+  const int x = threadIdx.x % kRedCols, y = threadIdx.x / kRedCols;
+  const int q = blockIdx.x * kRedCols + x;  // group of four entries
+  float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
+  if (4 * q <= kNP) {
+    const float4* p = reinterpret_cast<const float4*>(part) + q;
+#pragma unroll 8
+    for (int c = y; c < nparts; c += kRedRows) {
+      const float4 v = p[(size_t)c * (kPartLd / 4)];
+      s.x += v.x; s.y += v.y; s.z += v.z; s.w += v.w;
+    }
+  }
+  sum[y][x] = s;
+  __syncthreads();
+  if (threadIdx.x >= 4 * kRedCols) return;
+  const int p = 4 * blockIdx.x * kRedCols + threadIdx.x;
   if (p > kNP) return;
-  float s = 0.f;
-  for (int c = 0; c < nparts; ++c) s += part[(size_t)c * kPartLd + p];
-  if (p < kNP) grad[p] = s;
-  else if (loss) *loss = s / (float)batch;
+  float r = 0.f;
+#pragma unroll
+  for (int i = 0; i < kRedRows; ++i) r += reinterpret_cast<const float*>(sum[i])[threadIdx.x];
+  if (p < kNP) grad[p] = r;
+  else if (loss) *loss = r / (float)batch;
 }
 
 __global__ void adam_kernel(float* __restrict__ theta, const float* __restrict__ grad, float* __restrict__ m,
@@ -659,7 +701,7 @@ int smem_opt_in(K kernel, int bytes) {
   return 0;
 }
 
-long long grad_parts(long long batch) { return (batch + kRows - 1) / kRows; }
+long long grad_parts(long long batch) { return (batch + kTRows - 1) / kTRows; }
 
 bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 
@@ -751,9 +793,9 @@ int dg_mlp_grad(const float* theta, const float* X, const float* T, long long np
   if (smem_opt_in(mlp_grad_kernel, kTrainSmem))
     return fail(nullptr, DG_ERR_CUDA, "cannot opt in to the shared memory of the training kernel");
   const int nparts = (int)grad_parts(batch);
-  mlp_grad_kernel<<<nparts, 32 * kWarps, kTrainSmem, st>>>(net, X, T, npairs, batch, seed, step, part, status);
+  mlp_grad_kernel<<<nparts, 32 * kTWarps, kTrainSmem, st>>>(net, X, T, npairs, batch, seed, step, part, status);
   MLP_CUDA(cudaGetLastError());
-  grad_reduce_kernel<<<(kNP + 1 + 255) / 256, 256, 0, st>>>(part, nparts, batch, grad, loss);
+  grad_reduce_kernel<<<(kNP + 4 * kRedCols) / (4 * kRedCols), kRedCols * kRedRows, 0, st>>>(part, nparts, batch, grad, loss);
   MLP_CUDA(cudaGetLastError());
   return DG_OK;
 }
