@@ -720,72 +720,12 @@ __global__ void __launch_bounds__(NT) pair_jacobi_kernel(int ne, int ns, const S
   }
 }
 
-// The same row products read straight from global memory: one thread per output row, `epc`
-// elements per CTA (b rows each), the input vectors in shared memory. Loads of one warp cover
-// 32 consecutive rows of a column (coalesced); eight independent accumulators keep eight loads
-// in flight per thread, and small CTAs keep many elements in flight per SM. (One thread per
-// pair of rows with paired loads halves the threads and was slower: 61 against 45 us at P2.)
-template <class R, int NBLK, class S>
-__global__ void __launch_bounds__(256) direct_apply_kernel(int ne, int b, int epc, const S* __restrict__ A,
-                                                           const int* __restrict__ nbr, const R* __restrict__ v,
-                                                           const R* __restrict__ w, R alpha, R beta, int x_zero,
-                                                           R* __restrict__ y) {
-  extern __shared__ __align__(16) unsigned char sraw_[];
-  R* rv = reinterpret_cast<R*>(sraw_);  // [epc][ncol]
-  const int ncol = NBLK * b;
-  const int tid = threadIdx.x, nt = blockDim.x;
-  for (int e0 = blockIdx.x * epc; e0 < ne; e0 += gridDim.x * epc) {
-    const int cnt = min(epc, ne - e0);
-    for (int t = tid; t < cnt * ncol; t += nt) {
-      const int el = t / ncol, q = t - el * ncol;
-      const int e = e0 + el;
-      const int s = q / b, c = q - s * b;
-      if (NBLK == 1) {
-        rv[t] = v[(size_t)e * b + c] - (w ? w[(size_t)e * b + c] : R(0));
-      } else {
-        const int src = s == 0 ? e : nbr[(size_t)e * 6 + s - 1];
-        rv[t] = src >= 0 ? v[(size_t)src * b + c] : R(0);  // no neighbour across a wall (zero block)
-      }
-    }
-    __syncthreads();
-    if (tid < cnt * b) {
-      const int el = tid / b, i = tid - el * b;
-      const S* Ae = A + (size_t)(e0 + el) * ncol * b + i;
-      const R* re = rv + (size_t)el * ncol;
-      R a[8];
-#pragma unroll
-      for (int u = 0; u < 8; ++u) a[u] = R(0);
-      int q = 0;
-      for (; q + 7 < ncol; q += 8) {
-#pragma unroll
-        for (int u = 0; u < 8; ++u) a[u] = fma(wide<R>(__ldg(Ae + (size_t)(q + u) * b)), re[q + u], a[u]);
-      }
-      for (; q < ncol; ++q) a[0] = fma(wide<R>(__ldg(Ae + (size_t)q * b)), re[q], a[0]);
-      const R acc = ((a[0] + a[1]) + (a[2] + a[3])) + ((a[4] + a[5]) + (a[6] + a[7]));
-      R* ye = y + (size_t)(e0 + el) * b + i;
-      if (NBLK == 1) *ye = (x_zero ? R(0) : *ye) + alpha * acc;
-      else *ye = alpha * acc + (beta == R(0) ? R(0) : beta * *ye);
-    }
-    __syncthreads();
-  }
+// Sixteen bytes of stored entries widened to the accumulator's type.
+__device__ __forceinline__ void widen16(const uint4& raw, const double*, double (&o)[2]) {
+  memcpy(o, &raw, 16);
 }
-
-template <class R, int NBLK, class S>
-int launch_direct(Handle* h, int b, const S* A, const R* v, const R* w, R alpha, R beta, int x_zero, R* y,
-                  cudaStream_t st) {
-  if (b > 256) return -1;  // -1, not a DG_ code: the caller falls back to bsr_kernel
-  const int epc = std::max(1, 256 / b);
-  const int threads = 32 * ((epc * b + 31) / 32);
-  const size_t smem = sizeof(R) * (size_t)epc * NBLK * b;
-  const int grid = (h->ne + epc - 1) / epc;
-  direct_apply_kernel<R, NBLK, S><<<grid, threads, smem, st>>>(h->ne, b, epc, A, h->nbr, v, w, alpha, beta, x_zero,
-                                                               y);
-  DG_LAUNCH_CHECK(h);
-  return DG_OK;
-}
-
-// Eight 16-bit entries (one 16-byte vector) widened to float.
-__device__ __forceinline__ void wide8(const uint4& raw, const __half*, float* o) {
+__device__ __forceinline__ void widen16(const uint4& raw, const float*, float (&o)[4]) { memcpy(o, &raw, 16); }
+__device__ __forceinline__ void widen16(const uint4& raw, const __half*, float (&o)[8]) {
   const __half2* h2 = reinterpret_cast<const __half2*>(&raw);
 #pragma unroll
   for (int j = 0; j < 4; ++j) {
@@ -794,7 +734,7 @@ __device__ __forceinline__ void wide8(const uint4& raw, const __half*, float* o)
     o[2 * j + 1] = f.y;
   }
 }
-__device__ __forceinline__ void wide8(const uint4& raw, const __nv_bfloat16*, float* o) {
+__device__ __forceinline__ void widen16(const uint4& raw, const __nv_bfloat16*, float (&o)[8]) {
   const __nv_bfloat162* h2 = reinterpret_cast<const __nv_bfloat162*>(&raw);
 #pragma unroll
   for (int j = 0; j < 4; ++j) {
@@ -804,74 +744,89 @@ __device__ __forceinline__ void wide8(const uint4& raw, const __nv_bfloat16*, fl
   }
 }
 
-// y = alpha A x + beta y over rows of 7 blocks stored in 16 bits (b a multiple of 8), FP32
-// accumulation. A task is eight consecutive rows of one block: per block column it loads one
-// 16-byte vector, so a warp's load moves 512 bytes and a thread keeps eight loads (128 bytes)
-// in flight. The seven block partial sums of a row meet in shared memory and are added in
-// block order.
-template <class S>
-__global__ void __launch_bounds__(256) direct7_vec_kernel(int ne, int b, int epc, const S* __restrict__ A,
-                                                          const int* __restrict__ nbr, const float* __restrict__ v,
-                                                          float alpha, float beta, float* __restrict__ y) {
+// y = alpha A x + beta y over rows of 7 blocks (b a multiple of 8) stored as S, accumulated as R.
+// Bound by the blocks' bytes in 16 and 32 bits and by the FP64 pipe in 64 bits (7 b^2 FMA per
+// element, 78 us at 16^3 with b = 40). A task is 16 bytes of rows of one block: per block column it
+// loads one vector, kColsAhead columns ahead of their use, and the first ones before the slices of
+// x are there, so that each warp keeps up to 2 kColsAhead of its 512-byte loads in flight. The seven
+// partial sums of a row meet in shared memory and are added in block order.
+// Before, FP64 and FP32 rows had one thread per row over all 7 b columns, which left too few loads
+// in flight (b = 40, FP64 at 12^3: 60 us, now 46; at 16^3: 116, now 93; FP32 at 12^3: 29, now 16), and
+// the 16-bit rows waited for x before their first load (16^3: 28 us, now 24; 32^3: 149, now 137). Four
+// CTAs per SM in 16 bits: at 16^3 three leave an eighth of the CTAs to a second wave (29 us).
+constexpr int kColsAhead = 4, kRowThreads = 288;
+
+template <class R, class S>
+__global__ void __launch_bounds__(kRowThreads, sizeof(S) == 2 ? 4 : 3) block_row_kernel(int ne, int b, int epc, const S* __restrict__ A,
+                                                                const int* __restrict__ nbr, const R* __restrict__ v,
+                                                                R alpha, R beta, R* __restrict__ y) {
+  constexpr int VW = 16 / sizeof(S), U = kColsAhead;  // rows of a task, columns loaded at a time (b % U == 0)
   extern __shared__ __align__(16) unsigned char sraw_[];
-  const int ncol = 7 * b, rg = b / 8, tpe = 7 * rg;
-  float* rv = reinterpret_cast<float*>(sraw_);  // [epc][ncol] the seven slices of v
-  float* part = rv + (size_t)epc * ncol;       // [epc][7][b] block partial sums
-  const int tid = threadIdx.x, nt = blockDim.x;
-  for (int e0 = blockIdx.x * epc; e0 < ne; e0 += gridDim.x * epc) {
-    const int cnt = min(epc, ne - e0);
-    for (int t = tid; t < cnt * ncol; t += nt) {
-      const int el = t / ncol, q = t - el * ncol;
-      const int e = e0 + el;
-      const int sb = q / b, c = q - sb * b;
-      const int src = sb == 0 ? e : nbr[(size_t)e * 6 + sb - 1];
-      rv[t] = src >= 0 ? v[(size_t)src * b + c] : 0.0f;  // no neighbour across a wall (zero block)
-    }
-    __syncthreads();
-    if (tid < cnt * tpe) {
-      const int el = tid / tpe, r = tid - el * tpe, sb = r / rg, r8 = r - sb * rg;
-      const S* As = A + (size_t)(e0 + el) * ncol * b + (size_t)sb * b * b + 8 * r8;
-      const float* re = rv + (size_t)el * ncol + sb * b;
-      float acc[8];
+  const int ncol = 7 * b, rg = b / VW, tpe = 7 * rg;
+  R* rv = reinterpret_cast<R*>(sraw_);    // [epc][ncol] the seven slices of v
+  R* part = rv + (size_t)epc * ncol;      // [epc][7][b] block partial sums
+  const int tid = threadIdx.x, nt = blockDim.x, e0 = blockIdx.x * epc, cnt = min(epc, ne - e0);
+  const int el = tid / tpe, r = tid - el * tpe, sb = r / rg, row = VW * (r - sb * rg);
+  const bool on = el < cnt;
+  const S* As = A + ((size_t)(e0 + (on ? el : 0)) * 7 + sb) * b * b + row;
+  uint4 cur[U], nxt[U];
 #pragma unroll
-      for (int u = 0; u < 8; ++u) acc[u] = 0.0f;
-#pragma unroll 8
-      for (int c = 0; c < b; ++c) {
-        const uint4 raw = __ldg(reinterpret_cast<const uint4*>(As + (size_t)c * b));
-        float a8[8];
-        wide8(raw, As, a8);
-        const float xc = re[c];
+  for (int u = 0; u < U; ++u)
+    if (on) cur[u] = __ldg(reinterpret_cast<const uint4*>(As + (size_t)u * b));
+  for (int t = tid; t < cnt * ncol; t += nt) {
+    const int et = t / ncol, q = t - et * ncol;
+    const int e = e0 + et;
+    const int st = q / b, c = q - st * b;
+    const int src = st == 0 ? e : nbr[(size_t)e * 6 + st - 1];
+    rv[t] = src >= 0 ? v[(size_t)src * b + c] : R(0);  // no neighbour across a wall (zero block)
+  }
+  __syncthreads();
+  if (on) {
+    const R* re = rv + (size_t)el * ncol + sb * b;
+    R acc[VW];
 #pragma unroll
-        for (int u = 0; u < 8; ++u) acc[u] = fmaf(a8[u], xc, acc[u]);
+    for (int j = 0; j < VW; ++j) acc[j] = R(0);
+    for (int c = 0; c < b; c += U) {
+      if (c + U < b) {
+#pragma unroll
+        for (int u = 0; u < U; ++u) nxt[u] = __ldg(reinterpret_cast<const uint4*>(As + (size_t)(c + U + u) * b));
       }
-      float* ps = part + ((size_t)el * 7 + sb) * b + 8 * r8;
 #pragma unroll
-      for (int u = 0; u < 8; ++u) ps[u] = acc[u];
-    }
-    __syncthreads();
-    for (int t = tid; t < cnt * b; t += nt) {
-      const int el = t / b, i = t - el * b;
-      const float* pe = part + (size_t)el * 7 * b + i;
-      float acc = pe[0];
+      for (int u = 0; u < U; ++u) {
+        R a[VW];
+        widen16(cur[u], As, a);
+        const R xc = re[c + u];
 #pragma unroll
-      for (int sb = 1; sb < 7; ++sb) acc += pe[sb * b];
-      float* ye = y + (size_t)(e0 + el) * b + i;
-      *ye = alpha * acc + (beta == 0.0f ? 0.0f : beta * *ye);
+        for (int j = 0; j < VW; ++j) acc[j] = fma(a[j], xc, acc[j]);
+      }
+#pragma unroll
+      for (int u = 0; u < U; ++u) cur[u] = nxt[u];
     }
-    __syncthreads();
+    R* ps = part + ((size_t)el * 7 + sb) * b + row;
+#pragma unroll
+    for (int j = 0; j < VW; ++j) ps[j] = acc[j];
+  }
+  __syncthreads();
+  for (int t = tid; t < cnt * b; t += nt) {
+    const int et = t / b, i = t - et * b;
+    const R* pe = part + (size_t)et * 7 * b + i;
+    R acc = pe[0];
+#pragma unroll
+    for (int st = 1; st < 7; ++st) acc += pe[st * b];
+    R* ye = y + (size_t)(e0 + et) * b + i;
+    *ye = alpha * acc + (beta == R(0) ? R(0) : beta * *ye);
   }
 }
 
-template <class S>
-int launch_direct7_vec(Handle* h, int b, const S* A, const float* v, float alpha, float beta, float* y,
-                       cudaStream_t st) {
-  const int tpe = 7 * (b / 8);
-  if (b % 8 != 0 || tpe > 256) return -1;  // -1: unsuited; the caller reports it
-  const int epc = std::max(1, 256 / tpe);
+template <class R, class S>
+int launch_block_rows(Handle* h, int b, const S* A, const R* v, R alpha, R beta, R* y, cudaStream_t st) {
+  const int tpe = 7 * (b / (16 / (int)sizeof(S)));
+  if (b % 8 != 0 || tpe > kRowThreads) return -1;  // -1, not a DG_ code: unsuited, the caller's general path
+  const int epc = kRowThreads / tpe;
   const int threads = 32 * ((epc * tpe + 31) / 32);
-  const size_t smem = sizeof(float) * (size_t)epc * 14 * b;  // slices of v and partial sums
+  const size_t smem = sizeof(R) * (size_t)epc * 14 * b;  // slices of v and partial sums
   const int grid = (h->ne + epc - 1) / epc;
-  direct7_vec_kernel<S><<<grid, threads, smem, st>>>(h->ne, b, epc, A, h->nbr, v, alpha, beta, y);
+  block_row_kernel<R, S><<<grid, threads, smem, st>>>(h->ne, b, epc, A, h->nbr, v, alpha, beta, y);
   DG_LAUNCH_CHECK(h);
   return DG_OK;
 }
@@ -1007,7 +962,7 @@ int staged_bsr(Handle* h, int lvl, const R* B, R alpha, const R* x, R beta, R* y
   cudaEvent_t e0 = nullptr;
   int rc;
   if (lvl == 1 && (rc = prof_begin(h, st, &e0))) return rc;
-  rc = launch_direct<R, 7, R>(h, b, B, x, nullptr, alpha, beta, 0, y, st);
+  rc = launch_block_rows<R, R>(h, b, B, x, alpha, beta, y, st);
   if (rc) return rc;
   // algorithmic bytes: the 7 blocks of every row, x and the old y read once, y written once
   const double vec = (double)h->ne * b * sizeof(R);
@@ -1022,18 +977,11 @@ int bsr16_f(Handle* h, int lvl, int storage, float alpha, const float* x, float 
   cudaEvent_t e0 = nullptr;
   int rc;
   if (lvl == 1 && (rc = prof_begin(h, st, &e0))) return rc;
-  if (L.b % 8 == 0) {  // 16-byte vectors of eight rows
-    if (storage == DG_PRECOND_FP32_H16)
-      rc = launch_direct7_vec<__half>(h, L.b, static_cast<const __half*>(L.Bsr16), x, alpha, beta, y, st);
-    else
-      rc = launch_direct7_vec<__nv_bfloat16>(h, L.b, static_cast<const __nv_bfloat16*>(L.Bsr16), x, alpha, beta, y,
-                                             st);
-  } else if (storage == DG_PRECOND_FP32_H16) {
-    rc = launch_direct<float, 7, __half>(h, L.b, static_cast<const __half*>(L.Bsr16), x, nullptr, alpha, beta, 0, y, st);
-  } else {
-    rc = launch_direct<float, 7, __nv_bfloat16>(h, L.b, static_cast<const __nv_bfloat16*>(L.Bsr16), x, nullptr, alpha,
-                                                beta, 0, y, st);
-  }
+  if (storage == DG_PRECOND_FP32_H16)
+    rc = launch_block_rows<float, __half>(h, L.b, static_cast<const __half*>(L.Bsr16), x, alpha, beta, y, st);
+  else
+    rc = launch_block_rows<float, __nv_bfloat16>(h, L.b, static_cast<const __nv_bfloat16*>(L.Bsr16), x, alpha, beta, y,
+                                                 st);
   if (rc) return rc;
   const double vec = (double)h->ne * L.b * sizeof(float);
   const double bytes = 7.0 * h->ne * L.b * L.b * 2 + vec * (2 + (beta != 0.0f ? 1 : 0));
