@@ -81,13 +81,15 @@ int launch_axpby(Handle* h, long long n, double a, const double* x, double b, do
 }
 
 // ------------------------------------------------------ transfer operators
+// xc = I (xf - yf), or I xf without yf: only the coarse modes of the difference are formed (as a
+// difference over the whole level and a restriction it took two launches)
 template <class R>
-__global__ void restrict_kernel(int ne, int nbf, int nbc, const R* xf, R* xc) {
+__global__ void restrict_kernel(int ne, int nbf, int nbc, const R* xf, const R* yf, R* xc) {
   const long long n = (long long)ne * 4 * nbc;
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
     const long long ev = i / nbc;
     const int m = (int)(i - ev * nbc);
-    xc[i] = xf[ev * nbf + m];
+    xc[i] = xf[ev * nbf + m] - (yf ? yf[ev * nbf + m] : R(0));
   }
 }
 template <class R>
@@ -166,13 +168,14 @@ __global__ void __launch_bounds__(128) bsr_t_kernel(int ne, int b, const int* nb
 // rows still to be updated fill the fewest slots of 32 (385 warp FMAs per pass at B = 140, of
 // 304 in full lanes). Columns are loaded kLuAhead at a time, one group ahead of their use: the
 // first version (vector in shared memory, no load ahead) waited on memory at every one of its 2B
-// dependent steps and took 0.495 ms at 16^3 P4 (642 MB of factors).
+// dependent steps and took 0.495 ms at 16^3 P4 (642 MB of factors); now 0.20 ms (0.22 with the column
+// stride at run time). Loading 8 or 16 columns ahead is no faster, at B = 40 and B = 80 either.
 constexpr int kApplyWarps = 4;
 constexpr int kLuAhead = 4;
 
 // kLuAhead columns j0, j0 + step, ... of slots 0..M of this lane's rows (row(s) in [0, B), or not loaded)
-template <int M, class Row>
-__device__ __forceinline__ void lu_load(double (&A)[kLuAhead][M + 1], const double* L, int B, int j0, int step, int j1,
+template <int B, int M, class Row>
+__device__ __forceinline__ void lu_load(double (&A)[kLuAhead][M + 1], const double* L, int j0, int step, int j1,
                                         Row row) {
 #pragma unroll
   for (int u = 0; u < kLuAhead; ++u) {
@@ -200,9 +203,9 @@ __device__ __forceinline__ void lu_substitute(double (&z)[SL], const double* L, 
     return q < qj ? (FWD ? B - 1 - q : q) : -1;
   };
   double A[kLuAhead][M + 1], N[kLuAhead][M + 1];
-  lu_load<M>(A, L, B, jf, step, je, row);
+  lu_load<B, M>(A, L, jf, step, je, row);
   for (int j = jf; FWD ? j < je : j > je; j += kLuAhead * step) {
-    lu_load<M>(N, L, B, j + kLuAhead * step, step, je, row);
+    lu_load<B, M>(N, L, j + kLuAhead * step, step, je, row);
 #pragma unroll
     for (int u = 0; u < kLuAhead; ++u) {
       const int ju = j + u * step, q = (FWD ? B - 1 - ju : ju) - 32 * M;
@@ -449,9 +452,9 @@ static int smooth(Handle* h, int lvl, const double* g, double* x, int iters, dou
   return jacobi_sweeps(h, lvl, g, x, iters, omega, x_zero, st);
 }
 
-static int restrict_to(Handle* h, int lvl, const double* xf, double* xc, cudaStream_t st) {
+static int restrict_to(Handle* h, int lvl, const double* xf, const double* yf, double* xc, cudaStream_t st) {
   const Level &F = h->lev[lvl], &C = h->lev[lvl + 1];
-  restrict_kernel<double><<<grid_for(h, C.n / 64 + 1), 256, 0, st>>>(h->ne, F.nb, C.nb, xf, xc);
+  restrict_kernel<double><<<grid_for(h, C.n / 64 + 1), 256, 0, st>>>(h->ne, F.nb, C.nb, xf, yf, xc);
   DG_LAUNCH_CHECK(h);
   return DG_OK;
 }
@@ -552,12 +555,10 @@ static int mg_v(Handle* h, int l, const double* g, double* x, bool x_zero, const
   Level& C = h->lev[l + 1];
   const bool xz = x_zero && o.pre_sweeps == 0;
   if (xz) {
-    if ((rc = restrict_to(h, l, g, C.t0, st))) return rc;
+    if ((rc = restrict_to(h, l, g, nullptr, C.t0, st))) return rc;
   } else {
     if ((rc = level_matvec(h, l, x, L.t2, st))) return rc;
-    axpby_kernel<double><<<grid_for(h, L.n / 256 + 1), 256, 0, st>>>(L.n, 1.0, g, -1.0, L.t2);  // t2 = g - G x
-    DG_LAUNCH_CHECK(h);
-    if ((rc = restrict_to(h, l, L.t2, C.t0, st))) return rc;
+    if ((rc = restrict_to(h, l, g, L.t2, C.t0, st))) return rc;  // I (g - G x)
   }
   if ((rc = mg_v(h, l + 1, C.t0, C.t1, true, o, st))) return rc;
   if (xz) DG_CUDA(h, cudaMemsetAsync(x, 0, sizeof(double) * L.n, st));
@@ -573,7 +574,7 @@ static int mg_full(Handle* h, int l, const double* g, double* x, const dg_solve_
   Level& L = h->lev[l];
   Level& C = h->lev[l + 1];
   // g_{l+1} = I g_l; w_{l+1} = MG_full(l+1, g_{l+1}); keep them in the coarse level's t0/t1
-  if ((rc = restrict_to(h, l, g, C.t0, st))) return rc;
+  if ((rc = restrict_to(h, l, g, nullptr, C.t0, st))) return rc;
   if ((rc = mg_full(h, l + 1, C.t0, C.t1, o, st))) return rc;
   DG_CUDA(h, cudaMemsetAsync(x, 0, sizeof(double) * L.n, st));
   if ((rc = prolong_add(h, l, C.t1, x, st))) return rc;  // w_hat_l = I w_{l+1}
@@ -715,13 +716,11 @@ static int mg_v_f(Handle* h, int l, const float* g, float* x, bool x_zero, const
   Level& C = h->lev[l + 1];
   const bool xz = x_zero && o.pre_sweeps == 0;
   if (xz) {
-    restrict_kernel<float><<<grid_for(h, C.n / 64 + 1), 256, 0, st>>>(h->ne, L.nb, C.nb, g, C.t0f);
+    restrict_kernel<float><<<grid_for(h, C.n / 64 + 1), 256, 0, st>>>(h->ne, L.nb, C.nb, g, nullptr, C.t0f);
     DG_LAUNCH_CHECK(h);
   } else {
     if ((rc = level_matvec_f(h, l, x, L.t2f, o.precision, st))) return rc;
-    axpby_kernel<float><<<grid_for(h, L.n / 256 + 1), 256, 0, st>>>(L.n, 1.0f, g, -1.0f, L.t2f);
-    DG_LAUNCH_CHECK(h);
-    restrict_kernel<float><<<grid_for(h, C.n / 64 + 1), 256, 0, st>>>(h->ne, L.nb, C.nb, L.t2f, C.t0f);
+    restrict_kernel<float><<<grid_for(h, C.n / 64 + 1), 256, 0, st>>>(h->ne, L.nb, C.nb, g, L.t2f, C.t0f);
     DG_LAUNCH_CHECK(h);
   }
   if ((rc = mg_v_f(h, l + 1, C.t0f, C.t1f, true, o, st))) return rc;
@@ -994,7 +993,7 @@ int pmg_restrict(dg_handle* hh, int lvl, const double* xf, double* xc, void* str
   Handle* h = reinterpret_cast<Handle*>(hh);
   if (!h) return DG_ERR_ARG;
   if (lvl < 0 || lvl + 1 >= h->nlev || !xf || !xc) return fail(h, DG_ERR_ARG, "bad level or pointer");
-  return restrict_to(h, lvl, xf, xc, as_stream(stream));
+  return restrict_to(h, lvl, xf, nullptr, xc, as_stream(stream));
 }
 
 int pmg_prolong(dg_handle* hh, int lvl, const double* xc, double* xf, void* stream) {
