@@ -181,8 +181,8 @@ struct Handle {
   int kry_m = 0;
   double* V = nullptr;  // [(m+1)][n0]
   double* Z = nullptr;  // [m][n0]
-  double* hcol = nullptr;     // device [m+2]
-  double* hcol_host = nullptr;  // pinned [m+2]
+  double* hcol = nullptr;       // device [2 m + 8]: an iteration's Gram-Schmidt coefficients and |w|^2
+  double* hcol_host = nullptr;  // pinned, the same
   // GMRES smoother workspace: per-level Krylov basis and small device arrays
   double* smV[DG_MAX_LEVELS] = {nullptr, nullptr, nullptr, nullptr};  // [(its+1)][n_l]
   int smV_its[DG_MAX_LEVELS] = {0, 0, 0, 0};
