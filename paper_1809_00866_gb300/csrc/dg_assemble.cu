@@ -16,7 +16,9 @@
 #include <algorithm>
 #include <vector>
 
+#include "dg_async.h"
 #include "dg_internal.h"
+#include "dg_pencil.h"
 
 namespace dg {
 
@@ -33,37 +35,86 @@ namespace dg {
 //    E_ij = sum_q w2_q dF_i/ds_j(q) B2[q][n2] B2[q][n2'].
 // Diagonal blocks use the own side's columns of the Jacobian; the level-1 off-diagonal
 // blocks the other side's, restricted to the coarse modes.
+//
+// Bound: the bytes of the blocks and of the linear part (240 KB per element at k = 4 over k = 2 in
+// FP32), if the instructions stay few. So
+//  * E and U come from the same step, plane by plane: a plane of point values against the products
+//    of 1D polynomials along its first axis, then along the second, in registers, the pair of 1D
+//    exponents fixed at compile time (975 FMA per 15 x 15 matrix instead of 3000);
+//  * the two faces of an axis are added before that step: P_hat_a(-1) P_hat_a'(-1) = (-1)^(a+a')
+//    P_hat_a(1) P_hat_a'(1), so the faces' difference serves the mode pairs with a + a' even and
+//    their sum those with a + a' odd;
+//  * the flux Jacobian's zeros are left out: (i, j) couples through axis d only if j is the pressure
+//    or d, or if i = j, which leaves 10 of 16 pairs;
+//  * one column variable j at a time, so that the matrices take little shared memory (57 KB in FP32 at
+//    k = 4) and several elements per SM hide each other's phases; a thread of the output phase
+//    keeps one row and loads the linear part kAsmAhead columns at a time.
+//  * the next element's Jacobian records and velocity arrive by asynchronous copies while the last column
+//    of this one is written, and the linear part is brought to L2 one column variable ahead.
+// With every E by direct quadrature and six face terms per entry, FP64 at 12^3 P3 took 1.59 ms, now
+// 0.5; FP32 at 24 x 12 x 12 P3 0.61 ms, now 0.37; at 32^3 P4 12.2 ms, now 5.1.
+template <int K>
+struct PairProducts {
+  double v[(K + 1) * (K + 2) / 2][K + 1];
+};
+// P_hat_a1 P_hat_a2 at the Gauss nodes (ascending), pairs a1 <= a2 at tri(a2) + a1
+template <int K>
+constexpr PairProducts<K> make_pair_products() {
+  PairProducts<K> t{};
+  for (int a2 = 0; a2 <= K; ++a2)
+    for (int a1 = 0; a1 <= a2; ++a1)
+      for (int q = 0; q <= K; ++q) {
+        const double x = 2 * q < K ? -gauss_x(K + 1, q) : gauss_x(K + 1, K - q);
+        t.v[tri(a2) + a1][q] = leg_scale(a1) * legendre(a1, x) * leg_scale(a2) * legendre(a2, x);
+      }
+  return t;
+}
+template <class R, int K>
+struct PairTab {
+  R v[(K + 1) * (K + 2) / 2][K + 1];
+};
+template <class R, int K>
+constexpr PairTab<R, K> make_pair_tab() {
+  constexpr PairProducts<K> p = make_pair_products<K>();
+  PairTab<R, K> t{};
+  for (int j = 0; j < (K + 1) * (K + 2) / 2; ++j)
+    for (int q = 0; q <= K; ++q) t.v[j][q] = R(p.v[j][q]);
+  return t;
+}
+template <class R, int K>
+__constant__ PairTab<R, K> pair_tab = make_pair_tab<R, K>();
+
 template <int K, class R = double>
 struct AsmSmem {
-  static constexpr int NB = nb_of(K), N1 = K + 1, NQ = N1 * N1 * N1, NQF = N1 * N1, N2 = (K + 1) * (K + 2) / 2;
-  static constexpr int N2C = K * (K + 1) / 2;   // 2D modes of a coarser level (degree <= K - 1)
-  static constexpr int B = 0;                   // [NQ][NB]
-  static constexpr int UB = B + NQ * NB;        // [3][NQ] w_q ubar_c(q)
-  static constexpr int U = UB + 3 * NQ;         // [3][NB][NB]
-  static constexpr int E = U + 3 * NB * NB;     // [4 j][6 slot][N2][N2] face matrices of one row variable i
-  static constexpr int JQ = E + 24 * N2 * N2;   // [2 buffers][2 own/other][6 slot][NQF][4 j] weighted Jacobian entries
-  static constexpr int B2 = JQ + 2 * 2 * 6 * NQF * 4;  // [NQF][N2]
-  static constexpr int W2 = B2 + NQF * N2;      // [NQF]
-  static constexpr int PVN = W2 + NQF;          // [6 slot][NB] P_hat_a(side) of mode n's exponent along the slot's axis
-  static constexpr int SLOT = PVN + 6 * NB;     // [6] scale of the slot's off-diagonal block
-  // last, sized for the coarse degree of the handle (n2c 2D modes): [6 slot][4 j][n2c][n2c] the
-  // face matrices with the other side's columns; the ints follow it
-  static constexpr int EO = SLOT + 6;
-  __host__ __device__ static constexpr int doubles(int n2c) { return EO + 24 * n2c * n2c; }
-  static constexpr int FMN = 0;                 // [6 slot][NB] 2D mode of mode n on the slot's face
-  static constexpr int PVO = FMN + 6 * NB;      // [6 slot][NB] index of P_hat_a(other side) of mode n (into pv)
-  static constexpr int SINFO = PVO + 6 * NB;    // [6][3] face index, neighbour, target slot
-  static constexpr int INTS = SINFO + 18;
-  __host__ __device__ static constexpr size_t bytes(int n2c) { return sizeof(R) * doubles(n2c) + sizeof(int) * INTS; }
+  static constexpr int NB = nb_of(K), NBM = nb_of(K - 1), N1 = K + 1, NN = N1 * N1, NQ = NN * N1, N2 = tri(K + 1);
+  static constexpr int VP = NN | 1, EP = N2 * N2 | 1;  // odd strides of planes and matrices: no bank conflicts
+  static constexpr int NT = K == 4 ? 288 : 256;          // threads: whole sets of 4 NB rows
+  static constexpr int MATS = 24;                        // matrices of the pressure column, the most at a time
+  static constexpr int RAW = 0;                          // [6][4][NN][4] the slots' Jacobian records
+  static constexpr int V = RAW + 6 * 16 * NN;            // [2 MATS][NN] weighted point values: own side, other side
+  static constexpr int E = V + 2 * MATS * VP;            // [MATS][N2][N2]
+  static constexpr int U = E + MATS * EP;                // [3][NBM][NB]
+  static constexpr int S = U + 3 * NBM * NB;             // [NB][NB] sum_p J_p (D_p^T U_p)
+  static constexpr int PV = S + NB * NB;                 // [2][N1] P_hat_a(+1), P_hat_a(-1)
+  static constexpr int PP = PV + 2 * N1;                 // [N2][N1] pair_tab
+  static constexpr int PN = PP + N2 * N1;                // [3][NB] P_hat of mode n's exponent along d at +1
+  static constexpr int UB = PN + 3 * NB;                 // [3][NQ] the linearisation velocity
+  static constexpr int SLOT = UB + 3 * NQ;               // [2 elements][6] scale of the slot's off-diagonal block
+  static constexpr int EO = SLOT + 12;                   // [MATS][n2c][n2c] the other side's, for the coarse 2D modes
+  __host__ __device__ static constexpr int reals(int n2c) { return EO + MATS * (n2c * n2c | 1); }
+  static constexpr int FM = 0;                           // [3][NB] 2D mode of mode n on a face normal to d
+  static constexpr int EX = FM + 3 * NB;                 // [3][NB] exponent of mode n along d
+  static constexpr int OFF = EX + 3 * NB;                // [3][2][NB] matrix pair and column of mode n, by the row's parity
+  static constexpr int SI = OFF + 6 * NB;                // [2 elements][6][2] neighbour (-1: wall), first slot facing it
+  static constexpr int INTS = SI + 24;
+  __host__ __device__ static constexpr size_t bytes(int n2c) { return sizeof(R) * reals(n2c) + sizeof(int) * INTS; }
 };
 
 template <class R>
 struct AsmArgs {
   MeshDev M;
   Tables T;
-  const R* Bvol;       // tables in the assembly precision
-  const R* wvol;
-  const R* B2;
+  const R* wvol;       // tables in the assembly precision
   const R* W2;
   const R* pv;
   const R* Dcol_val;
@@ -93,307 +144,334 @@ __device__ __forceinline__ R flux_jacobian(const R* p, int stride, int d, int i,
   return j == 3 ? v : v + p[3 * stride + 2 * t + s];
 }
 
+// M[A][B] = sum_{q1, q2} v[q1][q2] B_A B_B(q1, q2) over the 2D modes A, B of degree <= kmax (<= K),
+// symmetric, rows of ld; plane(it, v, m, kmax, ld): the plane and matrix of item it < items, false to
+// skip it. One thread per item and pair a1 <= a2 of exponents along the first axis. A loop with the
+// exponents at run time: unrolled over the pairs at compile time (15 code paths at k = 4, three instances)
+// the kernel waited on instruction fetch 60 % of the time.
+template <int K, class R, class Plane>
+__device__ __forceinline__ void plane_matrices(int items, const R* sPP, int tid, int nt, Plane plane) {
+  constexpr int N1 = K + 1;
+  for (int w = tid; w < items * tri(N1); w += nt) {
+    const int pr = w / items, it = w - pr * items;
+    int a2 = 0;
+    while (tri(a2 + 1) <= pr) ++a2;
+    const int a1 = pr - tri(a2);
+    const R* v;
+    R* m;
+    int kmax, ld;
+    if (!plane(it, v, m, kmax, ld)) continue;
+    R t[N1];
+#pragma unroll
+    for (int q2 = 0; q2 < N1; ++q2) t[q2] = R(0);
+#pragma unroll
+    for (int q = 0; q < N1; ++q) {
+      const R pp = sPP[pr * N1 + q];
+#pragma unroll
+      for (int q2 = 0; q2 < N1; ++q2) t[q2] += pp * v[q * N1 + q2];
+    }
+    const bool sym = a1 == a2;
+    const int n2 = kmax - a2;
+    // the 2D modes (a1, b1), (a2, b2)
+    for (int b1 = 0, b2 = 0; b1 <= kmax - a1 && b2 <= n2;) {
+      const int i = tri(a1 + b1) + b1, j = tri(a2 + b2) + b2;
+      const R* pp = sPP + (b1 <= b2 ? tri(b2) + b1 : tri(b1) + b2) * N1;
+      R s = R(0);
+#pragma unroll
+      for (int q = 0; q < N1; ++q) s += pp[q] * t[q];
+      m[i * ld + j] = s;
+      m[j * ld + i] = s;
+      if (++b2 > n2) {
+        ++b1;
+        b2 = sym ? b1 : 0;
+      }
+    }
+  }
+}
+
+constexpr int kAsmAhead = 6;  // columns of the linear part a thread loads at a time
+
 template <int K, class R>
-__global__ void __launch_bounds__(256) assemble_state_kernel(AsmArgs<R> a) {
+__global__ void __launch_bounds__(AsmSmem<K, R>::NT, sizeof(R) == 4 ? 3 : 2) assemble_state_kernel(AsmArgs<R> a) {
   using L = AsmSmem<K, R>;
-  constexpr int NB = L::NB, NQ = L::NQ, NQF = L::NQF, N2 = L::N2, K1 = K + 1, BS = 4 * NB, DW = Tables::kDw;
-  constexpr int NDT = 4 * NB;  // diagonal-block tasks (j, m) of one row variable
+  constexpr int NB = L::NB, NBM = L::NBM, N1 = L::N1, NN = L::NN, NQ = L::NQ, N2 = L::N2, VP = L::VP, NN2 = L::EP;
+  constexpr int BS = 4 * NB, MATS = L::MATS, nt = L::NT, nw = nt / 32, DW = (K + 1) / 2, TW = Tables::kDw;
   extern __shared__ __align__(16) unsigned char smraw_[];
   R* sm = reinterpret_cast<R*>(smraw_);
-  R* sB = sm + L::B;
-  R* sUb = sm + L::UB;
-  R* sU = sm + L::U;
+  R* sRaw = sm + L::RAW;
+  R* sV = sm + L::V;
   R* sE = sm + L::E;
+  R* sU = sm + L::U;
+  R* sS = sm + L::S;
+  R* sPv = sm + L::PV;
+  R* sPP = sm + L::PP;
+  R* sPn = sm + L::PN;
+  R* sUb = sm + L::UB;
   R* sEo = sm + L::EO;
-  R* sJ = sm + L::JQ;
-  R* sB2 = sm + L::B2;
-  R* sW2 = sm + L::W2;
-  R* PVN = sm + L::PVN;
-  R* sScl = sm + L::SLOT;
-  const int tid = threadIdx.x, nt = blockDim.x;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int nb1 = a.nb1, b1 = 4 * nb1;
-  // coarse 2D modes: the graded 2D ordering lists the modes of degree <= k_1 first
-  int k1 = 0;
+  int k1 = 0;  // the coarse degree: the graded orderings list the modes of degree <= k1 first
   while (nb1 > 0 && nb_of(k1) < nb1) ++k1;
-  const int N2c = nb1 > 0 ? (k1 + 1) * (k1 + 2) / 2 : 0;  // <= L::N2C: the coarse degree is below K
-  int* ism = reinterpret_cast<int*>(sm + L::doubles(N2c));
-  int* FMN = ism + L::FMN;
-  int* PVO = ism + L::PVO;
-  int* SI = ism + L::SINFO;  // per slot: face index, neighbour (-1 at a wall), target block slot
-  for (int t = tid; t < NQ * NB; t += nt) sB[t] = a.Bvol[t];
-  for (int t = tid; t < NQF * N2; t += nt) sB2[t] = a.B2[t];
-  for (int t = tid; t < NQF; t += nt) sW2[t] = a.W2[t];
-  // per slot sl (face normal d = sl / 2, the element on side 1 of slot 2d and side 0 of slot 2d+1)
-  // and mode n: P_hat of n's exponent along d on the element's side, its 2D face mode, and the
-  // index of P_hat on the other side
-  for (int t = tid; t < 6 * NB; t += nt) {
-    const int sl = t / NB, n = t - sl * NB, d = sl >> 1, side = (sl & 1) ? 0 : 1;
-    PVN[t] = a.pv[side * K1 + a.T.fa[d * NB + n]];
-    PVO[t] = (1 - side) * K1 + a.T.fa[d * NB + n];
-    FMN[t] = a.T.fmap[d * NB + n];
+  const int N2c = nb1 > 0 ? tri(k1 + 1) : 0, NC2 = N2c * N2c | 1;
+  int* ism = reinterpret_cast<int*>(sm + L::reals(N2c));
+  int* FM = ism + L::FM;
+  int* EX = ism + L::EX;
+  int* OFF = ism + L::OFF;
+  for (int t = tid; t < 3 * NB; t += nt) {
+    const int d = t / NB, x = a.T.fa[t], f = a.T.fmap[t];
+    FM[t] = f;
+    EX[t] = x;
+    sPn[t] = a.pv[x];
+    OFF[t + d * NB] = (x & 1 ? NN2 : 0) + f;  // row of even exponent
+    OFF[t + (d + 1) * NB] = (x & 1 ? 0 : NN2) + f;
   }
+  for (int t = tid; t < 2 * N1; t += nt) sPv[t] = a.pv[t];
+  for (int t = tid; t < N2 * N1; t += nt) sPP[t] = pair_tab<R, K>.v[t / N1][t % N1];
   __syncthreads();
-  for (int e = blockIdx.x; e < a.M.ne; e += gridDim.x) {
-    const ElemGeom g = elem_geom(a.M, e);
-    const R Jd[3] = {R(g.J[0]), R(g.J[1]), R(g.J[2])};
-    // Jd at a run-time index through selects (no local-memory copy of the array)
-    auto jd = [&](int c) { return c == 0 ? Jd[0] : (c == 1 ? Jd[1] : Jd[2]); };
-    // the weighted Jacobian entries (i, j) of the six face slots at the face points: the own
-    // side's columns (diagonal block) and the other side's (off-diagonal block); buffer i & 1
-    auto load_jac = [&](int i) {
-      R* dst = sJ + (i & 1) * 2 * 6 * NQF * 4;
-      for (int t = tid; t < 2 * 6 * NQF * 4; t += nt) {
-        const int oth = t / (6 * NQF * 4), r = t - oth * 6 * NQF * 4, sl = r / (NQF * 4), r2 = r - sl * NQF * 4;
-        const int q = r2 >> 2, j = r2 & 3, d = sl >> 1, side = (sl & 1) ? 0 : 1;
-        const int nb_ = a.M.nbr[e * 6 + sl];
-        R v = R(0);
-        if (!oth) {
-          const int f = side == 0 ? 3 * e + d : (nb_ >= 0 ? 3 * nb_ + d : 3 * a.M.ne + a.M.bslot[e]);
-          const R* Jq = a.dFlux + ((size_t)f * 4 * NQF + q) * 4;
-          v = flux_jacobian(Jq, 4 * NQF, d, i, j, side);
-          // at a wall the ghost state (-u_K, p_K) is the element's own: its columns add with
-          // sign -1 (velocity) and +1 (pressure)
-          if (nb_ < 0) v += (j == 3 ? R(1) : -R(1)) * flux_jacobian(Jq, 4 * NQF, d, i, j, 1 - side);
-        } else if (nb_ >= 0 && nb1 > 0) {
-          const int f = side == 0 ? 3 * e + d : 3 * nb_ + d;
-          v = flux_jacobian(a.dFlux + ((size_t)f * 4 * NQF + q) * 4, 4 * NQF, d, i, j, 1 - side);
-        }
-        dst[t] = v * sW2[q];
-      }
-    };
-    for (int t = tid; t < 3 * NQ; t += nt) {
-      const int q = t % NQ;
-      sUb[t] = a.wvol[q] * a.ubar[(size_t)e * 3 * NQ + t];
+  // the rows of the output phases: thread -> row (i, m) of every PARTS-th column
+  constexpr int PARTS = nt / BS;
+  const int row = tid % BS, part = tid / BS, ri = row / NB, rm = row - ri * NB;
+  const int parts1 = nb1 > 0 ? nt / b1 : 1, row1 = nb1 > 0 ? tid % b1 : 0, part1 = nb1 > 0 ? tid / b1 : 0;
+  const int ri1 = nb1 > 0 ? row1 / nb1 : 0, rm1 = row1 - ri1 * nb1;
+  const int qs = nb1 > 0 ? parts1 / nb1 : 0, rs = parts1 - qs * nb1;
+
+  // asynchronous copies of the next element's Jacobian records and velocity, its neighbours and block
+  // scales; its linear part goes to L2 one column variable ahead of its use
+  auto fetch = [&](int e, int buf) {
+    constexpr int CH = NN * (int)sizeof(R);  // 16-byte pieces of a record
+    for (int t = tid; t < 6 * CH; t += nt) {
+      const int sl = t / CH, c = t - sl * CH, d = sl >> 1, nb = a.M.nbr[(size_t)e * 6 + sl];
+      const int f = sl & 1 ? 3 * e + d : (nb >= 0 ? 3 * nb + d : 3 * a.M.ne + a.M.bslot[e]);
+      async_16(reinterpret_cast<unsigned char*>(sRaw) + 16 * t,
+               reinterpret_cast<const unsigned char*>(a.dFlux + (size_t)f * 16 * NN) + 16 * c);
     }
-    if (tid < 6) {
-      const int sl = tid, d = sl >> 1, side = (sl & 1) ? 0 : 1;
-      const int p = a.M.nbr[e * 6 + sl];
+    for (int t = tid; t < 3 * NQ; t += nt) async_value(sUb + t, a.ubar + (size_t)e * 3 * NQ + t, true);
+    const int sl = nt - 1 - tid;
+    if (sl < 6) {
+      int* SI = ism + L::SI + 12 * buf;
+      const int d = sl >> 1, p = a.M.nbr[(size_t)e * 6 + sl];
       int tgt = sl;
       for (int s2 = 0; s2 < sl; ++s2)
-        if (a.M.nbr[e * 6 + s2] == p) { tgt = s2; break; }
-      SI[3 * sl + 0] = side == 0 ? 3 * e + d : (p >= 0 ? 3 * p + d : -1);
-      SI[3 * sl + 1] = p;
-      SI[3 * sl + 2] = tgt;
+        if (a.M.nbr[(size_t)e * 6 + s2] == p) { tgt = s2; break; }
+      SI[2 * sl] = p;
+      SI[2 * sl + 1] = tgt;
       R sc = R(0);
       if (p >= 0) {
-        const ElemGeom gp = elem_geom(a.M, p);
-        const int t1 = (d + 1) % 3, t2 = (d + 2) % 3;
+        const ElemGeom g = elem_geom(a.M, e), gp = elem_geom(a.M, p);
         auto h3 = [&](int c) { return c == 0 ? g.h[0] : (c == 1 ? g.h[1] : g.h[2]); };  // no local memory
-        sc = R((side == 0 ? 1.0 : -1.0) * 0.25 * h3(t1) * h3(t2) * g.is * gp.is);
+        sc = R((sl & 1 ? 1.0 : -1.0) * 0.25 * h3((d + 1) % 3) * h3((d + 2) % 3) * g.is * gp.is);
       }
-      sScl[sl] = sc;
+      sm[L::SLOT + 6 * buf + sl] = sc;
     }
-    load_jac(0);
-    __syncthreads();
-    // weighted mass matrices U_c (symmetric): one thread per mode pair n1 <= n computes all three
-    // c, so the two basis values of a point are loaded once
-    for (int t = tid; t < NB * (NB + 1) / 2; t += nt) {
-      int n1 = 0, r = t;
-      while (r >= NB - n1) { r -= NB - n1; ++n1; }
-      const int n = n1 + r;
-      R acc[3] = {R(0), R(0), R(0)};
-      for (int q = 0; q < NQ; ++q) {
-        const R bb = sB[q * NB + n1] * sB[q * NB + n];
-#pragma unroll
-        for (int c = 0; c < 3; ++c) acc[c] += sUb[c * NQ + q] * bb;
-      }
-#pragma unroll
-      for (int c = 0; c < 3; ++c) {
-        sU[(c * NB + n1) * NB + n] = acc[c];
-        sU[(c * NB + n) * NB + n1] = acc[c];
-      }
+  };
+  auto prefetch_linear = [&](int e, int j) {
+    if (warp != 0 || lane > 6) return;
+    if (lane == 6) {
+      const double* p = a.Dlin + ((size_t)e * BS + j * NB) * BS;
+      prefetch_l2(p, p + NB * BS);
+    } else if (nb1 > 0) {
+      const double* p = a.Blin + ((size_t)e * 7 + 1 + lane) * b1 * b1 + (size_t)j * nb1 * b1;
+      prefetch_l2(p, p + nb1 * b1);
     }
-    for (int i = 0; i < 4; ++i) {
-      // face matrices of row variable i: E[j][sl] = sum_q w_q dF_ij(q) B2[q][j1] B2[q][j2], symmetric
-      // in (j1, j2): threads [0, ntE) take one 2D mode pair j1 <= j2 each (all 4 j and 6 slots;
-      // the four j of a point are one vector) and write both halves; the threads after them
-      // form the other side's matrices for the coarse 2D modes, symmetric as well
-      const R* Jo = sJ + (i & 1) * 2 * 6 * NQF * 4;  // own columns [6][NQF][4]
-      const R* Jx = Jo + 6 * NQF * 4;                 // other side's columns
-      constexpr int NPE = N2 * (N2 + 1) / 2;
-      const int ntE = NPE < nt - 32 ? NPE : nt - 32;
-      const int NPc = N2c * (N2c + 1) / 2;
-      if (tid < ntE) {
-        for (int t = tid; t < NPE; t += ntE) {
-          int j1 = 0, r = t;
-          while (r >= N2 - j1) { r -= N2 - j1; ++j1; }
-          const int j2 = j1 + r;
-          R acc[4][6];
+  };
+  int buf = 0;
+  if ((int)blockIdx.x < a.M.ne) {
+    fetch(blockIdx.x, 0);
+    prefetch_linear(blockIdx.x, 0);
+  }
+  for (int e = blockIdx.x; e < a.M.ne; e += gridDim.x, buf ^= 1) {
+    const int* SI = ism + L::SI + 12 * buf;
+    const R* sScl = sm + L::SLOT + 6 * buf;
+    const R* geo = geo_row<R>(a.M, e);
+    const R J[3] = {geo[5], geo[6], geo[7]};
+    auto jd = [&](int c) { return c == 0 ? J[0] : (c == 1 ? J[1] : J[2]); };  // no local-memory copy
+    // weighted entries of column j: own side, the two faces of an axis combined (planes 2 p even, 2 p + 1
+    // odd), and the other side's slot by slot. Pairs p of j < 3: (axis j, i = p) for p < 4, then
+    // (the other two axes, i = j); of j = 3: (axis p / 4, i = p % 4).
+    auto load_column = [&](int j) {
+      const int np = j < 3 ? 6 : 12;
+      for (int t = tid; t < 3 * np * NN; t += nt) {
+        const int w = t / NN, q = t - w * NN;
+        const int p = w < np ? w : (w - np) >> 1;
+        const int d = j == 3 ? p >> 2 : (p < 4 ? j : (j + p - 3) % 3), i = j == 3 ? p & 3 : (p < 4 ? p : j);
+        const R w2 = __ldg(a.W2 + q);
+        if (w < np) {
+          R v[2];
 #pragma unroll
-          for (int j = 0; j < 4; ++j)
-#pragma unroll
-            for (int sl = 0; sl < 6; ++sl) acc[j][sl] = R(0);
-#pragma unroll 5
-          for (int q = 0; q < NQF; ++q) {
-            const R bb = sB2[q * N2 + j1] * sB2[q * N2 + j2];
-#pragma unroll
-            for (int sl = 0; sl < 6; ++sl) {
-              const R* jv = Jo + (sl * NQF + q) * 4;
-#pragma unroll
-              for (int j = 0; j < 4; ++j) acc[j][sl] += jv[j] * bb;
-            }
+          for (int hi = 0; hi < 2; ++hi) {
+            const R* pj = sRaw + ((2 * d + hi) * 4 * NN + q) * 4;
+            v[hi] = flux_jacobian(pj, 4 * NN, d, i, j, 1 - hi);
+            // at a wall the ghost state (-u_K, p_K) is the element's own: its columns add with
+            // sign -1 (velocity) and +1 (pressure)
+            if (SI[2 * (2 * d + hi)] < 0) v[hi] += (j == 3 ? R(1) : -R(1)) * flux_jacobian(pj, 4 * NN, d, i, j, hi);
           }
-#pragma unroll
-          for (int j = 0; j < 4; ++j)
-#pragma unroll
-            for (int sl = 0; sl < 6; ++sl) {
-              R* Ejs = sE + (j * 6 + sl) * N2 * N2;
-              Ejs[j1 * N2 + j2] = acc[j][sl];
-              Ejs[j2 * N2 + j1] = acc[j][sl];
-            }
-        }
-      } else {
-        for (int t = tid - ntE; t < 6 * 4 * NPc; t += nt - ntE) {
-          const int sl = t / (4 * NPc), r0 = t - sl * 4 * NPc, j = r0 / NPc;
-          int j1 = 0, r = r0 - j * NPc;
-          while (r >= N2c - j1) { r -= N2c - j1; ++j1; }
-          const int j2 = j1 + r;
-          R acc = R(0);
-#pragma unroll 5
-          for (int q = 0; q < NQF; ++q) acc += Jx[(sl * NQF + q) * 4 + j] * (sB2[q * N2 + j1] * sB2[q * N2 + j2]);
-          R* Eo = sEo + (sl * 4 + j) * N2c * N2c;
-          Eo[j1 * N2c + j2] = acc;
-          Eo[j2 * N2c + j1] = acc;
+          sV[(2 * p) * VP + q] = w2 * (v[1] - v[0]);
+          sV[(2 * p + 1) * VP + q] = w2 * (v[1] + v[0]);
+        } else if (nb1 > 0) {
+          const int hi = (w - np) & 1, sl = 2 * d + hi;
+          sV[(MATS + 2 * p + hi) * VP + q] =
+              SI[2 * sl] >= 0 ? w2 * flux_jacobian(sRaw + (sl * 4 * NN + q) * 4, 4 * NN, d, i, j, hi) : R(0);
         }
       }
+    };
+    async_wait_all();
+    __syncthreads();
+    // planes of the weighted linearisation velocity
+    for (int t = tid; t < 3 * NQ; t += nt) sV[t / NN * VP + t % NN] = __ldg(a.wvol + t % NQ) * sUb[t];
+    const bool dup = SI[1] != 0 || SI[3] != 1 || SI[5] != 2 || SI[7] != 3 || SI[9] != 4 || SI[11] != 5;
+    const R shift = R(a.inv_gdt * a.M.geo[(size_t)e * kGeo + 11]);
+#pragma unroll 1
+    for (int j = -1; j < 4; ++j) {  // the volume term's planes, then the column variables
+      const int n = j < 0 ? 3 * N1 : (j < 3 ? 12 : 24);
+      auto planes = [&](int it, const R*& v, R*& m, int& kmax, int& ld) {
+        const bool oth = it >= n;
+        const int p = oth ? it - n : it;
+        v = sV + (oth ? MATS + p : p) * VP;
+        m = oth ? sEo + p * NC2 : sE + p * NN2;
+        kmax = oth ? k1 : K;
+        ld = oth ? N2c : N2;
+        return !oth || nb1 > 0;
+      };
       __syncthreads();
-      if (i < 3) load_jac(i + 1);  // the other buffer, read after the next barrier
-      if constexpr (sizeof(R) == 4) {
-        // FP32: one thread per (j, n, m) over the whole CTA, so that many loads of the probed
-        // linear part are in flight (the FP32 assembly waits on memory, not on its arithmetic)
-        R* Dout = a.D + (size_t)e * BS * BS;
-        const double* Dl = a.Dlin + (size_t)e * BS * BS;
-#pragma unroll 4
-        for (int t = tid; t < 4 * NB * NB; t += nt) {
-          const int j = t / (NB * NB), r = t - j * NB * NB, n = r / NB, m = r - n * NB;
-          R v = R(__ldg(Dl + (size_t)(j * NB + n) * BS + i * NB + m));
-          if (i == j && i < 3 && m == n) v += R(a.inv_gdt * g.sh);
-          if (i < 3 && j < 3) {
-            // -J_j (D_j^T U_i)[m][n] - delta_ij sum_p J_p (D_p^T U_p)[m][n]
-            R cv = R(0);
+      plane_matrices<K, R>(j < 0 ? n : 2 * n, sPP, tid, nt, planes);
+      if (j == 0)
+        for (int t = tid; t < NB * NB; t += nt) {
+          const int m = t / NB, n2 = t - m * NB;
+          R s = R(0);
+#pragma unroll
+          for (int p = 0; p < 3; ++p)
 #pragma unroll
             for (int q = 0; q < DW; ++q) {
-              const int o = (j * NB + m) * DW + q;
-              cv += a.Dcol_val[o] * sU[(i * NB + a.T.Dcol_idx[o]) * NB + n];
+              const int o = (p * NB + m) * TW + q;
+              s += J[p] * __ldg(a.Dcol_val + o) * sU[(p * NBM + __ldg(a.T.Dcol_idx + o)) * NB + n2];
             }
-            v -= jd(j) * cv;
-            if (i == j) {
+          sS[t] = s;
+        }
+      __syncthreads();
+      const int en = e + gridDim.x;
+      if (j < 3) {
+        load_column(j + 1);
+        if (j >= 0) prefetch_linear(e, j + 1);
+      } else if (en < a.M.ne) {
+        fetch(en, buf ^ 1);
+        prefetch_linear(en, 0);
+      }
+      if (j < 0) {
+        // U_c[n1][n], n1 of degree <= K - 1 (what a derivative reaches), along the planes' normal
+        for (int t = tid; t < NBM * NB; t += nt) {
+          const int n1 = t / NB, n2 = t - n1 * NB, x1 = EX[n1], x = EX[n2];
+          const R* pp = sPP + (x1 <= x ? tri(x) + x1 : tri(x1) + x) * N1;
+          const R* Et = sE + FM[n1] * N2 + FM[n2];
 #pragma unroll
-              for (int pp = 0; pp < 3; ++pp) {
-                R c2 = R(0);
+          for (int c = 0; c < 3; ++c) {
+            R u = R(0);
 #pragma unroll
-                for (int q = 0; q < DW; ++q) {
-                  const int o = (pp * NB + m) * DW + q;
-                  c2 += a.Dcol_val[o] * sU[(pp * NB + a.T.Dcol_idx[o]) * NB + n];
+            for (int q = 0; q < N1; ++q) u += pp[q] * Et[(c * N1 + q) * NN2];
+            sU[c * NBM * NB + t] = u;
+          }
+        }
+        continue;
+      }
+      if (part < PARTS) {
+        const double* Dl = a.Dlin + ((size_t)e * BS + j * NB) * BS + row;
+        R* Dout = a.D + ((size_t)e * BS + j * NB) * BS + row;
+        // face terms of the row: up to three axes, coefficient J_d P_hat_a(1) and row of a matrix pair
+        R fc[3];
+        const R* fe[3];
+        const R* fp[3];
+        const int* fo[3];
+#pragma unroll
+        for (int x = 0; x < 3; ++x) {
+          const int d = j == 3 ? x : (j + x) % 3;
+          const int mat = j == 3 ? 8 * x + 2 * ri : (x == 0 ? 2 * ri : 6 + 2 * x);
+          fc[x] = jd(d) * sPn[d * NB + rm];
+          fe[x] = sE + mat * NN2 + FM[d * NB + rm] * N2;
+          fp[x] = sPn + d * NB;
+          fo[x] = OFF + (2 * d + (EX[d * NB + rm] & 1)) * NB;
+        }
+        const bool same = ri == j && j < 3, vol = ri < 3 && j < 3;
+        const int nx = j == 3 || same ? 3 : 1;
+        const R* uq[DW];
+        R uc[DW];
+#pragma unroll
+        for (int q = 0; q < DW; ++q) {
+          const int o = ((vol ? j : 0) * NB + rm) * TW + q;
+          uq[q] = sU + ((vol ? ri : 0) * NBM + __ldg(a.T.Dcol_idx + o)) * NB;
+          uc[q] = vol ? jd(j) * __ldg(a.Dcol_val + o) : R(0);
+        }
+        for (int n0 = part; n0 < NB; n0 += kAsmAhead * PARTS) {
+          double dl[kAsmAhead];
+#pragma unroll
+          for (int u = 0; u < kAsmAhead; ++u) {
+            const int n = n0 + u * PARTS;
+            dl[u] = n < NB ? __ldg(Dl + (size_t)n * BS) : 0.0;
+          }
+#pragma unroll
+          for (int u = 0; u < kAsmAhead; ++u) {
+            const int n = n0 + u * PARTS;
+            if (n < NB) {
+              R v = R(dl[u]);
+              if (vol) {
+                R cv = R(0);
+#pragma unroll
+                for (int q = 0; q < DW; ++q) cv += uc[q] * uq[q][n];
+                v -= cv;
+                if (same) {
+                  v -= sS[rm * NB + n];
+                  if (n == rm) v += shift;
                 }
-                v -= Jd[pp] * c2;
               }
+#pragma unroll
+              for (int x = 0; x < 3; ++x)
+                if (x < nx) v += fc[x] * fp[x][n] * fe[x][fo[x][n]];
+              Dout[(size_t)n * BS] = v;
             }
           }
-#pragma unroll
-          for (int sl = 0; sl < 6; ++sl) {
-            const int d = sl >> 1;
-            const R scale = ((sl & 1) ? R(1) : -R(1)) * Jd[d];  // A4 / s^2 = 2 / h_d, sign of the side
-            v += scale * PVN[sl * NB + m] * PVN[sl * NB + n] *
-                 sE[((j * 6 + sl) * N2 + FMN[sl * NB + m]) * N2 + FMN[sl * NB + n]];
-          }
-          Dout[(size_t)(j * NB + n) * BS + i * NB + m] = v;
-        }
-        if (nb1 > 0)
-          for (int t = tid; t < 6 * 4 * nb1 * nb1; t += nt) {
-            const int so = t / (4 * nb1 * nb1), r = t - so * 4 * nb1 * nb1, j = r / (nb1 * nb1), r2 = r - j * nb1 * nb1;
-            const int n = r2 / nb1, m = r2 - n * nb1;
-            const size_t o = (size_t)(j * nb1 + n) * b1 + i * nb1 + m;
-            R* blk = a.Bsr + ((size_t)e * 7 + 1 + so) * b1 * b1;
-            if (SI[3 * so + 1] < 0 || SI[3 * so + 2] != so) {
-              blk[o] = R(0);
-              continue;
-            }
-            R v = R(a.Blin[((size_t)e * 7 + 1 + so) * b1 * b1 + o]);
-            for (int sl = so; sl < 6; ++sl) {
-              if (SI[3 * sl + 1] < 0 || SI[3 * sl + 2] != so) continue;
-              v += sScl[sl] * PVN[sl * NB + m] * a.pv[PVO[sl * NB + n]] *
-                   sEo[((sl * 4 + j) * N2c + FMN[sl * NB + m]) * N2c + FMN[sl * NB + n]];
-            }
-            blk[o] = v;
-          }
-      } else if (tid < NDT) {
-        // the diagonal block's rows of variable i: one thread per (j, m), all columns n
-        const int j = tid / NB, m = tid - j * NB;
-        R* Dout = a.D + (size_t)e * BS * BS + i * NB + m;
-        const double* Dl = a.Dlin + (size_t)e * BS * BS + i * NB + m;
-        R pm[6];
-        int fm[6];
-#pragma unroll
-        for (int sl = 0; sl < 6; ++sl) {
-          const int d = sl >> 1, side = (sl & 1) ? 0 : 1;
-          pm[sl] = (side == 0 ? R(1) : -R(1)) * Jd[d] * PVN[sl * NB + m];  // A4 / s^2 = 2 / h_d
-          fm[sl] = ((j * 6 + sl) * N2 + FMN[sl * NB + m]) * N2;
-        }
-        // -J_j (D_j^T U_i)[m][n] - delta_ij sum_p J_p (D_p^T U_p)[m][n]: rows of U the sparse
-        // derivative picks for (j, m) and, on the diagonal pair, for every p
-        const bool vol = i < 3 && j < 3;
-        int ui[4][DW];
-        R uv[4][DW];
-#pragma unroll
-        for (int pp = 0; pp < 4; ++pp)
-#pragma unroll
-          for (int q = 0; q < DW; ++q) {
-            const int dj = pp < 3 ? pp : j;  // slot 3: the off-diagonal term -J_j (D_j^T U_i)
-            const int ci = pp < 3 ? pp : i;
-            const int o = (dj * NB + m) * DW + q;
-            const bool use = vol && (pp == 3 || i == j);
-            ui[pp][q] = use ? (ci * NB + a.T.Dcol_idx[o]) * NB : 0;
-            uv[pp][q] = use ? -a.Dcol_val[o] * (pp < 3 ? jd(pp) : jd(j)) : R(0);
-          }
-        const R shift = R(a.inv_gdt * g.sh);
-#pragma unroll 5
-        for (int n = 0; n < NB; ++n) {
-          R v = R(__ldg(Dl + (size_t)(j * NB + n) * BS));
-          if (i == j && i < 3 && m == n) v += shift;
-          if (vol) {
-            R cv = R(0);
-#pragma unroll
-            for (int q = 0; q < DW; ++q) cv += uv[3][q] * sU[ui[3][q] + n];
-            v += cv;
-            if (i == j) {
-#pragma unroll
-              for (int pp = 0; pp < 3; ++pp) {
-                R c2 = R(0);
-#pragma unroll
-                for (int q = 0; q < DW; ++q) c2 += uv[pp][q] * sU[ui[pp][q] + n];
-                v += c2;
-              }
-            }
-          }
-#pragma unroll
-          for (int sl = 0; sl < 6; ++sl) v += pm[sl] * PVN[sl * NB + n] * sE[fm[sl] + FMN[sl * NB + n]];
-          Dout[(size_t)(j * NB + n) * BS] = v;
-        }
-      } else if (nb1 > 0) {
-        // level-1 off-diagonal blocks, rows of variable i, coarse modes only: the linear part of
-        // the slot plus the Riemann terms of every slot facing the same neighbour, in slot order
-        // (a neighbour met on two faces keeps its block at the first slot; the other is zero; a
-        // wall slot is zero)
-        for (int t = tid - NDT; t < 6 * 4 * nb1 * nb1; t += nt - NDT) {
-          const int so = t / (4 * nb1 * nb1), r = t - so * 4 * nb1 * nb1, j = r / (nb1 * nb1), r2 = r - j * nb1 * nb1;
-          const int n = r2 / nb1, m = r2 - n * nb1;
-          const size_t o = (size_t)(j * nb1 + n) * b1 + i * nb1 + m;
-          R* blk = a.Bsr + ((size_t)e * 7 + 1 + so) * b1 * b1;
-          if (SI[3 * so + 1] < 0 || SI[3 * so + 2] != so) {
-            blk[o] = R(0);
-            continue;
-          }
-          R v = R(a.Blin[((size_t)e * 7 + 1 + so) * b1 * b1 + o]);
-          for (int sl = so; sl < 6; ++sl) {
-            if (SI[3 * sl + 1] < 0 || SI[3 * sl + 2] != so) continue;
-            v += sScl[sl] * PVN[sl * NB + m] * a.pv[PVO[sl * NB + n]] *
-                 sEo[((sl * 4 + j) * N2c + FMN[sl * NB + m]) * N2c + FMN[sl * NB + n]];
-          }
-          blk[o] = v;
         }
       }
-      __syncthreads();
+      // level-1 off-diagonal blocks, coarse modes only: the linear part of the slot plus the Riemann
+      // terms of every slot facing the same neighbour, in slot order (a neighbour met on two faces
+      // keeps its block at the first slot; the other is zero; a wall slot is zero)
+      if (part1 < parts1 && nb1 > 0) {
+        const size_t base = (size_t)e * 7 * b1 * b1 + (size_t)j * nb1 * b1 + row1;
+        // every parts1-th (slot, column) pair in order, without a division per entry
+        int so_l = part1 / nb1, n_l = part1 - so_l * nb1, so_s = so_l, n_s = n_l;
+        auto next = [&](int& so, int& n) {
+          so += qs;
+          n += rs;
+          if (n >= nb1) {
+            n -= nb1;
+            ++so;
+          }
+        };
+        while (so_s < 6) {
+          double bl[kAsmAhead];
+#pragma unroll
+          for (int u = 0; u < kAsmAhead; ++u) {
+            bl[u] = so_l < 6 ? __ldg(a.Blin + base + (size_t)(1 + so_l) * b1 * b1 + (size_t)n_l * b1) : 0.0;
+            next(so_l, n_l);
+          }
+#pragma unroll
+          for (int u = 0; u < kAsmAhead; ++u) {
+            const int so = so_s, n = n_s;
+            if (so >= 6) break;
+            next(so_s, n_s);
+            R v = R(0);
+            if (SI[2 * so] >= 0 && SI[2 * so + 1] == so) {
+              v = R(bl[u]);
+              for (int sl = so; sl < (dup ? 6 : so + 1); ++sl) {
+                if (SI[2 * sl] < 0 || SI[2 * sl + 1] != so) continue;
+                const int d = sl >> 1, hi = sl & 1, dj = d - j + (d < j ? 3 : 0);
+                if (j < 3 && d != j && ri1 != j) continue;  // no coupling through this axis
+                const int mat = j == 3 ? 2 * (4 * d + ri1) + hi : (d == j ? 2 * ri1 + hi : 6 + 2 * dj + hi);
+                v += sScl[sl] * sPv[(1 - hi) * N1 + EX[d * NB + rm1]] * sPv[hi * N1 + EX[d * NB + n]] *
+                     sEo[mat * NC2 + FM[d * NB + rm1] * N2c + FM[d * NB + n]];
+              }
+            }
+            a.Bsr[base + (size_t)(1 + so) * b1 * b1 + (size_t)n * b1] = v;
+          }
+        }
+      }
     }
   }
 }
@@ -401,18 +479,15 @@ __global__ void __launch_bounds__(256) assemble_state_kernel(AsmArgs<R> a) {
 template <int K, class R>
 static int launch_assemble_state(Handle* h, const AsmArgs<R>& a, cudaStream_t st) {
   // the coarse face matrices are sized for the handle's level-1 degree
-  const int n2c = a.nb1 > 0 ? (h->lev[1].k + 1) * (h->lev[1].k + 2) / 2 : 0;
+  const int n2c = a.nb1 > 0 ? tri(h->lev[1].k + 1) : 0, threads = AsmSmem<K, R>::NT;
   const size_t smem = AsmSmem<K, R>::bytes(n2c);
   DG_CUDA(h, cudaFuncSetAttribute(assemble_state_kernel<K, R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-  int per_sm = (int)((227 * 1024) / (smem + 1024));  // 1 KB of each CTA's shared memory is reserved
-  int res = 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&res, assemble_state_kernel<K, R>, 256, smem) == cudaSuccess &&
-      res > 0 && res < per_sm)
-    per_sm = res;
-  per_sm = per_sm < 1 ? 1 : (per_sm > 4 ? 4 : per_sm);
-  int grid = h->nsm * per_sm;
-  if (grid > h->ne) grid = h->ne;
-  assemble_state_kernel<K, R><<<grid, 256, smem, st>>>(a);
+  int per_sm = 0;
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, assemble_state_kernel<K, R>, threads, smem) != cudaSuccess ||
+      per_sm < 1)
+    per_sm = 1;
+  const int grid = std::min(h->ne, h->nsm * per_sm);
+  assemble_state_kernel<K, R><<<grid, threads, smem, st>>>(a);
   DG_LAUNCH_CHECK(h);
   return DG_OK;
 }
@@ -814,7 +889,7 @@ int assemble_all(Handle* h, int precision, cudaStream_t st) {
     AsmArgs<double> a;
     a.M = mesh_dev(h);
     a.T = h->tab;
-    a.Bvol = h->tab.Bvol; a.wvol = h->tab.wvol; a.B2 = h->tab.B2; a.W2 = h->tab.W2; a.pv = h->tab.pv;
+    a.wvol = h->tab.wvol; a.W2 = h->tab.W2; a.pv = h->tab.pv;
     a.Dcol_val = h->tab.Dcol_val;
     a.ubar = h->ubar;
     a.dFlux = h->dFlux;
@@ -839,7 +914,7 @@ int assemble_all(Handle* h, int precision, cudaStream_t st) {
     const TablesF& F = h->tabf;
     a.M = mesh_dev(h);
     a.T = h->tab;
-    a.Bvol = F.Bvol; a.wvol = F.wvol; a.B2 = F.B2; a.W2 = F.W2; a.pv = F.pv; a.Dcol_val = F.Dcol_val;
+    a.wvol = F.wvol; a.W2 = F.W2; a.pv = F.pv; a.Dcol_val = F.Dcol_val;
     a.ubar = h->ubar_f;
     a.dFlux = h->dFlux_f;
     a.Dlin = L0.Dlin;

@@ -49,6 +49,10 @@ __device__ __forceinline__ void async_value8(R* dst, const R* src, bool on) {
   asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;" ::"r"(smem_u32(dst)), "l"(src), "r"(on ? 8 : 0)
                : "memory");
 }
+// the same for 16 bytes (both addresses 16-byte aligned)
+__device__ __forceinline__ void async_16(void* dst, const void* src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(dst)), "l"(src) : "memory");
+}
 __device__ __forceinline__ void async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 // Order this thread's earlier generic-proxy accesses of shared memory (ordinary loads and
 // stores) before later async-proxy accesses of it (a bulk copy that overwrites the same bytes).
