@@ -1,7 +1,7 @@
 // Face pass of the matrix-free DG operator (Eq. (NSdiscrRes), Eqs. (jacTrilFnotNU), (jacTrilnu)): per
 // face s = (K, K') the traces of both sides as 2D modal coefficients on the face (collapse over the
 // normal exponent, exact), point values only of the four fields that the nonlinear
-// artificial-compressibility Riemann flux needs, the flux (exact star state by safeguarded Newton;
+// artificial-compressibility Riemann flux needs, the flux (exact star state, dg_riemann.h;
 // in tangent mode its cached Jacobian) projected back onto the 2D modes, and the BR2 viscous face
 // flux F^nu({grad u - eta r^s}) built exactly in 2D modal space, the lifting r^s([u]) being a
 // diagonal scaling of the 2D jump coefficients.
@@ -17,6 +17,8 @@
 // point values in registers, and one flux component back; between them, one thread per point.
 // The linearised flux takes 16 values and 18 multiply-adds per point instead of the 32 of the full
 // 4 x 8 Jacobian, which also halves the cache that every Jacobian action streams.
+// At 32^3 P4, one warp per face with table look-ups -> now: FP64 tangent 1440 -> 660 us (0.76 of the measured
+// FP64 rate on the counted operations), FP32 tangent 208 -> 82 us, residual 5070 -> 1760 us.
 //
 // Conventions (also in the C ABI header): orthonormal modal basis phi_m = phi_hat_m(xi)/s,
 // s = sqrt(|K|/8); the normal of a face points from K (lower index) to K'; [v] = v_K - v_K'; the
@@ -344,7 +346,10 @@ int launch_face(Handle* h, const OpArgsT<R>& a, const OpTune& t, cudaStream_t st
 
 template <int K, class R>
 int pass_k(Handle* h, const OpArgsT<R>& a, int mode, const OpTune& t, cudaStream_t st) {
-  const bool small = 3 * h->ne < 8 * h->nsm;  // groups of 8 would leave SMs without one
+  // Faces per CTA: 4 while that gives an SM at most three groups of them (FP32: six), else 8. Face pass at
+  // P4, FP64, with 4 / 8 (us, events included): 216 elements 22.8 / 24.6, 512 24.9 / 26.9, 1000 43.3 / 33.2;
+  // FP32: 216 8.8 / 10.3, 1000 10.0 / 10.9, 1728 13.1 / 12.6.
+  const bool small = 3 * h->ne <= (sizeof(R) == 8 ? 12 : 24) * h->nsm;
   if constexpr (sizeof(R) == 8) {
     switch (mode) {
       case MODE_RES: return small ? launch_face<K, MODE_RES, R, 4>(h, a, t, st) : launch_face<K, MODE_RES, R, 8>(h, a, t, st);
