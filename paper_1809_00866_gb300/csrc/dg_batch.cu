@@ -20,6 +20,7 @@
 #include <vector>
 
 #include "dg_internal.h"
+#include "dg_launch.h"
 #include "dg_reduce.h"
 
 namespace dg {
@@ -58,6 +59,7 @@ struct BatchDev {
 __global__ void __launch_bounds__(kSegThreads) seg_dot_kernel(int nchunk, const int2* chunk, int per_e, const double* V,
                                                               long long ldv, int nv_fixed, const int* jdev,
                                                               const double* w, double* part, int ld) {
+  if (!wait_previous()) return;
   __shared__ double red[kSegThreads / 32][8];
   const int nv = nv_fixed > 0 ? nv_fixed : jdev[0] + 1;
   for (int c = blockIdx.x; c < nchunk; c += gridDim.x) {
@@ -75,6 +77,7 @@ __global__ void __launch_bounds__(kSegThreads) seg_dot_kernel(int nchunk, const 
 __global__ void __launch_bounds__(kSegThreads) seg_reduce_kernel(const int* pchunk0, const double* part, int ld,
                                                                  int nv_fixed, const int* jdev, double* pass,
                                                                  double* sum, int accumulate, int pld) {
+  if (!wait_previous()) return;
   const int p = blockIdx.x;
   const int c0 = pchunk0[p], c1 = pchunk0[p + 1];
   const int nv = nv_fixed > 0 ? nv_fixed : jdev[0] + 1;
@@ -93,6 +96,7 @@ __global__ void __launch_bounds__(kSegThreads) seg_reduce_kernel(const int* pchu
 // w <- w - sum_{v <= j} V_v coef[p][v], p the problem of the entry
 __global__ void seg_axpy_kernel(long long n, int per_e, const int* elem_prob, const double* V, long long ldv,
                                 const int* jdev, const double* coef, int pld, double* w) {
+  if (!wait_previous()) return;
   const int nv = jdev[0] + 1;
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
     const double* cp = coef + (size_t)elem_prob[i / per_e] * pld;
@@ -106,6 +110,7 @@ __global__ void seg_axpy_kernel(long long n, int per_e, const int* elem_prob, co
 // V_j <- src * scale[p] and vin <- the same, j = jdev[0]
 __global__ void batch_normalize_kernel(long long n, int per_e, const int* elem_prob, const double* src,
                                        const double* scale, const int* jdev, double* V, double* vin) {
+  if (!wait_previous()) return;
   double* vj = V + (size_t)jdev[0] * n;
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
     const double v = src[i] * scale[elem_prob[i / per_e]];
@@ -116,6 +121,7 @@ __global__ void batch_normalize_kernel(long long n, int per_e, const int* elem_p
 
 // Z_j <- z, j = jdev[0]
 __global__ void batch_store_kernel(long long n, const double* z, const int* jdev, double* Z) {
+  if (!wait_previous()) return;
   double* zj = Z + (size_t)jdev[0] * n;
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
     zj[i] = z[i];
@@ -124,6 +130,7 @@ __global__ void batch_store_kernel(long long n, const double* z, const int* jdev
 // Start of a restart cycle: beta_p = ||r_p|| (nrm2), s_p = beta_p e_1, which problems iterate.
 __global__ void __launch_bounds__(1024) batch_cycle_init_kernel(int np, int m, int limit, int first, BatchDev d,
                                                                 cudaGraphConditionalHandle hc, int use_cond) {
+  if (!wait_previous()) return;
   int any = 0;
   for (int p = threadIdx.x; p < np; p += blockDim.x) {
     const double beta = sqrt(d.nrm2[p]);
@@ -156,6 +163,7 @@ __global__ void __launch_bounds__(1024) batch_cycle_init_kernel(int np, int m, i
 // loop condition.
 __global__ void __launch_bounds__(1024) batch_givens_kernel(int np, int m, int limit, double rtol, BatchDev d,
                                                             cudaGraphConditionalHandle hc, int use_cond) {
+  if (!wait_previous()) return;
   const int j = d.ctl[kCtlJ];
   int any = 0;
   for (int p = threadIdx.x; p < np; p += blockDim.x) {
@@ -211,6 +219,7 @@ __global__ void __launch_bounds__(1024) batch_givens_kernel(int np, int m, int l
 
 // y_p = R_p^-1 s_p over the problem's own steps (upper-triangular back substitution)
 __global__ void batch_backsub_kernel(int np, int m, BatchDev d) {
+  if (!wait_previous()) return;
   for (int p = blockIdx.x * blockDim.x + threadIdx.x; p < np; p += gridDim.x * blockDim.x) {
     const int jd = d.jdone[p];
     const double* H = d.H + (size_t)p * (m + 1) * m;
@@ -227,6 +236,7 @@ __global__ void batch_backsub_kernel(int np, int m, BatchDev d) {
 // x <- x + sum_{k < jdone_p} Z_k y_p[k]
 __global__ void batch_update_kernel(long long n, int per_e, const int* elem_prob, const double* Z, int m, BatchDev d,
                                     double* x) {
+  if (!wait_previous()) return;
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
     const int p = elem_prob[i / per_e];
     const int jd = d.jdone[p];
@@ -239,6 +249,7 @@ __global__ void batch_update_kernel(long long n, int per_e, const int* elem_prob
 
 // After the true residual of a cycle (its squared norms in nrm2): convergence per problem.
 __global__ void __launch_bounds__(1024) batch_cycle_end_kernel(int np, int limit, double rtol, int fixed, BatchDev d) {
+  if (!wait_previous()) return;
   int undone = 0, missed = 0;
   for (int p = threadIdx.x; p < np; p += blockDim.x) {
     const double rn = sqrt(d.nrm2[p]);
@@ -358,10 +369,10 @@ static void free_ws(BatchWs& b) {
 // squared norms per problem of x into d.nrm2
 static int seg_norm2(BatchWs& b, const double* x, cudaStream_t st) {
   Handle* h = b.h;
-  seg_dot_kernel<<<seg_grid(h, h->nchunk), kSegThreads, 0, st>>>(h->nchunk, h->chunk, b.per_e, x, 0, 1, nullptr, x,
-                                                                 b.part, b.m + 1);
+  launch(seg_dot_kernel, seg_grid(h, h->nchunk), kSegThreads, 0, st, h->nchunk, h->chunk, b.per_e, x, 0, 1, nullptr,
+         x, b.part, b.m + 1);
   DG_LAUNCH_CHECK(h);
-  seg_reduce_kernel<<<b.np, kSegThreads, 0, st>>>(h->pchunk0, b.part, b.m + 1, 1, nullptr, b.d.nrm2, nullptr, 0, 1);
+  launch(seg_reduce_kernel, b.np, kSegThreads, 0, st, h->pchunk0, b.part, b.m + 1, 1, nullptr, b.d.nrm2, nullptr, 0, 1);
   DG_LAUNCH_CHECK(h);
   return DG_OK;
 }
@@ -375,25 +386,26 @@ static int arnoldi_step(const Plan& P, BatchWs& b, cudaGraphConditionalHandle hc
   const int gv = seg_grid(h, n / 256 + 1);
   int rc;
   if ((rc = precond_apply(h, o, b.vin, b.zf, st))) return rc;
-  batch_store_kernel<<<gv, 256, 0, st>>>(n, b.zf, b.d.ctl + kCtlJ, b.Z);
+  launch(batch_store_kernel, gv, 256, 0, st, n, b.zf, b.d.ctl + kCtlJ, b.Z);
   DG_LAUNCH_CHECK(h);
   if ((rc = op_tangent(h, b.zf, b.wf, st))) return rc;
   for (int pass = 0; pass < 2; ++pass) {  // classical Gram-Schmidt, twice
-    seg_dot_kernel<<<seg_grid(h, h->nchunk), kSegThreads, 0, st>>>(h->nchunk, h->chunk, b.per_e, b.V, n, 0,
-                                                                   b.d.ctl + kCtlJ, b.wf, b.part, m + 1);
+    launch(seg_dot_kernel, seg_grid(h, h->nchunk), kSegThreads, 0, st, h->nchunk, h->chunk, b.per_e, b.V, n, 0,
+           b.d.ctl + kCtlJ, b.wf, b.part, m + 1);
     DG_LAUNCH_CHECK(h);
-    seg_reduce_kernel<<<b.np, kSegThreads, 0, st>>>(h->pchunk0, b.part, m + 1, 0, b.d.ctl + kCtlJ, b.d.hpass,
-                                                    b.d.hsum, pass, m + 1);
+    launch(seg_reduce_kernel, b.np, kSegThreads, 0, st, h->pchunk0, b.part, m + 1, 0, b.d.ctl + kCtlJ, b.d.hpass,
+           b.d.hsum, pass, m + 1);
     DG_LAUNCH_CHECK(h);
-    seg_axpy_kernel<<<gv, 256, 0, st>>>(n, b.per_e, h->elem_prob, b.V, n, b.d.ctl + kCtlJ, b.d.hpass, m + 1, b.wf);
+    launch(seg_axpy_kernel, gv, 256, 0, st, n, b.per_e, h->elem_prob, b.V, n, b.d.ctl + kCtlJ, b.d.hpass, m + 1, b.wf);
     DG_LAUNCH_CHECK(h);
   }
   if ((rc = seg_norm2(b, b.wf, st))) return rc;
   const int limit = o.fixed_its > 0 ? o.fixed_its : o.maxit;
   const double rtol = o.fixed_its > 0 ? -1.0 : o.rtol;
-  batch_givens_kernel<<<1, 1024, 0, st>>>(b.np, m, limit, rtol, b.d, hc, use_cond);
+  launch(batch_givens_kernel, 1, 1024, 0, st, b.np, m, limit, rtol, b.d, hc, use_cond);
   DG_LAUNCH_CHECK(h);
-  batch_normalize_kernel<<<gv, 256, 0, st>>>(n, b.per_e, h->elem_prob, b.wf, b.d.scale, b.d.ctl + kCtlJ, b.V, b.vin);
+  launch(batch_normalize_kernel, gv, 256, 0, st, n, b.per_e, h->elem_prob, b.wf, b.d.scale, b.d.ctl + kCtlJ, b.V,
+         b.vin);
   DG_LAUNCH_CHECK(h);
   return DG_OK;
 }
@@ -424,10 +436,10 @@ static int cycle_prologue(const Plan& P, BatchWs& b, bool first, cudaGraphCondit
   }
   // later cycles start from the true residual r and its norms left by the previous epilogue
   const int limit = o.fixed_its > 0 ? o.fixed_its : o.maxit;
-  batch_cycle_init_kernel<<<1, 1024, 0, st>>>(b.np, b.m, limit, first ? 1 : 0, b.d, hc, use_cond);
+  launch(batch_cycle_init_kernel, 1, 1024, 0, st, b.np, b.m, limit, first ? 1 : 0, b.d, hc, use_cond);
   DG_LAUNCH_CHECK(h);
-  batch_normalize_kernel<<<seg_grid(h, b.n / 256 + 1), 256, 0, st>>>(b.n, b.per_e, h->elem_prob, b.r, b.d.scale,
-                                                                    b.d.ctl + kCtlJ, b.V, b.vin);
+  launch(batch_normalize_kernel, seg_grid(h, b.n / 256 + 1), 256, 0, st, b.n, b.per_e, h->elem_prob, b.r, b.d.scale,
+         b.d.ctl + kCtlJ, b.V, b.vin);
   DG_LAUNCH_CHECK(h);
   return DG_OK;
 }
@@ -437,16 +449,16 @@ static int cycle_epilogue(const Plan& P, BatchWs& b, cudaStream_t st) {
   Handle* h = b.h;
   const dg_solve_opts& o = P.o;
   int rc;
-  batch_backsub_kernel<<<(b.np + 127) / 128, 128, 0, st>>>(b.np, b.m, b.d);
+  launch(batch_backsub_kernel, (b.np + 127) / 128, 128, 0, st, b.np, b.m, b.d);
   DG_LAUNCH_CHECK(h);
-  batch_update_kernel<<<seg_grid(h, b.n / 256 + 1), 256, 0, st>>>(b.n, b.per_e, h->elem_prob, b.Z, b.m, b.d, b.x);
+  launch(batch_update_kernel, seg_grid(h, b.n / 256 + 1), 256, 0, st, b.n, b.per_e, h->elem_prob, b.Z, b.m, b.d, b.x);
   DG_LAUNCH_CHECK(h);
   if ((rc = op_tangent(h, b.x, b.tmp, st))) return rc;
   DG_CUDA(h, cudaMemcpyAsync(b.r, b.g, sizeof(double) * b.n, cudaMemcpyDeviceToDevice, st));
   if ((rc = launch_axpby(h, b.n, -1.0, b.tmp, 1.0, b.r, st))) return rc;
   if ((rc = seg_norm2(b, b.r, st))) return rc;
   const int limit = o.fixed_its > 0 ? o.fixed_its : o.maxit;
-  batch_cycle_end_kernel<<<1, 1024, 0, st>>>(b.np, limit, o.rtol, o.fixed_its > 0 ? 1 : 0, b.d);
+  launch(batch_cycle_end_kernel, 1, 1024, 0, st, b.np, limit, o.rtol, o.fixed_its > 0 ? 1 : 0, b.d);
   DG_LAUNCH_CHECK(h);
   return DG_OK;
 }

@@ -18,6 +18,7 @@
 
 #include "dg_async.h"
 #include "dg_internal.h"
+#include "dg_launch.h"
 
 namespace dg {
 
@@ -441,6 +442,7 @@ __global__ void __launch_bounds__(kJacobiThreads) staged_jacobi_kernel(int ne, i
                                                                        const R* __restrict__ Gx, R alpha, int x_zero,
                                                                        R* __restrict__ x, unsigned* status,
                                                                        unsigned wait_polls, int withhold_first) {
+  if (!wait_previous()) return;
   extern __shared__ __align__(128) unsigned char sraw_[];
   __shared__ uint64_t bar[kJacobiSlots];
   __shared__ R red[2 * kJacobiThreads];  // partial sums of the column slices
@@ -601,6 +603,7 @@ __global__ void __launch_bounds__(NT) pair_jacobi_kernel(int ne, int ns, const S
                                                          const float* __restrict__ g, const float* __restrict__ Gx,
                                                          float alpha, int x_zero, float* __restrict__ x,
                                                          unsigned* status, unsigned wait_polls, int withhold_first) {
+  if (!wait_previous()) return;
   static_assert(B % 4 == 0 && sizeof(S) == 2, "16-bit blocks of 4 n rows");
   constexpr int CP = B / 4;                  // 16-byte chunks per column pair
   constexpr int NP = B / 2;                  // column pairs
@@ -760,6 +763,7 @@ template <class R, class S>
 __global__ void __launch_bounds__(kRowThreads, sizeof(S) == 2 ? 4 : 3) block_row_kernel(int ne, int b, int epc, const S* __restrict__ A,
                                                                 const int* __restrict__ nbr, const R* __restrict__ v,
                                                                 R alpha, R beta, R* __restrict__ y) {
+  if (!wait_previous()) return;
   constexpr int VW = 16 / sizeof(S), U = kColsAhead;  // rows of a task, columns loaded at a time (b % U == 0)
   extern __shared__ __align__(16) unsigned char sraw_[];
   const int ncol = 7 * b, rg = b / VW, tpe = 7 * rg;
@@ -826,7 +830,7 @@ int launch_block_rows(Handle* h, int b, const S* A, const R* v, R alpha, R beta,
   const int threads = 32 * ((epc * tpe + 31) / 32);
   const size_t smem = sizeof(R) * (size_t)epc * 14 * b;  // slices of v and partial sums
   const int grid = (h->ne + epc - 1) / epc;
-  block_row_kernel<R, S><<<grid, threads, smem, st>>>(h->ne, b, epc, A, h->nbr, v, alpha, beta, y);
+  launch(block_row_kernel<R, S>, grid, threads, smem, st, h->ne, b, epc, A, h->nbr, v, alpha, beta, y);
   DG_LAUNCH_CHECK(h);
   return DG_OK;
 }
@@ -853,8 +857,8 @@ int launch_pair_jacobi(Handle* h, const S* A, const float* g, const float* Gx, f
   const int cap = h->tune[1].jacobi_max_ctas;  // 0: one CTA per SM
   const int grid = std::min(h->ne, cap > 0 ? std::min(cap, h->nsm) : h->nsm);
   const unsigned polls = h->dbg.wait_polls > 0 ? (unsigned)h->dbg.wait_polls : kBulkWaitLimit;
-  pair_jacobi_kernel<B, NT, S><<<grid, NT, smem, st>>>(h->ne, ns, A, g, Gx, alpha, x_zero, x, h->status, polls,
-                                                      h->dbg.withhold_copy);
+  launch(pair_jacobi_kernel<B, NT, S>, grid, NT, smem, st, h->ne, ns, A, g, Gx, alpha, x_zero, x, h->status, polls,
+         h->dbg.withhold_copy);
   DG_LAUNCH_CHECK(h);
   return DG_OK;
 }
@@ -890,8 +894,8 @@ int launch_staged_jacobi(Handle* h, int b, const S* A, const R* g, const R* Gx, 
   const int per_sm = (int)std::max<size_t>(1, std::min<size_t>(4, (227 * 1024) / (smem + 1024)));
   const int grid = std::min(nstages, cap > 0 ? ctas : h->nsm * per_sm);
   const unsigned polls = h->dbg.wait_polls > 0 ? (unsigned)h->dbg.wait_polls : kBulkWaitLimit;
-  staged_jacobi_kernel<R, S><<<grid, kJacobiThreads, smem, st>>>(h->ne, b, G, ns, A, g, Gx, alpha, x_zero, x,
-                                                                h->status, polls, h->dbg.withhold_copy);
+  launch(staged_jacobi_kernel<R, S>, grid, kJacobiThreads, smem, st, h->ne, b, G, ns, A, g, Gx, alpha, x_zero, x,
+         h->status, polls, h->dbg.withhold_copy);
   DG_LAUNCH_CHECK(h);
   return DG_OK;
 }

@@ -27,6 +27,7 @@
 #include <algorithm>
 
 #include "dg_async.h"
+#include "dg_launch.h"
 #include "dg_opargs.h"
 #include "dg_pencil.h"
 #include "dg_riemann.h"
@@ -129,6 +130,7 @@ __device__ __forceinline__ void face_traces(const R* c, int side, int v, int wal
 
 template <int K, int MODE, class R, int F>
 __global__ void __launch_bounds__(256, sizeof(R) == 4 ? 3 : 2) face_kernel(OpArgsT<R> a) {
+  if (!wait_previous()) return;
   using L = FaceSmem<K, R, F>;
   constexpr int NB = L::NB, N1 = L::N1, NN = L::NN, N2 = L::N2, LD = L::LD, PX = L::PX;
   extern __shared__ __align__(16) unsigned char smraw_[];
@@ -339,7 +341,7 @@ int launch_face(Handle* h, const OpArgsT<R>& a, const OpTune& t, cudaStream_t st
   if (per_sm < 1) per_sm = 1;
   if (t.face_per_sm > 0 && per_sm > t.face_per_sm) per_sm = t.face_per_sm;
   const int groups = 3 * ((h->ne + F - 1) / F) + (h->nbf + F - 1) / F;
-  kern<<<std::min(groups, h->nsm * per_sm), threads, smem, st>>>(a);
+  launch(kern, std::min(groups, h->nsm * per_sm), threads, smem, st, a);
   DG_LAUNCH_CHECK(h);
   return DG_OK;
 }

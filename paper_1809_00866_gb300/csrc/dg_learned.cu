@@ -14,6 +14,7 @@
 
 #include "dg_async.h"
 #include "dg_internal.h"
+#include "dg_launch.h"
 
 namespace dg {
 
@@ -72,6 +73,7 @@ __device__ __forceinline__ float gelu_d(float z) {
 
 // theta (FP32) -> packed BF16 network; one thread per packed slot
 __global__ void pack_kernel(const float* __restrict__ theta, unsigned char* __restrict__ net) {
+  if (!wait_previous()) return;
   int i = blockIdx.x * blockDim.x + threadIdx.x;
   uint16_t* W1 = reinterpret_cast<uint16_t*>(net + kPW1);
   uint16_t* W2 = reinterpret_cast<uint16_t*>(net + kPW2);
@@ -188,6 +190,7 @@ __global__ void __launch_bounds__(32 * kWarps) mlp_forward_kernel(const unsigned
                                                                   const float* __restrict__ X, float* __restrict__ Y,
                                                                   const R* __restrict__ d, const int* __restrict__ nbr,
                                                                   R* __restrict__ x, int accumulate, unsigned* status) {
+  if (!wait_previous()) return;
   extern __shared__ __align__(128) unsigned char sm[];
   __shared__ uint64_t bar;
   start_weights(sm, net, &bar);
@@ -482,6 +485,7 @@ __global__ void __launch_bounds__(32 * kTWarps, 1) mlp_grad_kernel(const unsigne
                                                                   const float* __restrict__ T, long long npairs,
                                                                   int batch, long long seed, long long step,
                                                                   float* __restrict__ part, unsigned* status) {
+  if (!wait_previous()) return;
   extern __shared__ __align__(128) unsigned char sm[];
   __shared__ uint64_t bar;
   __shared__ int ok_all;
@@ -626,6 +630,7 @@ constexpr int kRedCols = 32, kRedRows = 8;
 __global__ void __launch_bounds__(kRedCols* kRedRows) grad_reduce_kernel(const float* __restrict__ part, int nparts,
                                                                          int batch, float* __restrict__ grad,
                                                                          float* __restrict__ loss) {
+  if (!wait_previous()) return;
   __shared__ float4 sum[kRedRows][kRedCols];
   const int x = threadIdx.x % kRedCols, y = threadIdx.x / kRedCols;
   const int q = blockIdx.x * kRedCols + x;  // group of four entries
@@ -732,8 +737,8 @@ int learned_coarse(Handle* h, const R* g, R* x, bool accumulate, cudaStream_t st
   if (smem_opt_in(mlp_forward_kernel<kModeCoarse, R>, kPBytes))
     return fail(h, DG_ERR_CUDA, "cannot opt in to the shared memory of the network kernel");
   const int grid = (int)((h->ne + kRows - 1) / kRows);
-  mlp_forward_kernel<kModeCoarse, R><<<grid, 32 * kWarps, kPBytes, st>>>(h->net, h->ne, nullptr, nullptr, g, h->nbr,
-                                                                         x, accumulate ? 1 : 0, h->status);
+  launch(mlp_forward_kernel<kModeCoarse, R>, grid, 32 * kWarps, kPBytes, st, h->net, h->ne, nullptr, nullptr, g,
+         h->nbr, x, accumulate ? 1 : 0, h->status);
   DG_LAUNCH_CHECK(h);
   return DG_OK;
 }
@@ -765,14 +770,14 @@ int dg_mlp_forward(const float* theta, const float* X, long long n, float* Y, vo
   unsigned* status = mlp_status_ptr();
   if (!status) return fail(nullptr, DG_ERR_CUDA, "cannot look up the status word");
   unsigned char* net = static_cast<unsigned char*>(ws);
-  pack_kernel<<<(kPackSlots + 255) / 256, 256, 0, st>>>(theta, net);
+  launch(pack_kernel, (kPackSlots + 255) / 256, 256, 0, st, theta, net);
   MLP_CUDA(cudaGetLastError());
   if (smem_opt_in(mlp_forward_kernel<kModeFeat, float>, kPBytes))
     return fail(nullptr, DG_ERR_CUDA, "cannot opt in to the shared memory of the network kernel");
   const long long grid = (n + kRows - 1) / kRows;
   if (grid > 0x7fffffffLL) return fail(nullptr, DG_ERR_ARG, "dg_mlp_forward: too many rows");
-  mlp_forward_kernel<kModeFeat, float><<<(unsigned)grid, 32 * kWarps, kPBytes, st>>>(net, n, X, Y, nullptr, nullptr,
-                                                                                  nullptr, 0, status);
+  launch(mlp_forward_kernel<kModeFeat, float>, (unsigned)grid, 32 * kWarps, kPBytes, st, net, n, X, Y, nullptr,
+         nullptr, nullptr, 0, status);
   MLP_CUDA(cudaGetLastError());
   return DG_OK;
 }
@@ -788,14 +793,15 @@ int dg_mlp_grad(const float* theta, const float* X, const float* T, long long np
   if (!status) return fail(nullptr, DG_ERR_CUDA, "cannot look up the status word");
   unsigned char* net = static_cast<unsigned char*>(ws);
   float* part = reinterpret_cast<float*>(net + kPBytes);
-  pack_kernel<<<(kPackSlots + 255) / 256, 256, 0, st>>>(theta, net);
+  launch(pack_kernel, (kPackSlots + 255) / 256, 256, 0, st, theta, net);
   MLP_CUDA(cudaGetLastError());
   if (smem_opt_in(mlp_grad_kernel, kTrainSmem))
     return fail(nullptr, DG_ERR_CUDA, "cannot opt in to the shared memory of the training kernel");
   const int nparts = (int)grad_parts(batch);
-  mlp_grad_kernel<<<nparts, 32 * kTWarps, kTrainSmem, st>>>(net, X, T, npairs, batch, seed, step, part, status);
+  launch(mlp_grad_kernel, nparts, 32 * kTWarps, kTrainSmem, st, net, X, T, npairs, batch, seed, step, part, status);
   MLP_CUDA(cudaGetLastError());
-  grad_reduce_kernel<<<(kNP + 4 * kRedCols) / (4 * kRedCols), kRedCols * kRedRows, 0, st>>>(part, nparts, batch, grad, loss);
+  launch(grad_reduce_kernel, (kNP + 4 * kRedCols) / (4 * kRedCols), kRedCols * kRedRows, 0, st, part, nparts, batch,
+         grad, loss);
   MLP_CUDA(cudaGetLastError());
   return DG_OK;
 }
@@ -822,7 +828,7 @@ int dg_set_coarse_network(dg_handle* hh, const float* theta, void* stream) {
   if (h->lev[h->nlev - 1].k != 1)
     return fail(h, DG_ERR_ARG, "the learned coarse correction needs k = 1 on the coarsest level");
   if (!h->net) DG_CUDA(h, cudaMalloc((void**)&h->net, kPBytes));
-  pack_kernel<<<(kPackSlots + 255) / 256, 256, 0, as_stream(stream)>>>(theta, h->net);
+  launch(pack_kernel, (kPackSlots + 255) / 256, 256, 0, as_stream(stream), theta, h->net);
   DG_LAUNCH_CHECK(h);
   h->net_ready = true;
   return DG_OK;

@@ -7,6 +7,7 @@
 #include <vector>
 
 #include "dg_internal.h"
+#include "dg_launch.h"
 #include "dg_reduce.h"
 
 namespace dg {
@@ -19,6 +20,7 @@ static int red_blocks(long long n) { return (int)std::min<long long>(kRedBlocks,
 // part[b][j] = sum over this block's entries of V[j][i] * w[i], j < nv (nv <= 8 per launch)
 __global__ void __launch_bounds__(256) multidot_partial_kernel(long long n, int nv, const double* V, long long ldv,
                                                                const double* w, double* part, int stride) {
+  if (!wait_previous()) return;
   __shared__ double red[8][8];
   const double s = block_dots<256>(V, ldv, nv, w, blockIdx.x * 256LL, n, gridDim.x * 256LL, red);
   if (threadIdx.x < nv) part[(size_t)blockIdx.x * stride + threadIdx.x] = s;
@@ -27,6 +29,7 @@ __global__ void __launch_bounds__(256) multidot_partial_kernel(long long n, int 
 // out[j] = sum_b part[b * stride + j] for j < nvec, in a fixed order: a warp per vector.
 __global__ void __launch_bounds__(256) reduce_partials_kernel(int nblk, int nvec, int stride, const double* part,
                                                               double* out) {
+  if (!wait_previous()) return;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   for (int j = warp; j < nvec; j += 8) {
     double acc = 0.0;
@@ -38,15 +41,16 @@ __global__ void __launch_bounds__(256) reduce_partials_kernel(int nblk, int nvec
 
 int vec_norm2(Handle* h, const double* x, long long n, double* dev_out, cudaStream_t st) {
   const int nb = red_blocks(n);
-  multidot_partial_kernel<<<nb, 256, 0, st>>>(n, 1, x, n, x, h->red, 1);
+  launch(multidot_partial_kernel, nb, 256, 0, st, n, 1, x, n, x, h->red, 1);
   DG_LAUNCH_CHECK(h);
-  reduce_partials_kernel<<<1, 256, 0, st>>>(nb, 1, 1, h->red, dev_out);
+  launch(reduce_partials_kernel, 1, 256, 0, st, nb, 1, 1, h->red, dev_out);
   DG_LAUNCH_CHECK(h);
   return DG_OK;
 }
 
 // w -= sum_j hcoef[j] * V[j], j < nv; also w is scaled by nothing
 __global__ void multi_axpy_kernel(long long n, int nv, const double* V, long long ldv, const double* hcoef, double* w) {
+  if (!wait_previous()) return;
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
     double acc = w[i];
     for (int j = 0; j < nv; ++j) acc -= hcoef[j] * V[j * ldv + i];
@@ -56,6 +60,7 @@ __global__ void multi_axpy_kernel(long long n, int nv, const double* V, long lon
 
 template <class R>
 __global__ void axpby_kernel(long long n, R a, const R* x, R b, R* y) {
+  if (!wait_previous()) return;
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
     y[i] = a * x[i] + (b == R(0) ? R(0) : b * y[i]);
 }
@@ -63,6 +68,7 @@ __global__ void axpby_kernel(long long n, R a, const R* x, R b, R* y) {
 // FP64 <-> FP32 copies at the boundary of the reduced-precision preconditioner
 template <class A, class B>
 __global__ void convert_kernel(long long n, const A* x, B* y) {
+  if (!wait_previous()) return;
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
     y[i] = (B)x[i];
 }
@@ -75,7 +81,7 @@ __global__ void scale_by_dev_kernel(long long n, const double* x, const double* 
 }
 
 int launch_axpby(Handle* h, long long n, double a, const double* x, double b, double* y, cudaStream_t st) {
-  axpby_kernel<double><<<h->nsm * 8, 256, 0, st>>>(n, a, x, b, y);
+  launch(axpby_kernel<double>, h->nsm * 8, 256, 0, st, n, a, x, b, y);
   DG_LAUNCH_CHECK(h);
   return DG_OK;
 }
@@ -85,6 +91,7 @@ int launch_axpby(Handle* h, long long n, double a, const double* x, double b, do
 // difference over the whole level and a restriction it took two launches)
 template <class R>
 __global__ void restrict_kernel(int ne, int nbf, int nbc, const R* xf, const R* yf, R* xc) {
+  if (!wait_previous()) return;
   const long long n = (long long)ne * 4 * nbc;
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
     const long long ev = i / nbc;
@@ -94,6 +101,7 @@ __global__ void restrict_kernel(int ne, int nbf, int nbc, const R* xf, const R* 
 }
 template <class R>
 __global__ void prolong_add_kernel(int ne, int nbf, int nbc, const R* xc, R* xf) {
+  if (!wait_previous()) return;
   const long long n = (long long)ne * 4 * nbc;
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
     const long long ev = i / nbc;
@@ -107,6 +115,7 @@ __global__ void prolong_add_kernel(int ne, int nbf, int nbc, const R* xc, R* xf)
 template <class R>
 __global__ void __launch_bounds__(128) bsr_kernel(int ne, int b, const int* nbr, const R* B, R alpha,
                                                   const R* x, R beta, R* y) {
+  if (!wait_previous()) return;
   extern __shared__ __align__(16) unsigned char sraw_[];
   R* sx = reinterpret_cast<R*>(sraw_);  // [7][b]
   for (int e = blockIdx.x; e < ne; e += gridDim.x) {
@@ -228,6 +237,7 @@ __global__ void __launch_bounds__(32 * kApplyWarps) bj_update_kernel(int ne, con
                                                                     const int* __restrict__ perm, const double* g,
                                                                     const double* Gx, double omega, int x_zero,
                                                                     double* x) {
+  if (!wait_previous()) return;
   constexpr int SL = (B + 31) / 32;
   __shared__ double sz[kApplyWarps][B];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -274,10 +284,10 @@ static int apply_block_inverse(Handle* h, const Level& L, const double* g, const
                                double* x, cudaStream_t st) {
   const int grid = (h->ne + kApplyWarps - 1) / kApplyWarps, nt = 32 * kApplyWarps;
   switch (L.b) {
-    case 16: bj_update_kernel<16><<<grid, nt, 0, st>>>(h->ne, L.Dinv, L.perm, g, Gx, omega, x_zero, x); break;
-    case 40: bj_update_kernel<40><<<grid, nt, 0, st>>>(h->ne, L.Dinv, L.perm, g, Gx, omega, x_zero, x); break;
-    case 80: bj_update_kernel<80><<<grid, nt, 0, st>>>(h->ne, L.Dinv, L.perm, g, Gx, omega, x_zero, x); break;
-    case 140: bj_update_kernel<140><<<grid, nt, 0, st>>>(h->ne, L.Dinv, L.perm, g, Gx, omega, x_zero, x); break;
+    case 16: launch(bj_update_kernel<16>, grid, nt, 0, st, h->ne, L.Dinv, L.perm, g, Gx, omega, x_zero, x); break;
+    case 40: launch(bj_update_kernel<40>, grid, nt, 0, st, h->ne, L.Dinv, L.perm, g, Gx, omega, x_zero, x); break;
+    case 80: launch(bj_update_kernel<80>, grid, nt, 0, st, h->ne, L.Dinv, L.perm, g, Gx, omega, x_zero, x); break;
+    case 140: launch(bj_update_kernel<140>, grid, nt, 0, st, h->ne, L.Dinv, L.perm, g, Gx, omega, x_zero, x); break;
     default: return fail(h, DG_ERR_ARG, "unsupported block size");
   }
   DG_LAUNCH_CHECK(h);
@@ -288,7 +298,8 @@ static int run_bsr(Handle* h, int lvl, double alpha, const double* x, double bet
   const Level& L = h->lev[lvl];
   const int rc = staged_bsr<double>(h, lvl, L.Bsr, alpha, x, beta, y, st);
   if (rc >= 0) return rc;  // -1: the blocks do not fit the staged kernel
-  bsr_kernel<double><<<grid_for(h, h->ne), 128, sizeof(double) * 7 * L.b, st>>>(h->ne, L.b, h->nbr, L.Bsr, alpha, x, beta, y);
+  launch(bsr_kernel<double>, grid_for(h, h->ne), 128, sizeof(double) * 7 * L.b, st, h->ne, L.b, h->nbr, L.Bsr, alpha,
+         x, beta, y);
   DG_LAUNCH_CHECK(h);
   return DG_OK;
 }
@@ -429,7 +440,7 @@ static int gmres_smooth(Handle* h, int lvl, const double* g, double* x, int its,
     if ((rc = apply_block_inverse(h, L, L.t2, nullptr, 1.0, 1, w, st))) return rc;
     for (int pass = 0; pass < 2; ++pass) {
       if ((rc = multidot(h, n, j + 1, V, w, tmp, st))) return rc;
-      multi_axpy_kernel<<<grid_for(h, n / 256 + 1), 256, 0, st>>>(n, j + 1, V, n, tmp, w);
+      launch(multi_axpy_kernel, grid_for(h, n / 256 + 1), 256, 0, st, n, j + 1, V, n, tmp, w);
       DG_LAUNCH_CHECK(h);
       hcol_accumulate_kernel<<<1, 64, 0, st>>>(Hc + (size_t)j * ld, tmp, j + 1, pass == 0 ? 1 : 0);
       DG_LAUNCH_CHECK(h);
@@ -441,7 +452,7 @@ static int gmres_smooth(Handle* h, int lvl, const double* g, double* x, int its,
   gmres_lsq_kernel<<<1, 32, 0, st>>>(its, Hc, hn2, beta2, ny);
   DG_LAUNCH_CHECK(h);
   if (x_zero) DG_CUDA(h, cudaMemsetAsync(x, 0, sizeof(double) * n, st));
-  multi_axpy_kernel<<<grid_for(h, n / 256 + 1), 256, 0, st>>>(n, its, V, n, ny, x);
+  launch(multi_axpy_kernel, grid_for(h, n / 256 + 1), 256, 0, st, n, its, V, n, ny, x);
   DG_LAUNCH_CHECK(h);
   return DG_OK;
 }
@@ -454,13 +465,13 @@ static int smooth(Handle* h, int lvl, const double* g, double* x, int iters, dou
 
 static int restrict_to(Handle* h, int lvl, const double* xf, const double* yf, double* xc, cudaStream_t st) {
   const Level &F = h->lev[lvl], &C = h->lev[lvl + 1];
-  restrict_kernel<double><<<grid_for(h, C.n / 64 + 1), 256, 0, st>>>(h->ne, F.nb, C.nb, xf, yf, xc);
+  launch(restrict_kernel<double>, grid_for(h, C.n / 64 + 1), 256, 0, st, h->ne, F.nb, C.nb, xf, yf, xc);
   DG_LAUNCH_CHECK(h);
   return DG_OK;
 }
 static int prolong_add(Handle* h, int lvl, const double* xc, double* xf, cudaStream_t st) {
   const Level &F = h->lev[lvl], &C = h->lev[lvl + 1];
-  prolong_add_kernel<double><<<grid_for(h, C.n / 64 + 1), 256, 0, st>>>(h->ne, F.nb, C.nb, xc, xf);
+  launch(prolong_add_kernel<double>, grid_for(h, C.n / 64 + 1), 256, 0, st, h->ne, F.nb, C.nb, xc, xf);
   DG_LAUNCH_CHECK(h);
   return DG_OK;
 }
@@ -505,7 +516,8 @@ static int record_coarse(Handle* h, const double* g, cudaStream_t st) {
 static int record_coarse_f(Handle* h, const float* g, cudaStream_t st) {
   if (!h->rec_buf || h->rec_count >= h->rec_cap) return DG_OK;
   const long long n = h->lev[h->nlev - 1].n;
-  convert_kernel<float, double><<<grid_for(h, n / 256 + 1), 256, 0, st>>>(n, g, h->rec_buf + (size_t)h->rec_count * n);
+  launch(convert_kernel<float, double>, grid_for(h, n / 256 + 1), 256, 0, st, n, g,
+         h->rec_buf + (size_t)h->rec_count * n);
   DG_LAUNCH_CHECK(h);
   ++h->rec_count;
   return DG_OK;
@@ -527,7 +539,7 @@ static int coarse_solve(Handle* h, const double* g, double* x, const dg_solve_op
     if ((rc = learned_coarse<double>(h, g, x, false, st))) return rc;
     for (int it = 0; it < o.coarse_sweeps; ++it) {
       if ((rc = run_bsr(h, Lc, 1.0, x, 0.0, C.t2, st))) return rc;
-      axpby_kernel<double><<<grid_for(h, C.n / 256 + 1), 256, 0, st>>>(C.n, 1.0, g, -1.0, C.t2);
+      launch(axpby_kernel<double>, grid_for(h, C.n / 256 + 1), 256, 0, st, C.n, 1.0, g, -1.0, C.t2);
       DG_LAUNCH_CHECK(h);
       if ((rc = learned_coarse<double>(h, C.t2, x, true, st))) return rc;
     }
@@ -580,7 +592,7 @@ static int mg_full(Handle* h, int l, const double* g, double* x, const dg_solve_
   if ((rc = prolong_add(h, l, C.t1, x, st))) return rc;  // w_hat_l = I w_{l+1}
   // d_l = g - G w_hat_l ; e_l = MG_V(l, d_l, 0) ; x = w_hat + e
   if ((rc = level_matvec(h, l, x, L.t2, st))) return rc;
-  axpby_kernel<double><<<grid_for(h, L.n / 256 + 1), 256, 0, st>>>(L.n, 1.0, g, -1.0, L.t2);
+  launch(axpby_kernel<double>, grid_for(h, L.n / 256 + 1), 256, 0, st, L.n, 1.0, g, -1.0, L.t2);
   DG_LAUNCH_CHECK(h);
   // The V-cycle below uses t2 as scratch on this level, so d_l moves out of it. On the fine
   // level t0/t1 are free here; on coarse levels they hold this level's (g, x), so the fine
@@ -589,7 +601,7 @@ static int mg_full(Handle* h, int l, const double* g, double* x, const dg_solve_
   double* e = l == 0 ? L.t0 : h->fd_f;
   DG_CUDA(h, cudaMemcpyAsync(d, L.t2, sizeof(double) * L.n, cudaMemcpyDeviceToDevice, st));
   if ((rc = mg_v(h, l, d, e, true, o, st))) return rc;
-  axpby_kernel<double><<<grid_for(h, L.n / 256 + 1), 256, 0, st>>>(L.n, 1.0, e, 1.0, x);
+  launch(axpby_kernel<double>, grid_for(h, L.n / 256 + 1), 256, 0, st, L.n, 1.0, e, 1.0, x);
   DG_LAUNCH_CHECK(h);
   return DG_OK;
 }
@@ -602,9 +614,9 @@ int prepare_lin_fp32(Handle* h, cudaStream_t st) {
   if (h->lin_f_ready) return DG_OK;
   const int ne = h->ne;
   const long long nu = (long long)ne * 3 * h->tab.nq, nf = (long long)(3 * ne + h->nbf) * h->tab.nqf * 16;
-  convert_kernel<double, float><<<grid_for(h, nu / 256 + 1), 256, 0, st>>>(nu, h->ubar, h->ubar_f);
+  launch(convert_kernel<double, float>, grid_for(h, nu / 256 + 1), 256, 0, st, nu, h->ubar, h->ubar_f);
   DG_LAUNCH_CHECK(h);
-  convert_kernel<double, float><<<grid_for(h, nf / 256 + 1), 256, 0, st>>>(nf, h->dFlux, h->dFlux_f);
+  launch(convert_kernel<double, float>, grid_for(h, nf / 256 + 1), 256, 0, st, nf, h->dFlux, h->dFlux_f);
   DG_LAUNCH_CHECK(h);
   if (int rc = tc_prepare_lin(h, st)) return rc;  // scales of the tensor-core volume pass
   h->lin_f_ready = true;
@@ -624,11 +636,11 @@ static int prepare_fp32(Handle* h, cudaStream_t st) {
       if (!L.t0f) DG_CUDA(h, cudaMalloc((void**)&L.t0f, sizeof(float) * L.n));
       if (!L.t1f) DG_CUDA(h, cudaMalloc((void**)&L.t1f, sizeof(float) * L.n));
       if (!L.t2f) DG_CUDA(h, cudaMalloc((void**)&L.t2f, sizeof(float) * L.n));
-      convert_kernel<double, float><<<grid_for(h, nbb / 256 + 1), 256, 0, st>>>(nbb, L.Dblk, L.LUf);
+      launch(convert_kernel<double, float>, grid_for(h, nbb / 256 + 1), 256, 0, st, nbb, L.Dblk, L.LUf);
       DG_LAUNCH_CHECK(h);
       if (l >= 1) {
         if (!L.Bsrf) DG_CUDA(h, cudaMalloc((void**)&L.Bsrf, sizeof(float) * nbb * 7));
-        convert_kernel<double, float><<<grid_for(h, 7 * nbb / 256 + 1), 256, 0, st>>>(7 * nbb, L.Bsr, L.Bsrf);
+        launch(convert_kernel<double, float>, grid_for(h, 7 * nbb / 256 + 1), 256, 0, st, 7 * nbb, L.Bsr, L.Bsrf);
         DG_LAUNCH_CHECK(h);
       }
     }
@@ -664,8 +676,8 @@ static int level_matvec_f(Handle* h, int lvl, const float* x, float* y, int prec
   }
   const int rc = staged_bsr<float>(h, lvl, L.Bsrf, 1.0f, x, 0.0f, y, st);
   if (rc >= 0) return rc;
-  bsr_kernel<float><<<grid_for(h, h->ne), 128, sizeof(float) * 7 * L.b, st>>>(h->ne, L.b, h->nbr, L.Bsrf, 1.0f, x,
-                                                                               0.0f, y);
+  launch(bsr_kernel<float>, grid_for(h, h->ne), 128, sizeof(float) * 7 * L.b, st, h->ne, L.b, h->nbr, L.Bsrf, 1.0f, x,
+         0.0f, y);
   DG_LAUNCH_CHECK(h);
   return DG_OK;
 }
@@ -703,7 +715,7 @@ static int mg_v_f(Handle* h, int l, const float* g, float* x, bool x_zero, const
       if ((rc = learned_coarse<float>(h, g, x, false, st))) return rc;
       for (int it = 0; it < o.coarse_sweeps; ++it) {
         if ((rc = level_matvec_f(h, l, x, C.t2f, o.precision, st))) return rc;
-        axpby_kernel<float><<<grid_for(h, C.n / 256 + 1), 256, 0, st>>>(C.n, 1.0f, g, -1.0f, C.t2f);
+        launch(axpby_kernel<float>, grid_for(h, C.n / 256 + 1), 256, 0, st, C.n, 1.0f, g, -1.0f, C.t2f);
         DG_LAUNCH_CHECK(h);
         if ((rc = learned_coarse<float>(h, C.t2f, x, true, st))) return rc;
       }
@@ -716,16 +728,16 @@ static int mg_v_f(Handle* h, int l, const float* g, float* x, bool x_zero, const
   Level& C = h->lev[l + 1];
   const bool xz = x_zero && o.pre_sweeps == 0;
   if (xz) {
-    restrict_kernel<float><<<grid_for(h, C.n / 64 + 1), 256, 0, st>>>(h->ne, L.nb, C.nb, g, nullptr, C.t0f);
+    launch(restrict_kernel<float>, grid_for(h, C.n / 64 + 1), 256, 0, st, h->ne, L.nb, C.nb, g, nullptr, C.t0f);
     DG_LAUNCH_CHECK(h);
   } else {
     if ((rc = level_matvec_f(h, l, x, L.t2f, o.precision, st))) return rc;
-    restrict_kernel<float><<<grid_for(h, C.n / 64 + 1), 256, 0, st>>>(h->ne, L.nb, C.nb, g, L.t2f, C.t0f);
+    launch(restrict_kernel<float>, grid_for(h, C.n / 64 + 1), 256, 0, st, h->ne, L.nb, C.nb, g, L.t2f, C.t0f);
     DG_LAUNCH_CHECK(h);
   }
   if ((rc = mg_v_f(h, l + 1, C.t0f, C.t1f, true, o, st))) return rc;
   if (xz) DG_CUDA(h, cudaMemsetAsync(x, 0, sizeof(float) * L.n, st));
-  prolong_add_kernel<float><<<grid_for(h, C.n / 64 + 1), 256, 0, st>>>(h->ne, L.nb, C.nb, C.t1f, x);
+  launch(prolong_add_kernel<float>, grid_for(h, C.n / 64 + 1), 256, 0, st, h->ne, L.nb, C.nb, C.t1f, x);
   DG_LAUNCH_CHECK(h);
   return jacobi_sweeps_f(h, l, g, x, o.post_sweeps, om, false, o.precision, st);
 }
@@ -737,10 +749,10 @@ static int vcycle_fp32(Handle* h, const dg_solve_opts& o, const double* v, doubl
   if (is16(o.precision) && (rc = prepare_blocks16(h, storage_of(o.precision), st))) return rc;
   if (tc_of(o.precision) && (rc = tc_prepare_tables(h))) return rc;
   Level& L0 = h->lev[0];
-  convert_kernel<double, float><<<grid_for(h, L0.n / 256 + 1), 256, 0, st>>>(L0.n, v, L0.t0f);
+  launch(convert_kernel<double, float>, grid_for(h, L0.n / 256 + 1), 256, 0, st, L0.n, v, L0.t0f);
   DG_LAUNCH_CHECK(h);
   if ((rc = mg_v_f(h, 0, L0.t0f, L0.t1f, true, o, st))) return rc;
-  convert_kernel<float, double><<<grid_for(h, L0.n / 256 + 1), 256, 0, st>>>(L0.n, L0.t1f, z);
+  launch(convert_kernel<float, double>, grid_for(h, L0.n / 256 + 1), 256, 0, st, L0.n, L0.t1f, z);
   DG_LAUNCH_CHECK(h);
   return DG_OK;
 }
@@ -806,9 +818,9 @@ static int outer_matvec(Handle* h, const dg_solve_opts& o, const double* x, doub
 static int multidot(Handle* h, long long n, int nv, const double* V, const double* w, double* hout, cudaStream_t st) {
   for (int j0 = 0; j0 < nv; j0 += 8) {
     const int c = nv - j0 < 8 ? nv - j0 : 8;
-    multidot_partial_kernel<<<red_blocks(n), 256, 0, st>>>(n, c, V + (size_t)j0 * n, n, w, h->red, 8);
+    launch(multidot_partial_kernel, red_blocks(n), 256, 0, st, n, c, V + (size_t)j0 * n, n, w, h->red, 8);
     DG_LAUNCH_CHECK(h);
-    reduce_partials_kernel<<<1, 256, 0, st>>>(red_blocks(n), c, 8, h->red, hout + j0);
+    launch(reduce_partials_kernel, 1, 256, 0, st, red_blocks(n), c, 8, h->red, hout + j0);
     DG_LAUNCH_CHECK(h);
   }
   return DG_OK;
@@ -894,7 +906,7 @@ static int fgmres(Handle* h, const double* g, double* x, const dg_solve_opts& o,
         for (int pass = 0; pass < 2; ++pass) {
           double* hp = h->hcol + pass * (j + 1);
           if ((rc = multidot(h, n, j + 1, V, w, hp, st))) return rc;
-          multi_axpy_kernel<<<grid_for(h, n / 256 + 1), 256, 0, st>>>(n, j + 1, V, n, hp, w);
+          launch(multi_axpy_kernel, grid_for(h, n / 256 + 1), 256, 0, st, n, j + 1, V, n, hp, w);
           DG_LAUNCH_CHECK(h);
         }
         const int nh = 2 * (j + 1);
@@ -946,7 +958,7 @@ static int fgmres(Handle* h, const double* g, double* x, const dg_solve_opts& o,
     }
     for (int i = 0; i < jdone; ++i) h->hcol_host[i] = -y[i];  // multi_axpy subtracts
     DG_CUDA(h, cudaMemcpyAsync(h->hcol, h->hcol_host, sizeof(double) * jdone, cudaMemcpyHostToDevice, st));
-    multi_axpy_kernel<<<grid_for(h, n / 256 + 1), 256, 0, st>>>(n, jdone, Z, n, h->hcol, x);
+    launch(multi_axpy_kernel, grid_for(h, n / 256 + 1), 256, 0, st, n, jdone, Z, n, h->hcol, x);
     DG_LAUNCH_CHECK(h);
     // true residual
     if ((rc = outer_matvec(h, o, x, tmp, st))) return rc;
@@ -1092,7 +1104,7 @@ int pmg_level_solve(dg_handle* hh, int lvl, const double* g, double* x, double r
       if (int c = vec_norm2(h, g, L.n, h->red_out, st)) return c;
     } else {
       if (int c = run_bsr(h, lvl, 1.0, x, 0.0, L.t1, st)) return c;
-      axpby_kernel<double><<<grid_for(h, L.n / 256 + 1), 256, 0, st>>>(L.n, 1.0, g, -1.0, L.t1);
+      launch(axpby_kernel<double>, grid_for(h, L.n / 256 + 1), 256, 0, st, L.n, 1.0, g, -1.0, L.t1);
       DG_LAUNCH_CHECK(h);
       if (int c = vec_norm2(h, L.t1, L.n, h->red_out, st)) return c;
     }

@@ -20,6 +20,7 @@
 #include <algorithm>
 
 #include "dg_async.h"
+#include "dg_launch.h"
 #include "dg_opargs.h"
 #include "dg_volume_phases.h"
 
@@ -49,6 +50,7 @@ struct VolSmem : VolPhases<K, R, E> {
 
 template <int K, int MODE, class R, int E>
 __global__ void __launch_bounds__(256, sizeof(R) == 4 ? 3 : 2) vol_kernel(OpArgsT<R> a) {
+  if (!wait_previous()) return;
   using L = VolSmem<K, R, E>;
   constexpr int N1 = L::N1, NN = L::NN, NQ = L::NQ, N2 = L::N2, NB = L::NB, NT = L::NT, PL = L::PL, LD = L::LD;
   constexpr bool kPoints = MODE != MODE_LINPART;
@@ -231,7 +233,7 @@ int launch_vol(Handle* h, const OpArgsT<R>& a, const OpTune& t, cudaStream_t st)
   if (per_sm < 1) per_sm = 1;
   if (t.vol_per_sm > 0 && per_sm > t.vol_per_sm) per_sm = t.vol_per_sm;
   const int grid = std::min((h->ne + E - 1) / E, h->nsm * per_sm);
-  kern<<<grid, t.vol_threads, smem, st>>>(a);
+  launch(kern, grid, t.vol_threads, smem, st, a);
   DG_LAUNCH_CHECK(h);
   return DG_OK;
 }
