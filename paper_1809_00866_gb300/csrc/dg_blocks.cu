@@ -24,12 +24,6 @@ namespace dg {
 
 namespace {
 
-// value of a stored block entry in the arithmetic type R (blocks may be stored narrower)
-template <class R> __device__ __forceinline__ R wide(float v) { return R(v); }
-template <class R> __device__ __forceinline__ R wide(double v) { return R(v); }
-template <class R> __device__ __forceinline__ R wide(__half v) { return R(__half2float(v)); }
-template <class R> __device__ __forceinline__ R wide(__nv_bfloat16 v) { return R(__bfloat162float(v)); }
-
 // two adjacent stored entries (rows i, i + 1 of one column; i even) as R
 template <class R> __device__ __forceinline__ void wide2(const float* p, R& a, R& b) {
   const float2 v = *reinterpret_cast<const float2*>(p);
@@ -835,6 +829,80 @@ int launch_block_rows(Handle* h, int b, const S* A, const R* v, R alpha, R beta,
   return DG_OK;
 }
 
+// x <- (x_zero ? 0 : x) + alpha D_e^-1 (g - Gx)_e with explicit inverses of b <= 80 (b a multiple of 16 / sizeof(S)
+// and of NC). Bound by the inverses' bytes. A task is 16 bytes of rows of one inverse over a slice of NC
+// columns, all of whose loads are in flight at once and before the residual's slice is there; the
+// slices of a row meet in shared memory and are added in order.
+// Against the ring of bulk copies (staged_jacobi_kernel), whose stages pass through shared memory with a
+// barrier each (us, events included): FP16, b = 80 at 24^3 44 -> 38, at 12^3 10.4 -> 9.2, b = 40 at 12^3
+// 8.3 -> 7.0; FP32, b = 80 at 24^3 65 -> 60, at 12^3 13.9 -> 10.9. Slices of 5 columns instead of 10 are faster for
+// FP16 rows of 40 (32^3: 28.5 against 32.5) and slower for FP32 ones (45 against 41).
+template <int NC, class S>
+__global__ void __launch_bounds__(kRowThreads) inverse_row_kernel(int ne, int b, int epc, const S* __restrict__ A,
+                                                                  const float* __restrict__ g,
+                                                                  const float* __restrict__ Gx, float alpha,
+                                                                  int x_zero, float* __restrict__ x) {
+  if (!wait_previous()) return;
+  constexpr int VW = 16 / sizeof(S);
+  extern __shared__ __align__(16) unsigned char sraw_[];
+  const int rg = b / VW, ns = b / NC, tpe = rg * ns;
+  float* rv = reinterpret_cast<float*>(sraw_);  // [epc][b] g - Gx
+  float* xo = rv + epc * b;                     // [epc][b] the old x
+  float* part = xo + epc * b;                   // [epc][ns][b] partial sums of the slices
+  const int tid = threadIdx.x, nt = blockDim.x, e0 = blockIdx.x * epc, cnt = min(epc, ne - e0);
+  const int el = tid / tpe, r = tid - el * tpe, sl = r / rg, row = VW * (r - sl * rg);
+  const bool on = el < cnt;
+  uint4 raw[NC];
+  if (on) {
+    const S* As = A + ((size_t)(e0 + el) * b + sl * NC) * b + row;
+#pragma unroll
+    for (int c = 0; c < NC; ++c) raw[c] = __ldg(reinterpret_cast<const uint4*>(As + (size_t)c * b));
+  }
+  const size_t v0 = (size_t)e0 * b;
+  for (int t = tid; t < cnt * b; t += nt) {
+    rv[t] = g[v0 + t] - (Gx ? Gx[v0 + t] : 0.0f);
+    xo[t] = x_zero ? 0.0f : x[v0 + t];
+  }
+  __syncthreads();
+  if (on) {
+    const float* re = rv + el * b + sl * NC;
+    float acc[VW];
+#pragma unroll
+    for (int j = 0; j < VW; ++j) acc[j] = 0.0f;
+#pragma unroll
+    for (int c = 0; c < NC; ++c) {
+      float a[VW];
+      widen16(raw[c], A, a);
+      const float xc = re[c];
+#pragma unroll
+      for (int j = 0; j < VW; ++j) acc[j] = fmaf(a[j], xc, acc[j]);
+    }
+    float4* ps = reinterpret_cast<float4*>(part + (el * ns + sl) * b + row);
+#pragma unroll
+    for (int j = 0; j < VW / 4; ++j) ps[j] = make_float4(acc[4 * j], acc[4 * j + 1], acc[4 * j + 2], acc[4 * j + 3]);
+  }
+  __syncthreads();
+  for (int t = tid; t < cnt * b; t += nt) {
+    const int et = t / b, i = t - et * b;
+    float sum = 0.0f;
+    for (int q = 0; q < ns; ++q) sum += part[(et * ns + q) * b + i];
+    x[v0 + t] = xo[t] + alpha * sum;
+  }
+}
+
+template <int NC, class S>
+int launch_inverse_rows(Handle* h, int b, const S* A, const float* g, const float* Gx, float alpha, int x_zero,
+                        float* x, cudaStream_t st) {
+  const int tpe = b / (16 / (int)sizeof(S)) * (b / NC);
+  // as many elements as a CTA takes, but no fewer than two CTAs per SM where there are that many elements
+  const int epc = std::max(1, std::min(kRowThreads / tpe, h->ne / (2 * h->nsm)));
+  const int threads = 32 * ((epc * tpe + 31) / 32), grid = (h->ne + epc - 1) / epc;
+  const size_t smem = sizeof(float) * (size_t)epc * b * (2 + b / NC);
+  launch(inverse_row_kernel<NC, S>, grid, threads, smem, st, h->ne, b, epc, A, g, Gx, alpha, x_zero, x);
+  DG_LAUNCH_CHECK(h);
+  return DG_OK;
+}
+
 constexpr size_t kStageTarget = 96 * 1024;  // bytes of inverses per stage (one buffer)
 constexpr size_t kSmemLimit = 220 * 1024;    // dynamic shared memory a kernel may take
 
@@ -868,6 +936,13 @@ int launch_staged_jacobi(Handle* h, int b, const S* A, const R* g, const R* Gx, 
                          cudaStream_t st) {
   if constexpr (std::is_same<R, float>::value && sizeof(S) == 2) {
     if (b == 140) return launch_pair_jacobi<140, S>(h, A, g, Gx, alpha, x_zero, x, st);
+  }
+  // The blocks of k <= 3 straight from memory (faster at every size, figures at the kernel), unless the ring is
+  // asked for: a cap on its CTAs, or a test of its bounded waits. The ring keeps the FP32 inverses of k = 4.
+  if (h->tune[1].jacobi_max_ctas == 0 && h->dbg.wait_polls <= 0 && !h->dbg.withhold_copy) {
+    if (b == 80) return launch_inverse_rows<10, S>(h, b, A, g, Gx, alpha, x_zero, x, st);
+    if (b == 40) return launch_inverse_rows<sizeof(S) == 2 ? 5 : 10, S>(h, b, A, g, Gx, alpha, x_zero, x, st);
+    if (b == 16) return launch_inverse_rows<8, S>(h, b, A, g, Gx, alpha, x_zero, x, st);
   }
   const size_t per = (size_t)b * b * sizeof(S);
   const size_t target = h->tune[1].jacobi_stage_kb > 0 ? (size_t)h->tune[1].jacobi_stage_kb * 1024 : kStageTarget;
