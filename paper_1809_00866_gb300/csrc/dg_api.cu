@@ -100,9 +100,8 @@ static int build_tables(Handle* h, int k) {
       }
   // d/dxi P_hat_a = sum_{a' < a, a - a' odd} sqrt((2a+1)(2a'+1)) P_hat_a'
   const int W = Tables::kDw;
-  std::vector<int> ri((size_t)3 * nb * W, 0), ci((size_t)3 * nb * W, 0);
-  std::vector<double> rv((size_t)3 * nb * W, 0.0), cv((size_t)3 * nb * W, 0.0);
-  std::vector<int> rc((size_t)3 * nb, 0), cc((size_t)3 * nb, 0);
+  std::vector<int> ci((size_t)3 * nb * W, 0), cc((size_t)3 * nb, 0);
+  std::vector<double> cv((size_t)3 * nb * W, 0.0);
   for (int b = 0; b < 3; ++b)
     for (int n = 0; n < nb; ++n)
       for (int m = 0; m < nb; ++m) {
@@ -112,86 +111,40 @@ static int build_tables(Handle* h, int k) {
         const int an = md[3 * n + b], am = md[3 * m + b];
         if (!same || am >= an || ((an - am) & 1) == 0) continue;
         const double val = std::sqrt((2.0 * an + 1.0) * (2.0 * am + 1.0));
-        int& r = rc[b * nb + m];
         int& c = cc[b * nb + n];
-        if (r >= W || c >= W) return fail(h, DG_ERR_ARG, "derivative table width exceeded");
-        ri[((size_t)b * nb + m) * W + r] = n;
-        rv[((size_t)b * nb + m) * W + r] = val;
-        ++r;
+        if (c >= W) return fail(h, DG_ERR_ARG, "derivative table width exceeded");
         ci[((size_t)b * nb + n) * W + c] = m;
         cv[((size_t)b * nb + n) * W + c] = val;
         ++c;
       }
-  // 1D values, 2D trace modes and the maps between 3D and face modes
+  // traces of the 1D basis, face weights and the map from 3D to face modes
   const int k1 = k + 1;
   T.n2 = k1 * (k + 2) / 2;
-  const int n2 = T.n2;
-  std::vector<double> L1((size_t)k1 * n1), pvv(2 * k1), pdv(2 * k1);
+  std::vector<double> pvv(2 * k1), W2(T.nqf);
   for (int a = 0; a <= k; ++a) {
-    for (int q = 0; q < n1; ++q) L1[(size_t)a * n1 + q] = phat1(a, xg[q]);
     const double na = std::sqrt((2.0 * a + 1.0) * 0.5);
-    const double der = na * a * (a + 1) * 0.5;  // P_a'(1) = a(a+1)/2
     pvv[a] = na;
     pvv[k1 + a] = (a & 1) ? -na : na;
-    pdv[a] = der;
-    pdv[k1 + a] = (a & 1) ? der : -der;  // P_a'(-1) = (-1)^(a+1) a(a+1)/2
   }
-  std::vector<int> pab, pidx((size_t)k1 * k1, -1);
-  for (int t = 0; t <= k; ++t)
-    for (int a = t; a >= 0; --a) {
-      pidx[a * k1 + (t - a)] = (int)(pab.size() / 2);
-      pab.push_back(a);
-      pab.push_back(t - a);
-    }
-  std::vector<double> B2((size_t)T.nqf * n2), W2(T.nqf);
   for (int q1 = 0; q1 < n1; ++q1)
-    for (int q2 = 0; q2 < n1; ++q2) {
-      const int q = q1 * n1 + q2;
-      W2[q] = wg[q1] * wg[q2];
-      for (int j = 0; j < n2; ++j) B2[(size_t)q * n2 + j] = phat1(pab[2 * j], xg[q1]) * phat1(pab[2 * j + 1], xg[q2]);
-    }
-  std::vector<int> M3((size_t)3 * n2 * k1, -1), fmap((size_t)3 * nb), fa((size_t)3 * nb), md3((size_t)nb * 3);
-  for (int m = 0; m < nb; ++m)
-    for (int t = 0; t < 3; ++t) md3[3 * m + t] = md[3 * m + t];
+    for (int q2 = 0; q2 < n1; ++q2) W2[q1 * n1 + q2] = wg[q1] * wg[q2];
+  std::vector<int> fmap((size_t)3 * nb), fa((size_t)3 * nb), md3(md);
   for (int d = 0; d < 3; ++d)
     for (int m = 0; m < nb; ++m) {
-      const int a = md[3 * m + d], b = md[3 * m + (d + 1) % 3], c = md[3 * m + (d + 2) % 3];
-      const int j = pidx[b * k1 + c];
-      fmap[(size_t)d * nb + m] = j;
-      fa[(size_t)d * nb + m] = a;
-      M3[((size_t)d * n2 + j) * k1 + a] = m;
+      const int b = md[3 * m + (d + 1) % 3], c = md[3 * m + (d + 2) % 3];
+      fmap[(size_t)d * nb + m] = (b + c) * (b + c + 1) / 2 + c;  // graded, then the first exponent descending
+      fa[(size_t)d * nb + m] = md[3 * m + d];
     }
-  std::vector<int> d2i((size_t)2 * n2 * W, 0), d2c((size_t)2 * n2, 0);
-  std::vector<double> d2v((size_t)2 * n2 * W, 0.0);
-  for (int dir = 0; dir < 2; ++dir)
-    for (int jo = 0; jo < n2; ++jo)
-      for (int ji = 0; ji < n2; ++ji) {
-        const int bo = pab[2 * jo + dir], co = pab[2 * jo + 1 - dir];
-        const int bi = pab[2 * ji + dir], ci2 = pab[2 * ji + 1 - dir];
-        if (co != ci2 || bo >= bi || ((bi - bo) & 1) == 0) continue;
-        int& r = d2c[dir * n2 + jo];
-        if (r >= W) return fail(h, DG_ERR_ARG, "2D derivative table width exceeded");
-        d2i[((size_t)dir * n2 + jo) * W + r] = ji;
-        d2v[((size_t)dir * n2 + jo) * W + r] = std::sqrt((2.0 * bi + 1.0) * (2.0 * bo + 1.0));
-        ++r;
-      }
   int rcode;
   if ((rcode = upload(h, &T.Bvol, Bv)) || (rcode = upload(h, &T.wvol, wv)) || (rcode = upload(h, &T.xg, xg)) ||
-      (rcode = upload(h, &T.Drow_idx, ri)) || (rcode = upload(h, &T.Drow_val, rv)) ||
       (rcode = upload(h, &T.Dcol_idx, ci)) || (rcode = upload(h, &T.Dcol_val, cv)) ||
-      (rcode = upload(h, &T.L1, L1)) || (rcode = upload(h, &T.B2, B2)) || (rcode = upload(h, &T.W2, W2)) ||
-      (rcode = upload(h, &T.pv, pvv)) || (rcode = upload(h, &T.pd, pdv)) || (rcode = upload(h, &T.M3, M3)) ||
-      (rcode = upload(h, &T.fmap, fmap)) || (rcode = upload(h, &T.fa, fa)) || (rcode = upload(h, &T.md3, md3)) ||
-      (rcode = upload(h, &T.pidx, pidx)) || (rcode = upload(h, &T.pab, pab)) || (rcode = upload(h, &T.D2_idx, d2i)) ||
-      (rcode = upload(h, &T.D2_val, d2v)))
+      (rcode = upload(h, &T.W2, W2)) || (rcode = upload(h, &T.pv, pvv)) || (rcode = upload(h, &T.fmap, fmap)) ||
+      (rcode = upload(h, &T.fa, fa)) || (rcode = upload(h, &T.md3, md3)))
     return rcode;
   auto tof = [](const std::vector<double>& v) { return std::vector<float>(v.begin(), v.end()); };
   TablesF& TF = h->tabf;
-  if ((rcode = upload(h, &TF.Bvol, tof(Bv))) || (rcode = upload(h, &TF.L1, tof(L1))) || (rcode = upload(h, &TF.wvol, tof(wv))) ||
-      (rcode = upload(h, &TF.B2, tof(B2))) || (rcode = upload(h, &TF.W2, tof(W2))) ||
-      (rcode = upload(h, &TF.pv, tof(pvv))) || (rcode = upload(h, &TF.pd, tof(pdv))) ||
-      (rcode = upload(h, &TF.Drow_val, tof(rv))) || (rcode = upload(h, &TF.Dcol_val, tof(cv))) ||
-      (rcode = upload(h, &TF.D2_val, tof(d2v))))
+  if ((rcode = upload(h, &TF.wvol, tof(wv))) || (rcode = upload(h, &TF.W2, tof(W2))) ||
+      (rcode = upload(h, &TF.pv, tof(pvv))) || (rcode = upload(h, &TF.Dcol_val, tof(cv))))
     return rcode;
   return DG_OK;
 }
@@ -241,11 +194,10 @@ static void free_all(Handle* h) {
   h->ev_pool.clear();
   auto F = [](void* p) { if (p) cudaFree(p); };
   Tables& T = h->tab;
-  F(T.Bvol); F(T.wvol); F(T.xg); F(T.Drow_idx); F(T.Drow_val); F(T.Dcol_idx); F(T.Dcol_val);
-  F(T.L1); F(T.B2); F(T.W2); F(T.pv); F(T.pd); F(T.M3); F(T.fmap); F(T.fa); F(T.md3); F(T.pidx); F(T.pab);
-  F(T.D2_idx); F(T.D2_val);
+  F(T.Bvol); F(T.wvol); F(T.xg); F(T.Dcol_idx); F(T.Dcol_val);
+  F(T.W2); F(T.pv); F(T.fmap); F(T.fa); F(T.md3);
   TablesF& TF = h->tabf;
-  F(TF.Bvol); F(TF.L1); F(TF.wvol); F(TF.B2); F(TF.W2); F(TF.pv); F(TF.pd); F(TF.Drow_val); F(TF.Dcol_val); F(TF.D2_val);
+  F(TF.wvol); F(TF.W2); F(TF.pv); F(TF.Dcol_val);
   F(h->face_buf_f); F(h->ubar_f); F(h->dFlux_f);
   F(h->tc_tab[0]); F(h->tc_tab[1]); F(h->ubar_scale);
   for (int d = 0; d < 3; ++d) F(h->dnode[d]);

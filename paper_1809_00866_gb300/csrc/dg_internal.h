@@ -23,43 +23,26 @@ struct Tables {
   double* Bvol = nullptr;   // [nq][nb]          phi_hat at volume points, q = (q0*n1 + q1)*n1 + q2
   double* wvol = nullptr;   // [nq]              reference volume weights
   double* xg = nullptr;     // [n1]              Gauss nodes on [-1,1]
-  double* L1 = nullptr;     // [k+1][n1]         normalised Legendre P_hat_a(x_q)
   // 2D trace modes on a face: pairs (b, c), b + c <= k, b the exponent along the first
   // tangential axis t1 = (d+1)%3 and c along t2 = (d+2)%3; n2 = (k+1)(k+2)/2 of them.
-  double* B2 = nullptr;     // [nqf][n2]         P_hat_b P_hat_c at the face points, q = q1*n1 + q2
   double* W2 = nullptr;     // [nqf]             reference face weights
   double* pv = nullptr;     // [2][k+1]          P_hat_a(+1), P_hat_a(-1)
-  double* pd = nullptr;     // [2][k+1]          P_hat_a'(+1), P_hat_a'(-1)
-  int* M3 = nullptr;        // [3][n2][k+1]      3D mode of (exponent a along d, 2D mode n2) or -1
   int* fmap = nullptr;      // [3][nb]           2D mode of 3D mode m seen from a face normal to d
   int* fa = nullptr;        // [3][nb]           exponent of m along d
   int* md3 = nullptr;       // [nb][3]           exponents of 3D mode m
-  int* pidx = nullptr;      // [(k+1)][(k+1)]    index of the pair (a, b), a + b <= k (the 2D ordering)
-  int* pab = nullptr;       // [n2][2]           the pair (a, b) of a pair index
-  // Sparse reference derivative operator: d/dxi_b phi_hat_n = sum_m D_b[m][n] phi_hat_m.
-  // Drow[b][m][j] / Dcol[b][n][j] hold at most kDw entries (index, value) of row m / column n.
-  int* Drow_idx = nullptr;     // [3][nb][kDw]
-  double* Drow_val = nullptr;  // [3][nb][kDw]
+  // Sparse reference derivative operator: d/dxi_b phi_hat_n = sum_m D_b[m][n] phi_hat_m;
+  // Dcol[b][n][j] holds at most kDw entries (index, value) of column n.
   int* Dcol_idx = nullptr;     // [3][nb][kDw]
   double* Dcol_val = nullptr;  // [3][nb][kDw]
-  // the same for the 2D trace modes along t1 (dir 0) and t2 (dir 1), by rows
-  int* D2_idx = nullptr;       // [2][n2][kDw]
-  double* D2_val = nullptr;    // [2][n2][kDw]
   static constexpr int kDw = 3;
 };
 
 // FP32 copies of the real-valued tables (reduced-precision preconditioner)
 struct TablesF {
-  float* Bvol = nullptr;
-  float* L1 = nullptr;
   float* wvol = nullptr;
-  float* B2 = nullptr;
   float* W2 = nullptr;
   float* pv = nullptr;
-  float* pd = nullptr;
-  float* Drow_val = nullptr;
   float* Dcol_val = nullptr;
-  float* D2_val = nullptr;
 };
 
 struct Level {
