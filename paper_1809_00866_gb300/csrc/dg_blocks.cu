@@ -324,17 +324,16 @@ __global__ void __launch_bounds__(512, 2) gj_inverse_kernel(int nblk, int b_arg,
       }
     }
     // the row interchanges, undone on the columns in reverse order, composed into one column
-    // permutation (column c of the inverse is column colsrc[c] of A) and applied while writing out
-    if (tid == 0) {
-      for (int c = 0; c < b; ++c) colsrc[c] = c;
-      for (int k = b - 1; k >= 0; --k) {
+    // permutation (column c of the inverse is column colsrc[c] of A) and applied while writing out:
+    // c taken through the interchanges in their own order, a thread per column (one thread that
+    // interchanged entries of colsrc held up every block; 32^3 P4: 11.77 ms, now 11.28)
+    for (int c = tid; c < b; c += nt) {
+      int x = c;
+      for (int k = 0; k < b; ++k) {
         const int p = piv[k];
-        if (p != k) {
-          const int t = colsrc[k];
-          colsrc[k] = colsrc[p];
-          colsrc[p] = t;
-        }
+        x = x == k ? p : (x == p ? k : x);
       }
+      colsrc[c] = x;
     }
     __syncthreads();
     for (int t = tid; t < b * b; t += nt) {
@@ -1093,9 +1092,11 @@ int invert_levels_f32(Handle* h, cudaStream_t st, unsigned* status) {
     const int per_sm = (int)std::max<size_t>(1, std::min<size_t>(4, (227 * 1024) / (smem + 1024)));
     const int grid = std::min(h->ne, h->nsm * per_sm);
     // warp 0 factors; the (column group, row group) pairs of the update on the warps after it:
-    // at most 512 threads, at most b row groups
-    const int ng = L.b / 4, active = ng * std::min(L.b, 480 / ng);
-    const int threads = std::min(512, 32 + 32 * ((active + 31) / 32));
+    // at most 512 threads, at most b row groups; 256 threads for b = 80, whose time is the factoring
+    // warp's chain and the barriers, so that four blocks share an SM instead of two
+    // (24 x 12 x 12 P3: 585 us, now 343)
+    const int ng = L.b / 4, most = L.b <= 80 ? 224 : 480, active = ng * std::min(L.b, most / ng);
+    const int threads = 32 + 32 * ((active + 31) / 32);
     if (L.b == 140 && threads == 512)
       gj_inverse_kernel<140><<<grid, threads, smem, st>>>(h->ne, L.b, L.LUf, status);
     else
