@@ -41,34 +41,36 @@ import synthetic as S  # noqa: E402
 METRIC = "Jv GDOF/s and s per implicit stage to rel-res 1e-8: chosen form vs plain FP64"
 CONFIG = "tgv32_p4"
 RTOL = 1e-8
-def jv_flops(k, sum_factorised=True):
+def pencil_ops(length, n):
+    """Operations (multiply-adds or additions) that take `length` plain Legendre coefficients to the n Gauss
+    nodes through their even and odd parts (L_0 = 1), or, transposed, n point values to coefficients."""
+    even, odd = (length + 1) // 2 - 1, length // 2
+    return (n // 2) * (even + odd + (2 if length > 1 else 0)) + (n % 2) * even
+
+
+def jv_flops(k):
     """Algorithmic work (FLOP) of the exact Jacobian action per element, as the kernels compute it.
 
-    Counted from the formulation (FMA = 2 FLOP; index arithmetic excluded):
-    face pass, per face (3 per element): 2D traces 2*7*N_b, point values of the
-    4 variables on both sides, linearised Riemann flux 32*N_qf, projection of the
-    4 flux components, 2D viscous flux and lifting ~24*N_2. The FP64 pass takes the
-    point values and the projection by sum factorisation over the face's two axes,
-    8*n*(N_2 + N_qf) and 4*n*(N_qf + N_2); the FP32 pass densely, 8*N_qf*N_2 and
-    4*N_qf*N_2 (sum_factorised=False).
-    volume pass: corrected gradients 9*N_b*2, sum-factorised interpolation of 3
-    fields 3*(N_b*n + N_2*n^2 + (k+1)*n^3), 6 products per point, sum-factorised
-    projection of 6 fields 6*((k+1)*n^3 + N_2*n^2 + N_b*n), the viscous flux and
-    the sparse modal derivatives ~30*N_b.
+    Counted from the formulation in plain Legendre coefficients; an addition holds the FP64 pipe as
+    long as a multiply-add, so each counts 2 FLOP (index arithmetic excluded):
+    face pass, per face (3 per element): traces of value and normal derivative 14 N_b, point values
+    of 4 variables on both sides by sum factorisation, the linearised Riemann flux from its 16 stored
+    values 22 N_qf, projection of 4 fluxes, viscous flux and lifting 24 N_2.
+    volume pass: corrected gradients and viscous flux 42 N_b(k-1), sum-factorised interpolation of 3
+    fields, 6 products 9 N_q, projection of 6 fields onto degree k - 1, modal derivatives with the
+    face terms, mass shift and scaling 43 N_b.
     Returns (face FLOP per element, volume FLOP per element).
     """
     n = k + 1
-    nb = (k + 1) * (k + 2) * (k + 3) // 6
-    n2 = (k + 1) * (k + 2) // 2
-    nqf, nq = n * n, n ** 3
-    if sum_factorised:
-        points, proj = 8 * n * (n2 + nqf), 4 * n * (nqf + n2)
-    else:
-        points, proj = 8 * nqf * n2, 4 * nqf * n2
-    face = 3 * 2 * (2 * 7 * nb + points + 32 * nqf + proj + 24 * n2)
-    vol = 2 * (9 * nb * 2 + 3 * (nb * n + n2 * n * n + (k + 1) * nq) + 6 * nq
-               + 6 * ((k + 1) * nq + n2 * n * n + nb * n) + 30 * nb)
-    return float(face), float(vol)
+    nb, nbm = n * (n + 1) * (n + 2) // 6, k * (k + 1) * (k + 2) // 6
+    n2 = n * (n + 1) // 2
+    ops = [pencil_ops(m, n) for m in range(n + 1)]
+    triangle = [sum(ops[1:m + 1]) + n * ops[m] for m in range(n + 1)]  # m (m + 1) / 2 coefficients <-> n^2 points
+    face = 3 * (14 * nb + 12 * triangle[n] + 22 * n * n + 24 * n2)
+    interp = sum(triangle[1:]) + n * n * ops[n]
+    project = n * n * ops[k] + n * sum(ops[1:k + 1]) + sum((g + 1) * ops[k - g] for g in range(k))
+    vol = 42 * nbm + 3 * interp + 9 * n ** 3 + 6 * project + 43 * nb
+    return 2.0 * face, 2.0 * vol
 
 
 # The dense-quadrature formulation (every contraction with the full N_q x N_b tables) needs
@@ -86,9 +88,8 @@ HBM_FALLBACK_GBS = 6800.0
 # One-pass captures (dram__bytes_read.sum + dram__bytes_write.sum) of the chosen stage at 32^3 P4
 # (FP16 blocks, 5/5/2 sweeps): the fine-level block-Jacobi apply moves 1.320 GB per sweep from
 # zero and 1.357 GB per sweep with G x, one and nine of a cycle's ten fine-level sweeps, 1.353 GB
-# per launch on average; the tensor-core volume pass 173.6 MB. (The FP64 face and volume passes
-# changed after their capture.)
-NCU_TRAFFIC = {("bj32_fine", 32, "half"): 1.353e9, ("vol_tc32", 32, "half"): 1.736e8}
+# per launch on average. (The operator passes changed after their capture.)
+NCU_TRAFFIC = {("bj32_fine", 32, "half"): 1.353e9}
 
 
 def measured_peaks():
@@ -876,11 +877,11 @@ def run_ours(args):
             if by > 0:
                 kernels[nm]["gbs"] = by / (ms_k / 1e3) / 1e9
     storage = {"fp32": "float", "h16": "half", "bf16": "bfloat16", "h16tc": "half", "bf16tc": "bfloat16"}.get(args.form)
-    names = {"bj32_fine": "staged_jacobi_kernel<float, %s> (fine level)" % storage,
+    names = {"bj32_fine": "%s<%s> (fine level)" % ("inverse_row_kernel" if k <= 3 else "staged_jacobi_kernel"
+                                                  if storage == "float" else "pair_jacobi_kernel", storage),
              "bj64_fine": "bj_update_kernel<double> (fine level)",
-             "bsr32_l1": ("direct_apply_kernel<float, 7, float> (P2 level)" if args.form == "fp32" else
-                          "direct7_vec_kernel<%s> (P2 level)" % storage),
-             "bsr64_l1": "direct_apply_kernel<double, 7, double> (P2 level)",
+             "bsr32_l1": "block_row_kernel<float, %s> (P2 level)" % storage,
+             "bsr64_l1": "block_row_kernel<double, double> (P2 level)",
              "face_tan32": "face_kernel<%d, tangent, float>" % k, "vol_tan32": "vol_kernel<%d, tangent, float>" % k,
              "vol_tc32": "tc_vol_kernel<%d, %s> (tcgen05)" % (k, "bf16" if args.form == "bf16tc" else "f16"),
              "face_tan": "face_kernel<%d, tangent, double>" % k, "vol_tan": "vol_kernel<%d, tangent, double>" % k}
@@ -911,7 +912,7 @@ def run_ours(args):
                    "frac_of_read_stream": ach / hbm_read if hbm_read else None}
         else:
             f32 = nm.endswith("32")
-            flop = ((jv_flops(k, sum_factorised=False)[0] if f32 else ff) if nm.startswith("face") else fv) * dg.ne
+            flop = (ff if nm.startswith("face") else fv) * dg.ne
             peak = fp32_peak if f32 else fp64_peak
             ach = flop / t / 1e12
             ent = {"bound": "alu", "achieved": ach, "peak": peak, "unit": "TFLOP/s", "frac": ach / peak,

@@ -488,8 +488,10 @@ typedef struct dg_tuning {
   int vol_threads;       /* threads per CTA of the volume pass: 64, 128, 160, 192 or 256 (128) */
   int face_ctas_per_sm;  /* cap on resident CTAs per SM of the face pass, 0..32 (0: shared memory decides) */
   int vol_ctas_per_sm;   /* the same for the volume pass */
-  int jacobi_stage_kb;   /* FP32 cycle: KB of element inverses per bulk-copy stage of the fine-level
-                            block-Jacobi apply, 8..224 (96); capped by shared memory */
+  int jacobi_stage_kb;   /* FP32 cycle: KB of element inverses per bulk-copy stage of the block-Jacobi
+                            apply by the ring (FP32 blocks of k = 4, and every block under a cap, next
+                            field; without one the blocks of k <= 3 are read straight from memory),
+                            8..224 (96); capped by shared memory */
   int jacobi_max_ctas;   /* cap on the CTAs of that apply, 0..4096 (0: no cap, one wave of the GPU). A
                             small cap makes every CTA take many stages through its ring of stage
                             buffers (the stage size then also shrinks to keep >= 2 stages per CTA);
