@@ -452,8 +452,8 @@ int tc_prepare_lin(Handle* h, cudaStream_t st) {
   return DG_OK;
 }
 
-// Volume pass of the FP32 Jacobian action on the tensor cores; the face pass (face_out_f,
-// face_lift_f) has run. tc = 1: FP16 operands, tc = 2: BF16 operands.
+// Volume pass of the FP32 Jacobian action on the tensor cores; the face pass has run (its
+// records are in face_buf_f). tc = 1: FP16 operands, tc = 2: BF16 operands.
 int tc_volume_tangent(Handle* h, const float* in, float* out, int tc, cudaStream_t st) {
   if (!h->tc_tab[0] || !h->ubar_scale) return fail(h, DG_ERR_STATE, "tensor-core tables not prepared");
   const int bf = tc == 2 ? 1 : 0;
