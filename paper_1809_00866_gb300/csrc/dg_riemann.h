@@ -106,16 +106,20 @@ __device__ __forceinline__ float ac_star_f(float ul, float ur, float dp, int max
 }
 
 // Tangential-velocity ratio u_t(star)/u_t(v) across the 1-wave and its derivatives in u and v.
-// Rarefaction: u_t (u + a) invariant, and 1/(u + a) = a - u; shock: s [u_t] = [u_n u_t].
+// Rarefaction: u_t w(u) invariant, w(x) = x + a = 1/(a - x), each w from the form whose terms have one sign
+// (the other loses (u/c)^2 units of roundoff to cancellation; u is positive, or zero up to the band of a
+// tie, where the side's ratio is used); shock: s [u_t] = [u_n u_t].
 __device__ __forceinline__ void ac_tangential(const AcWave& k, double u, double a, double ia, double v, double av,
                                               double iav, double& t, double& tu, double& tv) {
-  if (u < v) {
-    const double r = 1.0 / (1.0 + k.x), f = 2.0 * k.iq * r * r;
-    t = (1.0 - k.x) * r;
+  const bool shock = u < v;
+  const double w = u + a, m = av + fabs(v);  // w(v), or its inverse where v < 0
+  const double r = 1.0 / (shock ? 1.0 + k.x : (v >= 0.0 ? w : m * w));
+  t = (shock ? 1.0 - k.x : (v >= 0.0 ? m : 1.0)) * r;
+  if (shock) {
+    const double f = 2.0 * k.iq * r * r;
     tu = f * (k.kap * k.x - 1.0);
     tv = f * (k.kap * k.x + 1.0);
   } else {
-    t = (v + av) * (a - u);
     tu = -t * ia;
     tv = t * iav;
   }
@@ -164,17 +168,25 @@ __device__ __forceinline__ void ac_riemann(double unl, double t1l, double t2l, d
   const AcWave k1 = ac_wave(us, a, ia, ul, al), k3 = ac_wave(-us, a, ia, -ur, ar);
   const double band = 1e-12 * scale;
   const bool tie = us >= -band && us <= band;
-  const double wl = tie ? 0.5 : (us > 0.0 ? 1.0 : 0.0), wr = 1.0 - wl;  // weights of the sides' tangential values
-  // wl tau_L and its derivatives, wr tau_R and its derivatives
+  // weighted ratios of the left and right side and their derivatives: one evaluation for the side that the contact
+  // comes from, whichever it is in a lane (one per side took every warp through both), a second in a tie
   double tl = 0.0, tlu = 0.0, tlv = 0.0, tr = 0.0, tru = 0.0, trv = 0.0;
-  if (wl > 0.0) {
-    ac_tangential(k1, us, a, ia, ul, al, ial, tl, tlu, tlv);
-    tl *= wl; tlu *= wl; tlv *= wl;
-  }
-  if (!(wl >= 1.0)) {
-    ac_tangential(k3, -us, a, ia, -ur, ar, iar, tr, tru, trv);
-    tr *= wr; tru *= -wr; trv *= -wr;
-  }
+  auto side = [&](bool left, double weight) {
+    double t, tu, tv;
+    AcWave k;
+    k.x = left ? k1.x : k3.x;
+    k.kap = left ? k1.kap : k3.kap;
+    k.iq = left ? k1.iq : k3.iq;
+    ac_tangential(k, left ? us : -us, a, ia, left ? ul : -ur, left ? al : ar, left ? ial : iar, t, tu, tv);
+    if (left) {
+      tl = weight * t; tlu = weight * tu; tlv = weight * tv;
+    } else {
+      tr = weight * t; tru = -weight * tu; trv = -weight * tv;
+    }
+  };
+  const bool left = us > 0.0;
+  side(left, tie ? 0.5 : 1.0);
+  if (tie) side(!left, 0.5);
   F[0] = c2 * (us * us + k1.p) + pL;
   F[3] = c * us;
   const double T1 = tl * t1l + tr * t1r, T2 = tl * t2l + tr * t2r;
