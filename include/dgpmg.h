@@ -489,9 +489,10 @@ typedef struct dg_tuning {
   int face_ctas_per_sm;  /* cap on resident CTAs per SM of the face pass, 0..32 (0: shared memory decides) */
   int vol_ctas_per_sm;   /* the same for the volume pass */
   int jacobi_stage_kb;   /* FP32 cycle: KB of element inverses per bulk-copy stage of the block-Jacobi
-                            apply by the ring (FP32 blocks of k = 4, and every block under a cap, next
-                            field; without one the blocks of k <= 3 are read straight from memory),
-                            8..224 (96); capped by shared memory */
+                            apply by the ring, 8..224 (96); capped by shared memory. The ring takes the
+                            FP32 blocks of k = 4, and those of k <= 3 under a cap (next field); without
+                            one these are read straight from memory. 16-bit blocks of k = 4 always take one
+                            element per stage. */
   int jacobi_max_ctas;   /* cap on the CTAs of that apply, 0..4096 (0: no cap, one wave of the GPU). A
                             small cap makes every CTA take many stages through its ring of stage
                             buffers (the stage size then also shrinks to keep >= 2 stages per CTA);
@@ -507,10 +508,11 @@ int dg_set_tuning(dg_handle* h, int which, const dg_tuning* t);
 /* Measure the candidate shapes on h (CUDA events around the real kernels at h's current
  * linearisation; for DG_TUNE_FP32 the block-Jacobi stages too when an FP32 assembly exists) and
  * keep the fastest per kernel. The candidates: face_warps 2/4/8; vol_threads 64/128/160/192/256 with no
- * CTA cap and with 4 CTAs per SM; jacobi_stage_kb 48/96/144/200. use_cache != 0: reuse the result
- * of an earlier call in this process on the same (which, k, N_q, SM count, log2 N_e, block
- * storage). report: NULL or HOST [6] = device ms per launch of the default and of the chosen face
- * pass, volume pass and block-Jacobi apply (0 where not measured or taken from the cache).
+ * CTA cap and with 4 CTAs per SM; jacobi_stage_kb 48/96/144/200 where the fine level's apply reads
+ * it, else it stays as set and the apply is timed once. use_cache != 0: reuse the result of an
+ * earlier call in this process on the same (which, k, N_q, SM count, log2 N_e, block storage,
+ * jacobi_max_ctas). report: NULL or HOST [6] = device ms per launch of the default and of the
+ * chosen face pass, volume pass and block-Jacobi apply (0 where not measured or taken from the cache).
  * Overwrites the level-0 work vectors; keeps the profiler's accumulated counts. Synchronises. */
 int dg_autotune(dg_handle* h, int which, int use_cache, double* report, void* stream);
 

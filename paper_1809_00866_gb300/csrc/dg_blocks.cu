@@ -930,18 +930,23 @@ int launch_pair_jacobi(Handle* h, const S* A, const float* g, const float* Gx, f
   return DG_OK;
 }
 
+// The blocks of k <= 3 straight from memory (figures at inverse_row_kernel), unless the ring is asked for: a cap
+// on its CTAs, or a test of its bounded waits. The ring keeps the FP32 inverses of k = 4.
+bool rows_from_memory(const Handle* h, int b) {
+  return (b == 80 || b == 40 || b == 16) && h->tune[1].jacobi_max_ctas == 0 && h->dbg.wait_polls <= 0 &&
+         !h->dbg.withhold_copy;
+}
+
 template <class R, class S>
 int launch_staged_jacobi(Handle* h, int b, const S* A, const R* g, const R* Gx, R alpha, int x_zero, R* x,
                          cudaStream_t st) {
   if constexpr (std::is_same<R, float>::value && sizeof(S) == 2) {
     if (b == 140) return launch_pair_jacobi<140, S>(h, A, g, Gx, alpha, x_zero, x, st);
   }
-  // The blocks of k <= 3 straight from memory (faster at every size, figures at the kernel), unless the ring is
-  // asked for: a cap on its CTAs, or a test of its bounded waits. The ring keeps the FP32 inverses of k = 4.
-  if (h->tune[1].jacobi_max_ctas == 0 && h->dbg.wait_polls <= 0 && !h->dbg.withhold_copy) {
+  if (rows_from_memory(h, b)) {
     if (b == 80) return launch_inverse_rows<10, S>(h, b, A, g, Gx, alpha, x_zero, x, st);
     if (b == 40) return launch_inverse_rows<sizeof(S) == 2 ? 5 : 10, S>(h, b, A, g, Gx, alpha, x_zero, x, st);
-    if (b == 16) return launch_inverse_rows<8, S>(h, b, A, g, Gx, alpha, x_zero, x, st);
+    return launch_inverse_rows<8, S>(h, b, A, g, Gx, alpha, x_zero, x, st);
   }
   const size_t per = (size_t)b * b * sizeof(S);
   const size_t target = h->tune[1].jacobi_stage_kb > 0 ? (size_t)h->tune[1].jacobi_stage_kb * 1024 : kStageTarget;
@@ -1011,6 +1016,12 @@ int prepare_blocks16(Handle* h, int storage, cudaStream_t st) {
   }
   h->asm16 = storage;
   return DG_OK;
+}
+
+bool jacobi_reads_stage_kb(const Handle* h, int storage) {
+  const int b = h->lev[0].b;
+  const bool pair = b == 140 && storage != DG_PRECOND_FP32;  // one element per stage
+  return !pair && !rows_from_memory(h, b);
 }
 
 int staged_jacobi_f(Handle* h, int lvl, const float* g, const float* Gx, float omega, bool x_zero, float* x,

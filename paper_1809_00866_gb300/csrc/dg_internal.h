@@ -315,6 +315,8 @@ int level_matvec(Handle* h, int lvl, const double* x, double* y, cudaStream_t st
 // explicit inverses in Level::LUf (invert_levels_f32 turns the FP32 blocks held there into them).
 // status: the word the singular-block flags go to (the assembly's own word, or the handle's)
 int invert_levels_f32(Handle* h, cudaStream_t st, unsigned* status);
+// whether the fine level's apply stages elements by OpTune::jacobi_stage_kb (storage: a DG_PRECOND_FP32* value)
+bool jacobi_reads_stage_kb(const Handle* h, int storage);
 int staged_jacobi_f(Handle* h, int lvl, const float* g, const float* Gx, float omega, bool x_zero, float* x,
                     int storage, cudaStream_t st);  // x <- (x_zero ? 0 : x) + omega D^-1 (g - Gx); Gx may be null
 int prepare_blocks16(Handle* h, int storage, cudaStream_t st);  // LUf, Bsrf -> 16-bit copies

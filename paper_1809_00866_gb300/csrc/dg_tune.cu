@@ -1,11 +1,12 @@
 // Launch-shape tuning of the hot kernels per (degree k, quadrature size N_q): the warps per CTA
-// of the face pass, the threads per CTA of the volume pass, the CTAs per SM of both, and the
-// element blocks staged per bulk copy of the FP32 block-Jacobi apply. The paper's CPU code has no
-// counterpart; on a GPU the best shapes depend on k (the shared-memory footprint of a face or an
-// element grows with N_b and N_q) and on the mesh size (grid fill), so they are measured on the
-// handle itself: every candidate runs the real kernels on the handle's current linearisation and
-// the fastest per kernel is kept. Results are cached per (precision, k, N_q, SM count, log2 N_e)
-// for the process, so handles of the same shape (a batch of boxes) tune once.
+// of the face pass, the threads per CTA of the volume pass, the CTAs per SM of both, and, where the
+// fine level's FP32 block-Jacobi apply reads it, the element blocks staged per bulk copy. The
+// paper's CPU code has no counterpart; on a GPU the best shapes depend on k (the shared-memory
+// footprint of a face or an element grows with N_b and N_q) and on the mesh size (grid fill), so
+// they are measured on the handle itself: every candidate runs the real kernels on the handle's
+// current linearisation and the fastest per kernel is kept. Results are cached per (precision, k,
+// N_q, SM count, log2 N_e, block storage, CTA cap of the block-Jacobi apply) for the process, so
+// handles of the same shape (a batch of boxes) tune once.
 #include <cmath>
 #include <map>
 #include <mutex>
@@ -22,7 +23,8 @@ __global__ void tune_fill_kernel(long long n, R* x, double phase) {
     x[i] = R(sin(0.37 * (double)i + phase) * 0.01);
 }
 
-using TuneKey = std::tuple<int, int, int, int, int, int>;  // precision, k, N_q, SMs, log2 N_e, block storage
+// precision, k, N_q, SMs, log2 N_e, block storage, CTA cap of the block-Jacobi apply
+using TuneKey = std::tuple<int, int, int, int, int, int, int>;
 static std::map<TuneKey, OpTune> g_tune_cache;
 static std::mutex g_tune_mu;
 
@@ -84,12 +86,15 @@ static int time_classes(Handle* hh, F fn, int reps, double* ms, cudaStream_t st)
 static int autotune(Handle* h, int which, bool use_cache, double* report, cudaStream_t st) {
   const bool f32 = which == DG_TUNE_FP32;
   const int storage = f32 ? (h->asm16 ? h->asm16 : (h->asm_f_ready ? DG_PRECOND_FP32 : 0)) : 0;
-  const TuneKey key{which, h->tab.k, h->tab.nq, h->nsm, ilog2(h->ne), storage};
+  const bool stages = f32 && storage && jacobi_reads_stage_kb(h, storage);
+  const TuneKey key{which, h->tab.k, h->tab.nq, h->nsm, ilog2(h->ne), storage, h->tune[which].jacobi_max_ctas};
   if (use_cache) {
     std::lock_guard<std::mutex> lk(g_tune_mu);
     auto it = g_tune_cache.find(key);
     if (it != g_tune_cache.end()) {
+      const int kb = h->tune[which].jacobi_stage_kb;
       h->tune[which] = it->second;
+      if (!stages) h->tune[which].jacobi_stage_kb = kb;  // as set
       if (report)
         for (int i = 0; i < 6; ++i) report[i] = 0.0;
       return DG_OK;
@@ -143,22 +148,24 @@ static int autotune(Handle* h, int which, bool use_cache, double* report, cudaSt
       if (t.face_warps == 4 && i < 3) def_f = ms[cf];
       if (t.vol_threads == 128 && t.vol_per_sm == 0) def_v = ms[cv];
     }
-    // the FP32 block-Jacobi apply on the fine level, with the blocks the cycle will use
+    // the FP32 block-Jacobi apply on the fine level, with the blocks the cycle will use: the stage sizes
+    // where it reads them, else once with the field as it is set
     if (f32 && storage) {
       const int kb[4] = {48, 96, 144, 200};
       double bj = 1e30;
       tune_fill_kernel<float><<<h->nsm * 4, 256, 0, st>>>(n0, yf, 0.2);
       DG_LAUNCH_CHECK(h);
-      for (int i = 0; i < 4; ++i) {
+      for (int i = 0; i < (stages ? 4 : 1); ++i) {
+        const int size = stages ? kb[i] : base.jacobi_stage_kb;
         h->tune[which] = best;
-        h->tune[which].jacobi_stage_kb = kb[i];
+        h->tune[which].jacobi_stage_kb = size;
         auto sweep = [&]() -> int {
           const int q = staged_jacobi_f(h, 0, xf, yf, 0.9f, false, zf, storage, st);
           return q < 0 ? fail(h, DG_ERR_ARG, "element block unsuited to the staged apply") : q;
         };
         if ((r = time_classes(h, sweep, 5, ms, st))) return r;
-        if (kb[i] == base.jacobi_stage_kb) def_j = ms[DG_PROF_BJ32];
-        if (ms[DG_PROF_BJ32] < bj) { bj = ms[DG_PROF_BJ32]; best.jacobi_stage_kb = kb[i]; }
+        if (size == base.jacobi_stage_kb) def_j = ms[DG_PROF_BJ32];
+        if (ms[DG_PROF_BJ32] < bj) { bj = ms[DG_PROF_BJ32]; best.jacobi_stage_kb = size; }
       }
       best_j = bj;
     }
