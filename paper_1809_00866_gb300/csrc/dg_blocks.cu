@@ -818,7 +818,8 @@ __global__ void __launch_bounds__(kRowThreads, sizeof(S) == 2 ? 4 : 3) block_row
 template <class R, class S>
 int launch_block_rows(Handle* h, int b, const S* A, const R* v, R alpha, R beta, R* y, cudaStream_t st) {
   const int tpe = 7 * (b / (16 / (int)sizeof(S)));
-  if (b % 8 != 0 || tpe > kRowThreads) return -1;  // -1, not a DG_ code: unsuited, the caller's general path
+  // the levels below the finest have degrees 1..3, b = 16, 40 or 80: all of them fit (80 in FP64: 280 tasks)
+  if (b % 8 != 0 || tpe > kRowThreads) return fail(h, DG_ERR_ARG, "block size unsuited to the block-sparse product");
   const int epc = kRowThreads / tpe;
   const int threads = 32 * ((epc * tpe + 31) / 32);
   const size_t smem = sizeof(R) * (size_t)epc * 14 * b;  // slices of v and partial sums

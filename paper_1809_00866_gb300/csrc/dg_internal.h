@@ -322,7 +322,7 @@ int staged_jacobi_f(Handle* h, int lvl, const float* g, const float* Gx, float o
 int prepare_blocks16(Handle* h, int storage, cudaStream_t st);  // LUf, Bsrf -> 16-bit copies
 int bsr16_f(Handle* h, int lvl, int storage, float alpha, const float* x, float beta, float* y, cudaStream_t st);
 template <class R>
-int staged_bsr(Handle* h, int lvl, const R* B, R alpha, const R* x, R beta, R* y, cudaStream_t st);  // -1: n/a
+int staged_bsr(Handle* h, int lvl, const R* B, R alpha, const R* x, R beta, R* y, cudaStream_t st);
 
 // the preconditioner as the batched solver uses it (dg_solvers.cu)
 int solve_opts_check(Handle* h, const dg_solve_opts* o);

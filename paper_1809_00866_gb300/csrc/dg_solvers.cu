@@ -111,31 +111,6 @@ __global__ void prolong_add_kernel(int ne, int nbf, int nbc, const R* xc, R* xf)
 }
 
 // ------------------------------------------------------- block operations
-// y[e] = alpha * sum_s B[e][s] x[nbr(e,s)] + beta * y[e]; slot 0 is the element itself.
-template <class R>
-__global__ void __launch_bounds__(128) bsr_kernel(int ne, int b, const int* nbr, const R* B, R alpha,
-                                                  const R* x, R beta, R* y) {
-  if (!wait_previous()) return;
-  extern __shared__ __align__(16) unsigned char sraw_[];
-  R* sx = reinterpret_cast<R*>(sraw_);  // [7][b]
-  for (int e = blockIdx.x; e < ne; e += gridDim.x) {
-    for (int t = threadIdx.x; t < 7 * b; t += blockDim.x) {
-      const int s = t / b, c = t - s * b;
-      const int col = s == 0 ? e : nbr[e * 6 + s - 1];
-      sx[t] = col >= 0 ? x[(size_t)col * b + c] : R(0);  // no neighbour across a wall (zero block)
-    }
-    __syncthreads();
-    for (int r = threadIdx.x; r < b; r += blockDim.x) {
-      R acc = R(0);
-      const R* Be = B + (size_t)e * 7 * b * b;
-      for (int s = 0; s < 7; ++s)
-        for (int c = 0; c < b; ++c) acc += Be[((size_t)s * b + c) * b + r] * sx[s * b + c];
-      y[(size_t)e * b + r] = alpha * acc + (beta == R(0) ? R(0) : beta * y[(size_t)e * b + r]);
-    }
-    __syncthreads();
-  }
-}
-
 // y[e] = alpha * (G^T x)[e] + beta * y[e]: the blocks of column e are B[e][0] and, for each face
 // slot s of e, B[nbr(e,s)][opposite(s)] (the neighbour's block pointing back across that face).
 template <class R>
@@ -295,13 +270,7 @@ static int apply_block_inverse(Handle* h, const Level& L, const double* g, const
 }
 
 static int run_bsr(Handle* h, int lvl, double alpha, const double* x, double beta, double* y, cudaStream_t st) {
-  const Level& L = h->lev[lvl];
-  const int rc = staged_bsr<double>(h, lvl, L.Bsr, alpha, x, beta, y, st);
-  if (rc >= 0) return rc;  // -1: the blocks do not fit the staged kernel
-  launch(bsr_kernel<double>, grid_for(h, h->ne), 128, sizeof(double) * 7 * L.b, st, h->ne, L.b, h->nbr, L.Bsr, alpha,
-         x, beta, y);
-  DG_LAUNCH_CHECK(h);
-  return DG_OK;
+  return staged_bsr<double>(h, lvl, h->lev[lvl].Bsr, alpha, x, beta, y, st);
 }
 
 int level_matvec(Handle* h, int lvl, const double* x, double* y, cudaStream_t st) {
@@ -667,19 +636,9 @@ static bool is16(int precision) {
 // whether the fine level's volume contractions run on the tensor cores
 static int level_matvec_f(Handle* h, int lvl, const float* x, float* y, int precision, cudaStream_t st) {
   if (lvl == 0) return op_tangent_f32(h, x, y, tc_of(precision), st);
-  const Level& L = h->lev[lvl];
   const int storage = storage_of(precision);
-  if (is16(storage)) {
-    const int r16 = bsr16_f(h, lvl, storage, 1.0f, x, 0.0f, y, st);
-    if (r16 >= 0) return r16;
-    return fail(h, DG_ERR_ARG, "block size unsuited to the 16-bit block-sparse product");
-  }
-  const int rc = staged_bsr<float>(h, lvl, L.Bsrf, 1.0f, x, 0.0f, y, st);
-  if (rc >= 0) return rc;
-  launch(bsr_kernel<float>, grid_for(h, h->ne), 128, sizeof(float) * 7 * L.b, st, h->ne, L.b, h->nbr, L.Bsrf, 1.0f, x,
-         0.0f, y);
-  DG_LAUNCH_CHECK(h);
-  return DG_OK;
+  if (is16(storage)) return bsr16_f(h, lvl, storage, 1.0f, x, 0.0f, y, st);
+  return staged_bsr<float>(h, lvl, h->lev[lvl].Bsrf, 1.0f, x, 0.0f, y, st);
 }
 
 static int jacobi_sweeps_f(Handle* h, int lvl, const float* g, float* x, int sweeps, float omega, bool x_zero,
