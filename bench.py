@@ -41,35 +41,61 @@ import synthetic as S  # noqa: E402
 METRIC = "Jv GDOF/s and s per implicit stage to rel-res 1e-8: chosen form vs plain FP64"
 CONFIG = "tgv32_p4"
 RTOL = 1e-8
-def pencil_ops(length, n):
-    """Operations (multiply-adds or additions) that take `length` plain Legendre coefficients to the n Gauss
-    nodes through their even and odd parts (L_0 = 1), or, transposed, n point values to coefficients."""
+
+
+def interp_ops(length, n):
+    """Operations (multiply-adds, products or additions) that take `length` plain Legendre coefficients to
+    the n Gauss nodes through their even and odd parts (L_0 = 1)."""
     even, odd = (length + 1) // 2 - 1, length // 2
-    return (n // 2) * (even + odd + (2 if length > 1 else 0)) + (n % 2) * even
+    return (n // 2) * (even + (2 if odd == 1 else odd + 2 if odd else 0)) + (n % 2) * even
+
+
+def project_ops(length, n):
+    """The same for n point values to `length` coefficients, each pair's sum and difference first."""
+    even, odd = (length + 1) // 2, length // 2
+    return (n // 2) * ((2 if odd else 1) + even + odd) + (n % 2) * even
+
+
+def divergence_ops(k):
+    """Per equation and element: modal derivatives and face terms. The faces' sums are shared by the modes of
+    one pencil with the same parity, within each of the three z-exponent classes that a thread takes."""
+    modes = [(a, b, g - a - b) for g in range(k + 1) for a in range(g + 1) for b in range(g - a + 1)]
+    shared = {(min(m[2], 2), d, m[d - 2], m[d - 1], m[d] % 2) for m in modes for d in range(3)}
+    own = sum(1 + (m[d] >= 1) + (m[d] >= 3) for m in modes for d in range(3)) - sum(m[0] == 0 for m in modes)
+    return 2 * len(shared) + own
 
 
 def jv_flops(k):
-    """Algorithmic work (FLOP) of the exact Jacobian action per element, as the kernels compute it.
+    """Work (FLOP) of the exact Jacobian action per element, as the kernels do it.
 
-    Counted from the formulation in plain Legendre coefficients; an addition holds the FP64 pipe as
-    long as a multiply-add, so each counts 2 FLOP (index arithmetic excluded):
-    face pass, per face (3 per element): traces of value and normal derivative 14 N_b, point values
-    of 4 variables on both sides by sum factorisation, the linearised Riemann flux from its 16 stored
-    values 22 N_qf, projection of 4 fluxes, viscous flux and lifting 24 N_2.
-    volume pass: corrected gradients and viscous flux 42 N_b(k-1), sum-factorised interpolation of 3
-    fields, 6 products 9 N_q, projection of 6 fields onto degree k - 1, modal derivatives with the
-    face terms, mass shift and scaling 43 N_b.
+    An addition or product holds the FP64 pipe as long as a multiply-add, so each operation counts 2 FLOP
+    (index arithmetic excluded). Counted phase by phase:
+    face pass, per face (3 per element): traces of 4 variables on both sides with their scaling, jumps, sums
+    and normal derivatives, point values of the 8, the linearised Riemann flux from its 16 stored values (18
+    operations per point), projection of 4 fluxes, viscous flux and lifting.
+    volume pass: corrected gradients and viscous flux for the modes of degree <= k - 1, interpolation of 3
+    fields, 6 products (9 operations per point), projection of 6 fields onto degree k - 1, modal derivatives with
+    the face terms, scaling in and out and mass shift.
+    The FP64 instructions that Nsight Compute counts (additions, products and multiply-adds of all threads,
+    16^3, per element) are 2700 + 1537 at k = 2, 5670 + 4373 at k = 3, 9777 + 9059 at k = 4.
     Returns (face FLOP per element, volume FLOP per element).
     """
-    n = k + 1
-    nb, nbm = n * (n + 1) * (n + 2) // 6, k * (k + 1) * (k + 2) // 6
-    n2 = n * (n + 1) // 2
-    ops = [pencil_ops(m, n) for m in range(n + 1)]
-    triangle = [sum(ops[1:m + 1]) + n * ops[m] for m in range(n + 1)]  # m (m + 1) / 2 coefficients <-> n^2 points
-    face = 3 * (14 * nb + 12 * triangle[n] + 22 * n * n + 24 * n2)
-    interp = sum(triangle[1:]) + n * n * ops[n]
-    project = n * n * ops[k] + n * sum(ops[1:k + 1]) + sum((g + 1) * ops[k - g] for g in range(k))
-    vol = 42 * nbm + 3 * interp + 9 * n ** 3 + 6 * project + 43 * nb
+    def nb_of(d):
+        return (d + 1) * (d + 2) * (d + 3) // 6
+
+    n, nb, nbm = k + 1, nb_of(k), nb_of(k - 1)
+    n2, n2m = n * (n + 1) // 2, n * k // 2
+
+    def triangle(ops, m):  # m (m + 1) / 2 coefficients <-> n^2 points
+        return sum(ops(q, n) for q in range(1, m + 1)) + n * ops(m, n)
+
+    tangential = sum((g + 1) * len(range(1, k - g + 1, 2)) for g in range(k + 1))  # coefficients of a 2D derivative
+    face = 3 * (8 * (3 * nb + n2m + 2) + 8 * triangle(interp_ops, n) + 18 * n * n + 4 * triangle(project_ops, n)
+                + 26 * n2 + 4 * tangential)
+    gradient = k + 2 + n2m + (k - 1) * k // 2 + 2 * nbm + sum((g + 1) * max(0, k - 2 - g) for g in range(k))
+    interp = sum(triangle(interp_ops, m) for m in range(1, n + 1)) + n * n * interp_ops(n, n)
+    project = sum(triangle(project_ops, m) for m in range(1, k + 1)) + n * n * project_ops(k, n)
+    vol = 9 * gradient + 9 * nbm + 3 * interp + 9 * n ** 3 + 6 * project + 4 * divergence_ops(k) + 11 * nb
     return 2.0 * face, 2.0 * vol
 
 
@@ -896,8 +922,8 @@ def run_ours(args):
         t = ms_k / cnt / 1e3
         if nm == "vol_tc32":
             # algorithmic bytes per element: the input and output coefficients, the linearisation
-            # velocity at the points, the face-slot contributions and liftings (FP32, read once)
-            b_el = 4.0 * (2 * 4 * nb + 3 * nq + 6 * 4 * n2 + 6 * 3 * n2)
+            # velocity at the points, the records of 3 faces (flux and jump; FP32, read once)
+            b_el = 4.0 * (2 * 4 * nb + 3 * nq + 3 * 7 * n2)
             ach = b_el * dg.ne / t / 1e9
             tflop = 2.0 * nq * nb * 9 * dg.ne / t / 1e12  # the two dense contractions' useful FLOP
             ent = {"bound": "hbm", "achieved": ach, "peak": hbm, "unit": "GB/s", "frac": ach / hbm,
