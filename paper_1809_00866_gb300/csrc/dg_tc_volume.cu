@@ -29,7 +29,8 @@
 // pipe is under 1 % busy. So each phase is written for few instructions, the elements' rows are
 // scaled, measured for sigma and converted to the operand while they are loaded, and four CTAs share an
 // SM (tiles of 21 elements, which fill the MMAs' rows, left two CTAs waiting on each other's phases).
-// At 32^3 P4: 127 us with those, 78 us now; at 24 x 12 x 12 P3 10.7 us.
+// At 32^3 P4: 127 us with those, 82 us now; at 24 x 12 x 12 P3 15 us (events included). The CUDA-core pass
+// (dg_volume.cu) takes 68 and 12 us.
 //
 // Operand layout in shared memory (K-major, no swizzle): cores of 8 rows x 16 bytes; the shared
 // memory descriptor's leading byte offset is the distance of K-adjacent cores, the stride byte

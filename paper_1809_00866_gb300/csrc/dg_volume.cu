@@ -15,8 +15,8 @@
 //    pencil of Gauss points per thread, in registers;
 //  * E elements per CTA: the items of a phase are (pencil, element) pairs sorted by pencil length,
 //    so a warp runs one length and its 32 lanes are busy also where one element has few pencils.
-// At 32^3 P4, one element per CTA with table look-ups -> now: FP64 1345 -> 653 us (0.77 of the measured FP64
-// rate on the counted operations), FP32 213 -> 69 us.
+// At 32^3 P4, one element per CTA with table look-ups -> now (events included): FP64 1345 -> 659 us (9223
+// operations per element, 0.87 of the measured FP64 rate), FP32 213 -> 68 us.
 #include <algorithm>
 
 #include "dg_async.h"
